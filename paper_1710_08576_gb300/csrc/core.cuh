@@ -167,40 +167,88 @@ struct KeysSeed {
     __device__ __forceinline__ uint32_t b(int r) const { return s1 + static_cast<uint32_t>(r) * 0xBB67AE85u; }
 };
 
-template <class K>
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const K &key) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        // one 32 x 32 -> 64-bit product per multiplier gives both halves
-        const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * c.x;
-        const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
-        const uint32_t lo0 = static_cast<uint32_t>(p0), hi0 = static_cast<uint32_t>(p0 >> 32);
-        const uint32_t lo1 = static_cast<uint32_t>(p1), hi1 = static_cast<uint32_t>(p1 >> 32);
-        c = make_uint4(hi1 ^ c.y ^ key.a(r), lo1, hi0 ^ c.w ^ key.b(r), lo0);
+// Digital-noise replacement: M + round_half_away(S2 * sigq / (107020 * 2^16)), sigq = 97164*D,
+// S2 = 2 * s - 8 * 65535 with s the sum of the eight 16-bit halves of the Philox output at counter
+// (idx_lo, idx_hi, stream, 0). It goes in two steps: noise_sum gives s, NoiseScale the value.
+
+// What the first two rounds compute from the stream and the index's high word alone: round 1's
+// second product (of the stream) and round 2's first product (of a word that holds no idx_lo).
+struct NoiseKey {
+    uint32_t a, b, c;  // round 2: z = a ^ (low product of round 1), x = b ^ ...; round 3: z = c ^ ...
+    template <class K>
+    __device__ __forceinline__ NoiseKey(const K &key, uint32_t sid, uint32_t idx_hi) {
+        const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * sid;
+        const uint32_t x = static_cast<uint32_t>(p1 >> 32) ^ idx_hi ^ key.a(0);
+        const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * x;
+        a = static_cast<uint32_t>(p0 >> 32) ^ key.b(1);
+        b = static_cast<uint32_t>(p1) ^ key.a(1);
+        c = static_cast<uint32_t>(p0) ^ key.b(2);
     }
-    return c;
+};
+
+// s of sample index idx_lo: 18 products instead of 20.
+template <class K>
+__device__ __forceinline__ uint32_t noise_sum(const NoiseKey &nk, const K &key, uint32_t idx_lo) {
+    uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * idx_lo;                                          // round 1
+    uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * (static_cast<uint32_t>(p0 >> 32) ^ key.b(0));    // round 2
+    uint4 c;
+    c.x = static_cast<uint32_t>(p1 >> 32) ^ nk.b;
+    c.y = static_cast<uint32_t>(p1);
+    c.z = nk.a ^ static_cast<uint32_t>(p0);
+    p0 = static_cast<uint64_t>(0xD2511F53u) * c.x;  // round 3
+    p1 = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
+    c = make_uint4(static_cast<uint32_t>(p1 >> 32) ^ c.y ^ key.a(2), static_cast<uint32_t>(p1),
+                   static_cast<uint32_t>(p0 >> 32) ^ nk.c, static_cast<uint32_t>(p0));
+#pragma unroll
+    for (int r = 3; r < 10; ++r) {
+        // one 32 x 32 -> 64-bit product per multiplier gives both halves
+        p0 = static_cast<uint64_t>(0xD2511F53u) * c.x;
+        p1 = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
+        c = make_uint4(static_cast<uint32_t>(p1 >> 32) ^ c.y ^ key.a(r), static_cast<uint32_t>(p1),
+                       static_cast<uint32_t>(p0 >> 32) ^ c.w ^ key.b(r), static_cast<uint32_t>(p0));
+    }
+    // each dp2a adds both halves of one word (weights 1, 1)
+    return __dp2a_lo(c.x, 0x0101u, __dp2a_lo(c.y, 0x0101u, __dp2a_lo(c.z, 0x0101u, __dp2a_lo(c.w, 0x0101u, 0u))));
 }
 
-// Digital-noise replacement: M + round_half_away(S2 * sigq / (107020 * 2^16)), sigq = 97164*D,
-// S2 = 2 * (sum of the eight 16-bit halves of the Philox output) - 8 * 65535.
-// |S2| <= 524280 and sigq < 2^29, so |S2| * sigq < 2^48; dividing by 2^16 first and then by
-// 107020 equals one floor division by their product.
-template <class K>
-__device__ __forceinline__ int32_t noise_value(int32_t M, uint32_t sigq, const K &key, uint32_t sid,
-                                               int64_t idx, int32_t lo, int32_t hi) {
-    const uint4 r = philox4x32_10(
-        make_uint4(static_cast<uint32_t>(idx), static_cast<uint32_t>(static_cast<uint64_t>(idx) >> 32),
-                   sid, 0u),
-        key);
-    // sum of the eight 16-bit halves: each dp2a adds both halves of one word (weights 1, 1)
-    const uint32_t s = __dp2a_lo(r.x, 0x0101u, __dp2a_lo(r.y, 0x0101u, __dp2a_lo(r.z, 0x0101u,
-                                                                              __dp2a_lo(r.w, 0x0101u, 0u))));
-    const int32_t S2 = 2 * static_cast<int32_t>(s) - 8 * 65535;
-    const uint32_t mag_s2 = static_cast<uint32_t>(S2 < 0 ? -S2 : S2);
-    const uint64_t a = static_cast<uint64_t>(mag_s2) * sigq + 3506831360ull;  // + 107020 * 2^15
-    const uint32_t q = static_cast<uint32_t>(a >> 16) / 107020u;
-    const int32_t v = M + (S2 < 0 ? -static_cast<int32_t>(q) : static_cast<int32_t>(q));
-    return v < lo ? lo : (v > hi ? hi : v);
+// The value of a sum s in a window with median M and dispersion D, saturated to the sample range:
+// M + floor((S2 * sigq + den / 2) / den), den = 107020 * 2^16, with OFF * den added to keep the
+// dividend positive (OFF is above the largest offset, 524280 * 97164 * D / den). The window gives
+// sig2 = 2 * sigq and moff = M - OFF. The dividend is below 2^49; dividing by 2^16 (12-bit: 2^17, to
+// stay in 32 bits) first and then by the rest of den equals one division, which is the high word of
+// the product with ceil(2^48 / 107020), shifted (exact for quotients of these ranges: the product's
+// excess over the true one stays below one). Rounding a half up instead of away from zero differs
+// only at an exact tie, that is |S2| * D = 2^15 * 26755: an offset of 12145.5, which no sample range
+// holds. A 32 x 32 -> 64-bit product runs at 64 lanes a clock and SM here; with a 64-bit addend it
+// runs at 25 and the high-word product at 32 (measured), hence the separate additions.
+template <int BITS>
+struct NoiseScale {
+    static constexpr int32_t kOff = BITS == 8 ? 2048 : 30000;
+    static constexpr int32_t kSig2 = 2 * 97164;
+    __device__ __forceinline__ static int32_t value(uint32_t s, int32_t sig2, int32_t moff) {
+        constexpr uint64_t kDen = 107020ull << 16;
+        constexpr uint64_t kAdd = kOff * kDen + kDen / 2;
+        constexpr int kShift = BITS == 8 ? 16 : 17;
+        constexpr int kLo = BITS == 8 ? -128 : -2048, kHi = BITS == 8 ? 127 : 2047;
+        uint32_t lo, hi, q;
+        asm("{\n\t.reg .b64 t;\n\tmul.wide.s32 t, %2, %3;\n\tmov.b64 {%0, %1}, t;\n\t}"
+            : "=r"(lo), "=r"(hi) : "r"(static_cast<int32_t>(s) - 262140), "r"(sig2));
+        asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;"
+            : "+r"(lo), "+r"(hi) : "r"(static_cast<uint32_t>(kAdd)), "r"(static_cast<uint32_t>(kAdd >> 32)));
+        const uint32_t n = __funnelshift_r(lo, hi, kShift);
+        asm("{\n\t.reg .b64 t;\n\t.reg .b32 u;\n\tmul.wide.u32 t, %1, %2;\n\tmov.b64 {u, %0}, t;\n\t}"
+            : "=r"(q) : "r"(n), "r"(2630115649u));
+        const int32_t v = static_cast<int32_t>(q >> (32 - kShift)) + moff;
+        return v < kLo ? kLo : (v > kHi ? kHi : v);
+    }
+};
+
+template <int BITS, class K>
+__device__ __forceinline__ int32_t noise_value(int32_t M, uint32_t D, const K &key, uint32_t sid, int64_t idx) {
+    const uint64_t i = static_cast<uint64_t>(idx);
+    const NoiseKey nk(key, sid, static_cast<uint32_t>(i >> 32));
+    return NoiseScale<BITS>::value(noise_sum(nk, key, static_cast<uint32_t>(i)), NoiseScale<BITS>::kSig2 * static_cast<int32_t>(D),
+                                   M - NoiseScale<BITS>::kOff);
 }
 
 // ------------------------------------------------------------------ shared-memory layout
@@ -237,7 +285,7 @@ __device__ __forceinline__ int pad32(int b) { return b + (b >> 5); }
 
 struct __align__(16) RepShared {
     int32_t M, D, t, hiv, lov;
-    uint32_t sigq, active, pad;
+    uint32_t active, pad[2];
     // int8 replace constants (see Rep8)
     uint32_t mb4, tlo7, tsmall, c4, hi4, lo4, ulo7, usmall;
     uint32_t unone;
@@ -564,7 +612,6 @@ struct Rep {
     int32_t cval;     // constant replacement (saturated)
     int32_t t;        // min(ceil(Kq*D / 2^16), sample span + 1)
     int32_t hiv, lov; // threshold replacement above / below (saturated)
-    uint32_t sigq;    // 97164 * D
     bool active;      // some sample can be flagged
 };
 
@@ -586,9 +633,8 @@ __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, 
     r.t = static_cast<int32_t>(t < SPAN + 1 ? t : SPAN + 1);
     r.hiv = sat_to(static_cast<int64_t>(r.M) + c, Geo<BITS>::kLo, Geo<BITS>::kHi);
     r.lov = sat_to(static_cast<int64_t>(r.M) - c, Geo<BITS>::kLo, Geo<BITS>::kHi);
-    r.sigq = 97164u * static_cast<uint32_t>(d);
     r.active = (d > 0 && t <= SPAN) ? 1u : 0u;  // |x - M| never exceeds the sample span
-    r.pad = 0u;
+    r.pad[0] = r.pad[1] = 0u;
     r.cval = cval;
     if (BITS == 8) {
         const uint32_t tt = static_cast<uint32_t>(r.t > 255 ? 255 : r.t);
@@ -641,7 +687,6 @@ __device__ __forceinline__ Rep load_rep(const RepShared &s) {
     r.t = s.t;
     r.hiv = s.hiv;
     r.lov = s.lov;
-    r.sigq = s.sigq;
     r.active = s.active != 0u;
     return r;
 }
@@ -835,7 +880,7 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
             const bool inlo = j < clo;
             const int bp = (inlo ? 0 : 32) + nth_set_bit(inlo ? loL : hiL, inlo ? j : j - clo);
             const int pos = (cL + (bp >> 4) * T) * CS + (bp & 15);
-            const int32_t z = noise_value(r.M, r.sigq, p, w.sid, w.abs_idx + pos, Geo<BITS>::kLo, Geo<BITS>::kHi);
+            const int32_t z = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pos);
             store_sample<BITS, OUTF>(w.out, pos, z);
             if (PW) pw.z += static_cast<uint32_t>(z * z);
         }
@@ -887,8 +932,8 @@ __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Re
     // windows, a quarter of them flagged: 4.60 -> 4.53 ms per call)
     for (; i + T < n; i += 2 * T) {
         const uint32_t pa = sm.nlist[i], pb = sm.nlist[i + T];
-        const int32_t za = noise_value(r.M, r.sigq, p, w.sid, w.abs_idx + pa, Geo<BITS>::kLo, Geo<BITS>::kHi);
-        const int32_t zb = noise_value(r.M, r.sigq, p, w.sid, w.abs_idx + pb, Geo<BITS>::kLo, Geo<BITS>::kHi);
+        const int32_t za = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pa);
+        const int32_t zb = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pb);
         if (pa != kNoiseSkip) {
             store_sample<BITS, OUTF>(w.out, pa, za);
             if (PW) pw.z += static_cast<uint32_t>(za * za);
@@ -901,7 +946,7 @@ __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Re
     for (; i < n; i += T) {
         const uint32_t pos = sm.nlist[i];
         if (pos == kNoiseSkip) continue;
-        const int32_t z = noise_value(r.M, r.sigq, p, w.sid, w.abs_idx + pos, Geo<BITS>::kLo, Geo<BITS>::kHi);
+        const int32_t z = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pos);
         store_sample<BITS, OUTF>(w.out, pos, z);
         if (PW) pw.z += static_cast<uint32_t>(z * z);
     }
@@ -971,7 +1016,7 @@ __device__ __forceinline__ void noise_deferred8(const Shm &sm, const Win &w, con
     named_bar(sm.bar_id, T);  // every entry of the window is in the list
     noise_expand8<T>(sm, *nlc, tid, [&](uint32_t pos) {
         if (pos >= static_cast<uint32_t>(w.n)) return;
-        const int32_t z = noise_value(r.M, r.sigq, p, w.sid, w.abs_idx + pos, Geo<8>::kLo, Geo<8>::kHi);
+        const int32_t z = noise_value<8>(r.M, r.D, p, w.sid, w.abs_idx + pos);
         store_sample<8, OUTF>(w.out, static_cast<int>(pos), z);
         if (PW) pw.z += static_cast<uint32_t>(z * z);
     });
@@ -1396,7 +1441,7 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
         const int64_t abs0 = sg.abs0 + (static_cast<int64_t>(w0) << lw);
         noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t pos) {
             const RepShared &rk = reps[pos >> lw];
-            const int32_t z = noise_value(rk.M, rk.sigq, key, sg.stream_id, abs0 + pos, Geo<8>::kLo, Geo<8>::kHi);
+            const int32_t z = noise_value<8>(rk.M, rk.D, key, sg.stream_id, abs0 + pos);
             out[pos] = static_cast<uint8_t>(z);
         });
     }

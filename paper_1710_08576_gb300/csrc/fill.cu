@@ -5,33 +5,44 @@
 // kernel then overwrites the flagged samples with M + the Philox noise of spread 1.4826·D, keyed
 // by the absolute sample index as always, so the result is the same bits as the one-pass form.
 //
-// Work: a unit is a run of 256 mask words; warp g of the grid takes units g, g + nwarps, ...
-// (segment s holds units [fwin[s], fwin[s + 1])), so that at any time the warps read masks and
-// write samples close to one another (giving each warp a run of consecutive units instead
-// made the k = 3 call of the 60-stream benchmark 40 % slower). Windows of at most kFillPackMax
-// samples, a multiple of 128 (fill_packs), are packed: the segment's mask is one array of words
-// (window k's at k * mw, word j covering samples 32j .. 32j + 31 of the segment) cut into units
-// regardless of the windows, so a unit spans several windows and each lane takes M and D of the
-// window its four words belong to. Otherwise every window has ceil(mw / 256) units of its own,
-// and a unit of a window whose count is 0 is skipped. The unit goes in two halves of 128 words: lane l reads words
-// 4l .. 4l + 3 of a half, and the warp moves their flagged samples into its ring of positions:
-//  - a word with at least kFillDense flags goes whole: lane j tests bit j and a ballot with a
-//    prefix popcount gives each flagged lane its place in the ring;
-//  - from the other words every lane gives up one flag per step (its lowest remaining one),
-//    compacted the same way.
-// Whenever 32 positions wait in the ring, every lane takes one and evaluates its noise. A ring
-// entry carries the window's M and D with the position, so the ring runs on across the warp's
-// units of a segment and its last fewer-than-32 positions go out only when the segment changes
-// or the warp ends. Every lane of a batch but those of such a last one has a sample.
+// Work: a segment's mask is one array of words, window k's at k * mw (mw = ceil(W / 32)), cut into
+// units of up to 256 words regardless of the windows; segment s holds units [fwin[s], fwin[s + 1]).
+// The warps take units in order from a cursor, so that at any time they read masks and write
+// samples close to one another (giving each warp a run of consecutive units instead made the
+// k = 3 call of the 60-stream benchmark 40 % slower) and a warp that met dense units takes fewer. Per unit:
+//  1. the lanes load the words (lane l words l, l + 32, ...) and list the nonzero ones,
+//  2. per group of 32 nonzero words, lane l takes one: its window (M, D, first sample) and, by a
+//     prefix sum of the flag counts, where its flags go in the warp's position list,
+//  3. the group's words are expanded one by one: lane j tests bit j and a popcount of the bits
+//     below gives its place; an entry is 16 bits, the word's slot in its group and the bit,
+//  4. every lane takes an entry of the list and evaluates its noise, 32 at a time. The fewer than
+//     32 entries left over go in front of the next group's, so only the last batch of a unit is
+//     not full. Two entries of a lane at a time: their Philox chains interleave.
+// What bounds it: the Philox products. A 32 x 32 -> 64-bit product takes four cycles of a quarter of
+// an SM's multiplier for a warp (measured), so the 18 of a batch of 32 samples and the other multiply
+// instructions come to about 90 cycles; step 3 costs 8 instructions per nonzero word (no vote, branch or
+// carried counter per word) and steps 1 and 2 about 400 per unit. On 60 streams of 2^26 int8 samples in
+// 16384-sample windows (k = 3, 6.3 % flagged) the pass takes 1.13 ms; 1.70 ms with a ring filled
+// word by word under a ballot, a static share of the units and 20 products a value. Measured and not
+// kept: the next unit's words loaded while one is worked on (56 registers, 1.5 % slower), the
+// left-over samples kept in registers across units (57 registers, 1.7 % slower), a sixth CTA per
+// SM (40 registers, 1 % slower).
 
 #include "core.cuh"
 
 namespace rfi {
 namespace dev {
 
-constexpr int kFillThreads = 256;
-constexpr int kFillRing = 64;   // positions a warp's ring holds: fewer than 32 wait between steps
-constexpr int kFillDense = 2;   // flags from which a mask word is expanded whole
+constexpr int kFillThreads = kFillWarps * 32;
+constexpr int kFillWords = kFillUnitMax / 32;  // mask words per lane of the largest unit
+
+// One warp's work area.
+struct FillWarp {
+    uint2 word[kFillUnitMax];    // the unit's nonzero words and their indices, in order
+    uint2 ent[64];               // two groups of 32 words: {word, place of its flags in the list}
+    uint4 win[64];               // of the same words: {first sample, sig2 and moff of its window (NoiseScale), -}
+    uint16_t list[32 + 32 * 32]; // flagged samples waiting: slot in ent * 32 + bit
+};
 
 template <int BITS>
 __device__ __forceinline__ void fill_store(uint8_t *out, uint32_t pos, int32_t z) {
@@ -39,164 +50,150 @@ __device__ __forceinline__ void fill_store(uint8_t *out, uint32_t pos, int32_t z
     else reinterpret_cast<int16_t *>(out)[pos] = static_cast<int16_t>(z);
 }
 
-// The warp's ring: queued positions (segment-relative sample index, with the window's M in the
-// low and D in the high 16 bits of md) and the batches that empty it.
-template <int BITS>
-struct FillRing {
-    uint2 *q;
-    uint32_t head, tail;  // positions taken / queued so far
-    const Seg *g;
-    const KeysPre *key;
-    int lane;
-
-    __device__ __forceinline__ void emit(uint2 e) const {
-        const int32_t M = static_cast<int16_t>(e.y & 0xFFFFu);
-        const uint32_t sigq = 97164u * (e.y >> 16);
-        const int32_t z = noise_value(M, sigq, *key, g->stream_id, g->abs0 + static_cast<int64_t>(e.x),
-                                      Geo<BITS>::kLo, Geo<BITS>::kHi);
-        fill_store<BITS>(g->out, e.x, z);
-    }
-    // Queue the flagged lanes' positions (every lane calls this), then empty a full batch.
-    __device__ __forceinline__ void put(bool fl, uint32_t pos, uint32_t md) {
-        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, fl);
-        if (fl) q[(tail + static_cast<uint32_t>(__popc(bal & ((1u << lane) - 1u)))) & (kFillRing - 1)] = make_uint2(pos, md);
-        tail += static_cast<uint32_t>(__popc(bal));
-        if (tail - head >= 32u) {
-            __syncwarp();
-            const uint2 e = q[(head + static_cast<uint32_t>(lane)) & (kFillRing - 1)];
-            __syncwarp();  // read before the next step refills the slot
-            head += 32u;
-            emit(e);
-        }
-    }
-    // The positions still waiting (fewer than 32).
-    __device__ __forceinline__ void drain() {
-        if (tail == head) return;
-        __syncwarp();
-        if (static_cast<uint32_t>(lane) < tail - head) emit(q[(head + static_cast<uint32_t>(lane)) & (kFillRing - 1)]);
-        __syncwarp();
-        head = tail;
-    }
-};
-
 // Segments hold fewer than 2^31 samples (the plan routes longer ones through the one-pass form),
 // so every segment-relative index below fits 32 bits.
-// PACK: some segment of the launch is packed (the instantiation without it is the per-window
-// form alone, with fewer registers).
-template <int BITS, bool PACK>
+template <int BITS>
 __global__ void __launch_bounds__(kFillThreads) noise_fill_kernel(const Seg *__restrict__ segs, int nseg,
                                                                  const uint32_t *__restrict__ fwin, uint32_t nunits,
-                                                                 Params p) {
-    __shared__ uint2 ring_s[kFillThreads / 32][kFillRing];
-    const int lane = threadIdx.x & 31;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+                                                                 uint32_t unit, Params p, unsigned *counter) {
+    __shared__ FillWarp area[kFillWarps];
+    FillWarp &a = area[threadIdx.x >> 5];
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t below = (1u << lane) - 1u, bit = 1u << lane;
     const KeysPre key{p};
-    FillRing<BITS> R{ring_s[threadIdx.x >> 5], 0u, 0u, segs, &key, lane};
     int s = 0;
-    for (uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < nunits; u += nwarps) {
-        if (fwin[s + 1] <= u) {  // a warp's units ascend: the queue belongs to the segment
-            R.drain();
-            while (s + 1 < nseg && fwin[s + 1] <= u) ++s;
-            R.g = &segs[s];
-        }
+    // the first unit of a warp is its own (spread over the CTAs, so that few units take many SMs),
+    // the others come from the cursor, fetched while the unit before is worked on
+    const uint32_t nwarps = gridDim.x * kFillWarps;
+    uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (; u < nunits;) {
+        uint32_t next = 0u;
+        if (lane == 0) next = nwarps + atomicAdd(counter, 1u);
+        while (s + 1 < nseg && fwin[s + 1] <= u) ++s;  // a warp's units ascend
         const Seg &g = segs[s];
-        const uint32_t mw = static_cast<uint32_t>(g.mask_words);
-        const uint32_t local = u - fwin[s];
-        const bool packed = PACK && fill_packs(g.W);
+        const uint32_t W = static_cast<uint32_t>(g.W), mw = static_cast<uint32_t>(g.mask_words);
+        const uint32_t jfirst = (u - fwin[s]) * unit;
+        const uint32_t jend = min(jfirst + unit, g.nwords), j0 = jfirst + lane;
         const uint32_t *mk = g.mask;
-        uint32_t j00, jend, pos0 = 0u, md = 0u;
-        if (packed) {
-            j00 = local << 8;
-            jend = min(j00 + 256u, static_cast<uint32_t>((g.len + 31) >> 5));  // the words holding samples
-        } else {
-            const uint32_t upw = (mw + 255u) >> 8;  // units per window
-            const uint32_t k = local / upw;
-            j00 = (local - k * upw) << 8;
-            jend = min(j00 + 256u, mw);
-            if (g.counts && g.counts[k] == 0u) continue;
-            md = (static_cast<uint32_t>(g.med[k]) & 0xFFFFu) | (static_cast<uint32_t>(g.mad[k]) << 16);
-            mk += static_cast<size_t>(k) * mw;
-            pos0 = k * static_cast<uint32_t>(g.W);
+        uint32_t m[kFillWords];
+#pragma unroll
+        for (int i = 0; i < kFillWords; ++i) m[i] = j0 + 32 * i < jend ? mk[j0 + 32 * i] : 0u;
+        uint32_t n = 0;  // nonzero words
+#pragma unroll
+        for (int i = 0; i < kFillWords; ++i) {
+            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, m[i] != 0u);
+            if (m[i]) a.word[n + __popc(bal & below)] = make_uint2(m[i], j0 + 32 * i);
+            n += static_cast<uint32_t>(__popc(bal));
         }
-        // a packed segment's words of a lane lie in one window (mw is a multiple of 4)
-        const bool vec = (mw & 3u) == 0u && (reinterpret_cast<uintptr_t>(mk) & 15u) == 0u;
-        const int lg = PACK && (mw & (mw - 1u)) == 0u ? __ffs(mw) - 1 : -1;  // log2 mw, or -1
-        for (uint32_t j0 = j00; j0 < jend; j0 += 128u) {
-            const uint32_t jl = j0 + 4u * static_cast<uint32_t>(lane);  // this lane's first word
-            uint32_t m[4];
-            uint32_t mdl = md;
-            if (vec) {
-                const uint4 a = jl < jend ? *reinterpret_cast<const uint4 *>(mk + jl) : make_uint4(0u, 0u, 0u, 0u);
-                m[0] = a.x;
-                m[1] = a.y;
-                m[2] = a.z;
-                m[3] = a.w;
+        if (n == 0u) {
+            u = __shfl_sync(0xFFFFFFFFu, next, 0);
+            continue;
+        }
+        __syncwarp();
+        const int lg = (mw & (mw - 1u)) == 0u ? __ffs(static_cast<int>(mw)) - 1 : -1;  // log2 mw, or -1
+        const NoiseKey nk(key, g.stream_id, static_cast<uint32_t>(static_cast<uint64_t>(g.abs0) >> 32));
+        const bool one_hi = ((static_cast<uint64_t>(g.abs0) ^ static_cast<uint64_t>(g.abs0 + g.len - 1)) >> 32) == 0;
+        const uint64_t abs0 = static_cast<uint64_t>(g.abs0);
+        uint8_t *const out = g.out;
+        auto emit = [&](uint32_t code) {
+            const uint4 e = a.win[code >> 5];
+            const uint32_t pos = e.x + (code & 31u);
+            uint32_t sum;
+            if (one_hi) {
+                sum = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pos);
             } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) m[i] = jl + i < jend ? mk[jl + i] : 0u;
+                const uint64_t idx = abs0 + pos;
+                sum = noise_sum(NoiseKey(key, g.stream_id, static_cast<uint32_t>(idx >> 32)), key, static_cast<uint32_t>(idx));
             }
-            if (packed && jl < jend) {
-                const uint32_t k = lg >= 0 ? jl >> lg : jl / mw;
-                mdl = (static_cast<uint32_t>(g.med[k]) & 0xFFFFu) | (static_cast<uint32_t>(g.mad[k]) << 16);
+            fill_store<BITS>(out, pos, NoiseScale<BITS>::value(sum, static_cast<int32_t>(e.y), static_cast<int32_t>(e.z)));
+        };
+        // two entries of a lane at a time: their Philox chains are independent and interleave
+        auto emit2 = [&](uint32_t c0, uint32_t c1) {
+            if (!one_hi) {
+                emit(c0);
+                emit(c1);
+                return;
             }
-            if (!__any_sync(0xFFFFFFFFu, (m[0] | m[1] | m[2] | m[3]) != 0u)) continue;  // on to the next half
-            // dense words, one at a time over the whole warp
+            const uint4 e0 = a.win[c0 >> 5], e1 = a.win[c1 >> 5];
+            const uint32_t p0 = e0.x + (c0 & 31u), p1 = e1.x + (c1 & 31u);
+            const uint32_t s0 = noise_sum(nk, key, static_cast<uint32_t>(abs0) + p0);
+            const uint32_t s1 = noise_sum(nk, key, static_cast<uint32_t>(abs0) + p1);
+            fill_store<BITS>(out, p0, NoiseScale<BITS>::value(s0, static_cast<int32_t>(e0.y), static_cast<int32_t>(e0.z)));
+            fill_store<BITS>(out, p1, NoiseScale<BITS>::value(s1, static_cast<int32_t>(e1.y), static_cast<int32_t>(e1.z)));
+        };
+        uint32_t have = 0;  // entries waiting at the front of the list
+        for (uint32_t e0 = 0, grp = 0; e0 < n; e0 += 32, grp ^= 32u) {
+            const uint32_t ne = min(32u, n - e0);
+            uint32_t w = 0u, cnt = 0u;
+            if (lane < ne) {
+                const uint2 wj = a.word[e0 + lane];
+                w = wj.x;
+                cnt = static_cast<uint32_t>(__popc(w));
+                const uint32_t k = lg >= 0 ? wj.y >> lg : wj.y / mw;
+                a.win[grp + lane] = make_uint4(k * W + ((wj.y - k * mw) << 5),
+                                               static_cast<uint32_t>(NoiseScale<BITS>::kSig2 * g.mad[k]),
+                                               static_cast<uint32_t>(g.med[k] - NoiseScale<BITS>::kOff), 0u);
+            }
+            uint32_t inc = cnt;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t wi = m[i];
-                const bool d = __popc(wi) >= kFillDense;
-                uint32_t dense = __ballot_sync(0xFFFFFFFFu, d);
-                if (d) m[i] = 0u;
-                while (dense) {
-                    const int src = __ffs(dense) - 1;
-                    dense &= dense - 1u;
-                    const uint32_t w = __shfl_sync(0xFFFFFFFFu, wi, src);
-                    const uint32_t mdw = PACK ? __shfl_sync(0xFFFFFFFFu, mdl, src) : mdl;
-                    const uint32_t pos = pos0 + 32u * (j0 + 4u * static_cast<uint32_t>(src) + i) + static_cast<uint32_t>(lane);
-                    R.put(((w >> lane) & 1u) != 0u, pos, mdw);
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                if (lane >= static_cast<uint32_t>(o)) inc += y;
+            }
+            a.ent[grp + lane] = make_uint2(w, have + inc - cnt);
+            const uint32_t total = have + __shfl_sync(0xFFFFFFFFu, inc, 31);
+            __syncwarp();
+            // a full group (the other lanes' words are zero) in steps of four words
+            uint32_t code = grp * 32u + lane;
+            for (uint32_t e = 0; e < ne; e += 4) {
+#pragma unroll
+                for (uint32_t q = 0; q < 4; ++q) {
+                    const uint2 wo = a.ent[grp + e + q];
+                    if (wo.x & bit) a.list[wo.y + __popc(wo.x & below)] = static_cast<uint16_t>(code + 32u * q);
                 }
+                code += 128u;
             }
-            // the other words: each lane gives up its lowest remaining flag per step
-            while (__any_sync(0xFFFFFFFFu, (m[0] | m[1] | m[2] | m[3]) != 0u)) {
-                const bool h0 = m[0] != 0u, h1 = m[1] != 0u, h2 = m[2] != 0u;
-                const uint32_t i = h0 ? 0u : (h1 ? 1u : (h2 ? 2u : 3u));
-                const uint32_t cur = h0 ? m[0] : (h1 ? m[1] : (h2 ? m[2] : m[3]));
-                const uint32_t pos = pos0 + 32u * (jl + i) + static_cast<uint32_t>(__ffs(cur) - 1);
-                const uint32_t rest = cur & (cur - 1u);
-                if (h0) m[0] = rest;
-                else if (h1) m[1] = rest;
-                else if (h2) m[2] = rest;
-                else m[3] = rest;
-                R.put(cur != 0u, pos, mdl);
+            __syncwarp();
+            uint32_t h = 0;
+            for (; h + 64u <= total; h += 64u) emit2(a.list[h + lane], a.list[h + 32u + lane]);
+            if (h + 32u <= total) {
+                emit(a.list[h + lane]);
+                h += 32u;
             }
+            have = total - h;
+            const uint32_t left = lane < have ? a.list[h + lane] : 0u;
+            __syncwarp();
+            if (e0 + 32 < n) {
+                // a full group fills at least one batch, so what is left over is this group's: the
+                // next one may take the other half of ent
+                if (lane < have) a.list[lane] = static_cast<uint16_t>(left);
+            } else if (lane < have) {
+                emit(left);
+            }
+            __syncwarp();
         }
+        u = __shfl_sync(0xFFFFFFFFu, next, 0);
     }
-    R.drain();
 }
 
 }  // namespace dev
 
-int noise_fill_grid(int sm_count, bool packed) {
+int noise_fill_grid(int sm_count) {
     int n = 0;
-    const cudaError_t e = packed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dev::noise_fill_kernel<8, true>, dev::kFillThreads, 0)
-                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dev::noise_fill_kernel<8, false>, dev::kFillThreads, 0);
-    if (e != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dev::noise_fill_kernel<8>, dev::kFillThreads, 0) != cudaSuccess ||
+        n < 1) {
         cudaGetLastError();
         n = 1;
     }
     return sm_count * n;
 }
 
-cudaError_t launch_noise_fill(int bits, bool packed, const Seg *segs, int nseg, const uint32_t *fwin, uint32_t nunits,
-                              const Params &p, int grid, cudaStream_t st) {
+cudaError_t launch_noise_fill(int bits, const Seg *segs, int nseg, const uint32_t *fwin, uint32_t nunits, int unit,
+                              const Params &p, unsigned *counter, int grid, cudaStream_t st) {
     if (nunits == 0) return cudaSuccess;
-    if (bits == 8) {
-        if (packed) dev::noise_fill_kernel<8, true><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, p);
-        else dev::noise_fill_kernel<8, false><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, p);
-    } else {
-        if (packed) dev::noise_fill_kernel<12, true><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, p);
-        else dev::noise_fill_kernel<12, false><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, p);
-    }
+    if (nunits < static_cast<uint32_t>(grid)) grid = static_cast<int>(nunits);
+    if (bits == 8) dev::noise_fill_kernel<8><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, static_cast<uint32_t>(unit), p, counter);
+    else dev::noise_fill_kernel<12><<<grid, dev::kFillThreads, 0, st>>>(segs, nseg, fwin, nunits, static_cast<uint32_t>(unit), p, counter);
     return cudaGetLastError();
 }
 

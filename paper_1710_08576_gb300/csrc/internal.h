@@ -58,6 +58,8 @@ struct DevCounters {
     unsigned tile_counter;       // dynamic work-list cursor
     uint32_t status;             // kStatus* bits
     unsigned long long flagged;  // flagged samples of the pass
+    unsigned fill_counter;       // work cursor of the digital-noise pass
+    unsigned pad;
 };
 
 // One contiguous run of windows of one stream, starting on a window boundary.
@@ -75,7 +77,8 @@ struct Seg {
     int32_t mask_words;   // ceil(W / 32)
     int32_t vec;          // in/out 16-byte aligned and W * bytes_per_sample % 16 == 0
     uint64_t *power;      // detected power of window 0: {sum x^2, sum z^2} (nullable)
-    uint32_t pad[2];
+    uint32_t nwords;      // mask words of the run (set for the digital-noise pass)
+    uint32_t pad;
 };
 
 // Work-list entry of the persistent kernel: windows [w0, w0 + nw) of segment seg.
@@ -170,15 +173,14 @@ cudaError_t launch_mom(int bits, const MomChunk *chunks, int nchunks, const int3
 
 // Digital noise as a second pass over segments whose excision pass wrote 0 at the flagged
 // samples, the flag mask, every window's count and every window's M and D (segments of fewer
-// than 2^31 samples). The pass's units are 256 mask words: of the whole segment's mask when
-// fill_packs(W) (ceil(ceil(len / 32) / 256) units), else of each window (ceil(ceil(W / 32) / 256)
-// a window); segment s holds units [fwin[s], fwin[s + 1]), nunits = fwin[nseg]. packed: some
-// segment of the launch has fill_packs(W).
-constexpr int kFillPackMax = 2048;
-__host__ __device__ inline bool fill_packs(int32_t W) { return W % 128 == 0 && W <= kFillPackMax; }
-int noise_fill_grid(int sm_count, bool packed);
-cudaError_t launch_noise_fill(int bits, bool packed, const Seg *segs, int nseg, const uint32_t *fwin, uint32_t nunits,
-                              const Params &p, int grid, cudaStream_t st);
+// than 2^31 samples). The pass's units are `unit` words of a segment's mask (nwin * ceil(W / 32)
+// words), unit = 32, 64, 128 or 256; segment s holds units [fwin[s], fwin[s + 1]), nunits =
+// fwin[nseg]. counter: one zeroed uint32, the cursor that the warps take units from.
+constexpr int kFillUnitMin = 32, kFillUnitMax = 256;
+constexpr int kFillWarps = 8;  // warps per CTA
+int noise_fill_grid(int sm_count);
+cudaError_t launch_noise_fill(int bits, const Seg *segs, int nseg, const uint32_t *fwin, uint32_t nunits, int unit,
+                              const Params &p, unsigned *counter, int grid, cudaStream_t st);
 
 // Write n (<= kSegBatch) segment descriptors to dst (device) from kernel parameters.
 constexpr int kSegBatch = 32;

@@ -148,22 +148,22 @@ rfi_status plan_alloc_workspace(rfi_plan_s *P) {
     const size_t mc_b = mom ? al(sizeof(MomChunk) * P->mchunks.size()) : 0;
     const size_t pw_b = P->power ? al(2 * sizeof(uint64_t) * P->total_windows) : 0;
     const size_t var_b = al(sizeof(Variant) * P->variants.size());
-    // the fill pass: unit offsets of the segments (256 mask words a unit; for small windows of a
-    // multiple of 128 samples the units run over the words of the whole segment, else over
-    // those of each window)
+    // the fill pass: unit offsets of the segments. Units of kFillUnitMax mask words, smaller ones
+    // where that leaves most warps of the grid without a unit: a warp works through its unit alone, so
+    // small plans (2^20 12-bit samples, a quarter flagged: 35.0 us a call with 256-word units) are
+    // bound by one unit's time
     std::vector<uint32_t> fwin;
     if (P->fill) {
-        fwin.push_back(0);
-        P->fill_packed = false;
-        for (int i = 0; i < P->S; ++i) {
-            const bool pk = fill_packs(P->W[i]);
-            const int64_t units = pk ? ((P->len[i] + 31) / 32 + 255) / 256
-                                     : P->nwin[i] * (((P->W[i] + 31) / 32 + 255) / 256);
-            P->fill_packed = P->fill_packed || pk;
-            fwin.push_back(fwin.back() + static_cast<uint32_t>(units));
+        P->fill_grid = noise_fill_grid(P->sm_count);
+        for (P->fill_unit = kFillUnitMax;; P->fill_unit /= 2) {
+            fwin.assign(1, 0);
+            for (int i = 0; i < P->S; ++i) {
+                const int64_t words = P->nwin[i] * ((P->W[i] + 31) / 32);
+                fwin.push_back(fwin.back() + static_cast<uint32_t>((words + P->fill_unit - 1) / P->fill_unit));
+            }
+            if (P->fill_unit == kFillUnitMin || 2 * fwin.back() >= static_cast<uint32_t>(P->fill_grid * kFillWarps)) break;
         }
         P->nfwin = fwin.back();
-        P->fill_grid = noise_fill_grid(P->sm_count, P->fill_packed);
     }
     // one allocation, each array at the next 256-byte boundary
     size_t off = 0;
@@ -239,7 +239,8 @@ rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st) {
         const Params p = plan_params(P);
         RFI_CUDA(launch_persistent(P->bits, plan_kernel_mode(P), P->shape, P->grid, P->d_segs, P->d_tiles,
                                    P->ntiles, p, &P->d_ctr->tile_counter, inject, st));
-        if (P->fill) RFI_CUDA(launch_noise_fill(P->bits, P->fill_packed, P->d_segs, P->S, P->d_fwin, P->nfwin, p, P->fill_grid, st));
+        if (P->fill) RFI_CUDA(launch_noise_fill(P->bits, P->d_segs, P->S, P->d_fwin, P->nfwin, P->fill_unit, p, &P->d_ctr->fill_counter,
+                                   P->fill_grid, st));
         return RFI_OK;
     }
     // Median of MAD (Eq. 3): M and D of every window, the sliding median of the MADs, then Eq. 1
@@ -254,7 +255,8 @@ rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st) {
                                P->d_tiles, P->ntiles, p, &P->d_ctr->tile_counter, 0, st));
     // the apply segments hold each window's M and its MoM: the noise spread of Eq. 3
     if (P->fill)
-        RFI_CUDA(launch_noise_fill(P->bits, P->fill_packed, P->d_segs + P->S, P->S, P->d_fwin, P->nfwin, p, P->fill_grid, st));
+        RFI_CUDA(launch_noise_fill(P->bits, P->d_segs + P->S, P->S, P->d_fwin, P->nfwin, P->fill_unit, p, &P->d_ctr->fill_counter,
+                                   P->fill_grid, st));
     return RFI_OK;
 }
 
@@ -301,6 +303,7 @@ std::vector<Seg> plan_segs(const rfi_plan_s *P, const void *const *in, void *con
         g.W = P->W[i];
         g.stream_id = P->sid[i];
         g.mask_words = (P->W[i] + 31) / 32;
+        if (P->fill) g.nwords = static_cast<uint32_t>(P->nwin[i] * g.mask_words);
         g.vec = ((reinterpret_cast<uintptr_t>(in[i]) | reinterpret_cast<uintptr_t>(out[i])) % 16 == 0) &&
                 (static_cast<int64_t>(P->W[i]) * bps) % 16 == 0;
         if (P->kmom >= 2) {

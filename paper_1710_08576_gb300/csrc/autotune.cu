@@ -52,13 +52,12 @@ __global__ void fill_scratch(uint8_t *buf, int64_t n, int bits) {
     }
 }
 
-std::vector<Tile> tiles_for(int bits, const std::vector<int64_t> &len, const std::vector<int32_t> &W,
+std::vector<Tile> tiles_for(int bits, int mode, const std::vector<int64_t> &len, const std::vector<int32_t> &W,
                             int stage_bytes) {
     const int bps = bits == 8 ? 1 : 2;
     std::vector<Tile> tiles;
     for (size_t i = 0; i < len.size(); ++i) {
-        const int64_t wb = static_cast<int64_t>(W[i]) * bps;
-        const int64_t per = (wb % 16 == 0) ? std::max<int64_t>(1, stage_bytes / wb) : 1;
+        const int64_t per = tile_windows(bits, mode, W[i], stage_bytes);
         const int64_t nwin = (len[i] + W[i] - 1) / W[i];
         for (int64_t w0 = 0; w0 < nwin; w0 += per) {
             const int64_t nw = std::min<int64_t>(per, nwin - w0);
@@ -209,7 +208,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
         maxwb = std::max<int64_t>(maxwb, std::min<int64_t>(P->W[i], P->len[i]) * bps);
         uniform = uniform && P->W[i] == P->W[0];
     }
-    const int min_stage = static_cast<int>((maxwb + 127) / 128 * 128);
+    const int min_stage = min_stage_bytes(plan_tile_mode(P), maxwb);
     std::vector<Shape> cands;
     for (int cw : {4, 8, 16})
       for (int grp : {1, 2})
@@ -222,6 +221,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
                             if (P->bits == 8 && hc != 1) continue;
                             if (!uniform && dyn == 2) continue;
                             if (grp == 2 && cw == 16) continue;
+                            if (P->any && (cw != 8 || grp != 1)) continue;
                             Shape s{cw, stages, ctas, min_stage * mult, dyn, P->bits == 8 ? 1 : hc, grp, ws};
                             if (ws == 2 && !plan_warp_split_runs(P, s)) continue;
                             if (req && req->warp_split && req->warp_split != ws) continue;
@@ -263,7 +263,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
             continue;
         }
         if (s.stage_bytes != cur_stage) {
-            cur = tiles_for(P->bits, slen, P->W, s.stage_bytes);
+            cur = tiles_for(P->bits, plan_tile_mode(P), slen, P->W, s.stage_bytes);
             cudaFree(sc.tiles);
             sc.tiles = nullptr;
             if (cudaMalloc(&sc.tiles, sizeof(Tile) * cur.size()) != cudaSuccess ||

@@ -370,7 +370,7 @@ struct Pow {
 
 // One window to process.
 struct Win {
-    const uint8_t *data;  // shared memory, sample 0, 16-byte aligned
+    const uint8_t *data;  // shared memory, 16-byte aligned, sample 0 at byte off
     int32_t n;            // samples
     uint8_t *out;         // global output of sample 0
     uint32_t *mask;       // global mask block (nullable)
@@ -378,6 +378,7 @@ struct Win {
     int64_t abs_idx;      // absolute stream index of sample 0
     uint32_t sid;
     bool vec;             // out is 16-byte aligned: vector stores
+    int32_t off;          // any-window form: bytes of data before sample 0 (0..15); else 0
 };
 
 // ------------------------------------------------------------------ phase 1: histogram
@@ -460,6 +461,58 @@ __device__ __forceinline__ void phase_histogram(const Shm &sm, const Win &w, int
             red_add_shared(cb + (((x & 0xFFFu) ^ 0x800u) << 2), 1u);
             bad |= range12_bits(x) & 0xF000u;
         }
+        if (bad) atomicOr(&sm.ctl->err[par], 1u);
+    }
+}
+
+// Any-window form: sample 0 lies off bytes into the first 16-byte chunk. Thread i of the nt that
+// count this window takes the whole chunks c0 + i, c0 + i + nt, ... and, for i < 32, one sample of
+// the partial chunks at the window's ends (nt >= 32).
+template <int BITS, class Word, class One>
+__device__ __forceinline__ void hist_chunks(const Win &w, int i, int nt, Word &&word, One &&one) {
+    constexpr int BPS = Geo<BITS>::kBps, CS = Geo<BITS>::kChunkSamples;
+    const int end = w.off + w.n * BPS;
+    const int c0 = (w.off + 15) >> 4, c1 = end >> 4;  // whole chunks [c0, c1)
+    const uint4 *d4 = reinterpret_cast<const uint4 *>(w.data);
+    int c = c0 + i;
+    for (; c + nt < c1; c += 2 * nt) {
+        const uint4 a = d4[c], b = d4[c + nt];
+        word(a.x); word(a.y); word(a.z); word(a.w);
+        word(b.x); word(b.y); word(b.z); word(b.w);
+    }
+    if (c < c1) {
+        const uint4 a = d4[c];
+        word(a.x); word(a.y); word(a.z); word(a.w);
+    }
+    // samples before chunk c0 (all of them when no chunk is whole), then those from chunk c1 on
+    const int head = min(16 * c0, end) - w.off, tail = c1 >= c0 ? end - 16 * c1 : 0;
+    if (i < CS) {
+        if (i * BPS < head) one(w.off + i * BPS);
+    } else if (i < 2 * CS) {
+        if ((i - CS) * BPS < tail) one(16 * c1 + (i - CS) * BPS);
+    }
+}
+
+template <int BITS, int T>
+__device__ __forceinline__ void phase_histogram_any(const Shm &sm, const Win &w, int tid, int par) {
+    const int lane = tid & 31;
+    if constexpr (BITS == 8) {
+        const uint32_t lb = sm.hist_s + 4u * lane;
+        hist_chunks<8>(w, tid, T, [&](uint32_t v) { hist8_word<128>(lb, v); },
+                       [&](int at) { red_add_shared(lb + (static_cast<uint32_t>(w.data[at]) << 7), 1u); });
+    } else {
+        const uint32_t cb = sm.hist_s + static_cast<uint32_t>(lane & (sm.ncopies - 1)) * 16384u;
+        uint32_t bad = 0;
+        hist_chunks<12>(w, tid, T,
+                        [&](uint32_t v) {
+                            hist12_word(cb, v);
+                            bad |= range12_bits(v);
+                        },
+                        [&](int at) {
+                            const uint32_t x = *reinterpret_cast<const uint16_t *>(w.data + at);
+                            red_add_shared(cb + (((x & 0xFFFu) ^ 0x800u) << 2), 1u);
+                            bad |= range12_bits(x) & 0xF000u;
+                        });
         if (bad) atomicOr(&sm.ctl->err[par], 1u);
     }
 }
@@ -712,6 +765,22 @@ struct Rep8 {
     uint32_t unone;    // M == 127: nothing lies above the median
 };
 
+__device__ __forceinline__ Rep8 load_rep8(const RepShared *rsrc) {
+    const uint4 *rq = reinterpret_cast<const uint4 *>(rsrc);
+    const uint4 q2 = rq[2], q3 = rq[3], q4 = rq[4];
+    Rep8 k;
+    k.mb4 = q2.x;
+    k.tlo7 = q2.y;
+    k.tsmall = q2.z;
+    k.c4 = q2.w;
+    k.hi4 = q3.x;
+    k.lo4 = q3.y;
+    k.ulo7 = q3.z;
+    k.usmall = q3.w;
+    k.unone = q4.x;
+    return k;
+}
+
 // 4 int8 samples: returns the output word and sets f to 0xFF in flagged bytes. Noise bytes are
 // left 0 here and written by the compacted noise pass.
 template <int MODE>
@@ -839,19 +908,16 @@ __device__ __forceinline__ void store_chunk8(uint8_t *out, int c, const uint4 &v
     }
 }
 
-// Digital noise for the flagged samples of up to four rounds of the warp. Lane l holds in nb
-// the 16-bit flag masks of its chunks c0 + k*T (k = 0..3, mask k in bits [16k, 16k+16)). The
-// flagged samples are numbered across the warp (an exclusive prefix sum of the per-lane
-// counts); in each pass lane q takes sample q, found by a shuffle binary search for the lane
-// that owns it and a popcount search for its bit, and all 32 lanes evaluate Philox together.
-// The stores go straight to the output; they follow the chunks' own stores in warp order
+// Digital noise for the flagged samples of one round of the warp: lane l holds in bits the flags of
+// samples s0, s0 + 1, ... The flagged samples are numbered across the warp (an exclusive prefix sum
+// of the per-lane counts); in each pass lane q takes sample q, found by a shuffle binary search for
+// the lane that owns it and a popcount search for its bit, and all 32 lanes evaluate Philox
+// together. The stores go straight to the output; they follow the chunks' own stores in warp order
 // (__syncwarp before the call).
-template <int BITS, int T, bool PW, class K, int OUTF = 0>
-__device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K &p, int lane, int c0,
-                                            uint64_t nb, Pow &pw) {
-    constexpr int CS = Geo<BITS>::kChunkSamples;
-    const uint32_t lo = static_cast<uint32_t>(nb), hi = static_cast<uint32_t>(nb >> 32);
-    const uint32_t cnt = __popc(lo) + __popc(hi);
+template <int BITS, bool PW, class K, int OUTF = 0>
+__device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K &p, int lane, int s0,
+                                            uint32_t bits, Pow &pw) {
+    const uint32_t cnt = __popc(bits);
     uint32_t inc = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -871,15 +937,10 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
             if (e <= q) L += step;
         }
         const uint32_t eL = __shfl_sync(0xFFFFFFFFu, excl, L);
-        const uint32_t loL = __shfl_sync(0xFFFFFFFFu, lo, L);
-        const uint32_t hiL = __shfl_sync(0xFFFFFFFFu, hi, L);
-        const int cL = __shfl_sync(0xFFFFFFFFu, c0, L);
+        const uint32_t bL = __shfl_sync(0xFFFFFFFFu, bits, L);
+        const int sL = __shfl_sync(0xFFFFFFFFu, s0, L);
         if (q < total) {
-            const int j = static_cast<int>(q - eL);
-            const int clo = __popc(loL);
-            const bool inlo = j < clo;
-            const int bp = (inlo ? 0 : 32) + nth_set_bit(inlo ? loL : hiL, inlo ? j : j - clo);
-            const int pos = (cL + (bp >> 4) * T) * CS + (bp & 15);
+            const int pos = sL + nth_set_bit(bL, static_cast<int>(q - eL));
             const int32_t z = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pos);
             store_sample<BITS, OUTF>(w.out, pos, z);
             if (PW) pw.z += static_cast<uint32_t>(z * z);
@@ -891,11 +952,10 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
 // many list entries with one shared atomic, and each lane writes its positions. Windows of
 // 65536 samples (position 65535 would equal the skip mark) and rounds that do not fit in the
 // list take the per-warp path at once; list entries reserved beyond the written ones are
-// marked skipped. Called by all lanes of the warp with the round's chunk c and flag bits.
-template <int BITS, int T, bool PW, class K, int OUTF = 0>
+// marked skipped. Called by all lanes of the warp with the flags of samples s0, s0 + 1, ...
+template <int BITS, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const Rep &r, const K &p, int lane,
-                                             int c, uint32_t bits, uint32_t *nlc, Pow &pw) {
-    constexpr int CS = Geo<BITS>::kChunkSamples;
+                                             int s0, uint32_t bits, uint32_t *nlc, Pow &pw) {
     if (!__any_sync(0xFFFFFFFFu, bits != 0u)) return;
     const uint32_t cnt = __popc(bits);
     uint32_t inc = cnt;
@@ -911,12 +971,12 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
     if (base + total <= static_cast<uint32_t>(kNoiseList)) {
         uint32_t off = base + inc - cnt;
-        for (uint32_t m = bits; m; m &= m - 1u) sm.nlist[off++] = static_cast<uint16_t>(c * CS + __ffs(m) - 1);
+        for (uint32_t m = bits; m; m &= m - 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 + __ffs(m) - 1);
         return;
     }
     for (uint32_t i = base + lane; i < static_cast<uint32_t>(kNoiseList); i += 32) sm.nlist[i] = kNoiseSkip;
     __syncwarp();  // the round's chunk stores come first
-    noise_batch<BITS, T, PW, K, OUTF>(w, r, p, lane, c, static_cast<uint64_t>(bits), pw);
+    noise_batch<BITS, PW, K, OUTF>(w, r, p, lane, s0, bits, pw);
 }
 
 // Digital noise, after the group barrier that follows the replace pass: every thread of the
@@ -1014,7 +1074,8 @@ template <int T, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_deferred8(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
                                                 const uint32_t *nlc, Pow &pw) {
     named_bar(sm.bar_id, T);  // every entry of the window is in the list
-    noise_expand8<T>(sm, *nlc, tid, [&](uint32_t pos) {
+    noise_expand8<T>(sm, *nlc, tid, [&](uint32_t at) {
+        const uint32_t pos = at - static_cast<uint32_t>(w.off);
         if (pos >= static_cast<uint32_t>(w.n)) return;
         const int32_t z = noise_value<8>(r.M, r.D, p, w.sid, w.abs_idx + pos);
         store_sample<8, OUTF>(w.out, static_cast<int>(pos), z);
@@ -1043,18 +1104,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
     const uint4 *d4 = reinterpret_cast<const uint4 *>(w.data);
     uint32_t flagged = 0;
     if (BITS == 8) {
-        const uint4 *rq = reinterpret_cast<const uint4 *>(rsrc);
-        const uint4 q2 = rq[2], q3 = rq[3], q4 = rq[4];
-        Rep8 k;
-        k.mb4 = q2.x;
-        k.tlo7 = q2.y;
-        k.tsmall = q2.z;
-        k.c4 = q2.w;
-        k.hi4 = q3.x;
-        k.lo4 = q3.y;
-        k.ulo7 = q3.z;
-        k.usmall = q3.w;
-        k.unone = q4.x;
+        const Rep8 k = load_rep8(rsrc);
         uint16_t *mk = reinterpret_cast<uint16_t *>(w.mask);
         int base = warp * 32;
         if (r.active && w.vec && mk) {
@@ -1199,12 +1249,104 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
                 }
                 if (mk) mk[c] = static_cast<uint8_t>(bits);
             }
-            if (MODE == 3) noise_append<12, T, PW, K, OUTF>(sm, w, r, p, lane, c, bits, nlc, pw);
+            if (MODE == 3) noise_append<12, PW, K, OUTF>(sm, w, r, p, lane, c * 8, bits, nlc, pw);
         }
         if (mk) {
             for (int c = nchunks + tid; c < 4 * w.mask_words; c += T) mk[c] = 0;
         }
     }
+    return flagged;
+}
+
+// ------------------------------------------------------------------ any-window form
+// The replace pass of a window of any length at any alignment (BPS-aligned), in rounds of 31 chunks:
+// lane l takes the 16-byte chunk base + l of the window as it lies in shared memory, which is how
+// it lies in global memory too, so whole chunks go out as 16-byte stores where in and out are
+// aligned alike. The mask counts bits from sample 0, off samples into the first chunk: its
+// 16-bit piece h (8-bit for 12-bit samples) joins the flags of chunks h and h + 1, the second
+// from the next lane. Lane 31 only gives its flags to lane 30; its chunk is lane 0's of the next
+// round. Returns the lane's flags of its own chunk (0 for lane 31). (Each lane building its own
+// sample-aligned 16 bytes with funnel shifts needs a second load and leaves every store unaligned.)
+template <int BITS, int MODE>
+__device__ __forceinline__ uint32_t replace_round_any(const Win &w, const Rep &r, const RepShared *rsrc, int base, int lane) {
+    constexpr int BPS = Geo<BITS>::kBps, CS = Geo<BITS>::kChunkSamples;
+    const int offs = w.off / BPS;
+    const int c = base + lane;
+    const int lo = c == 0 ? offs : 0;
+    const int hi = min(CS, offs + w.n - c * CS);  // the window's samples of the chunk: [lo, hi)
+    const bool own = lane < 31 && hi > 0;
+    uint32_t bits = 0;
+    if (hi > 0) {
+        const uint4 v = reinterpret_cast<const uint4 *>(w.data)[c];
+        uint32_t ww[4] = {v.x, v.y, v.z, v.w};
+        if (r.active) {
+            uint32_t f[4];
+            if (BITS == 8) {
+                const Rep8 k = load_rep8(rsrc);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) ww[q] = rep8_word<MODE>(ww[q], k, f[q]);
+                bits = chunk_bits(f[0], f[1], f[2], f[3]);
+            } else {
+                const RepShared &k = *rsrc;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) ww[q] = rep12_word<MODE>(ww[q], k.mb4, k.tlo7, k.c4, k.hi4, k.lo4, f[q]);
+                const uint32_t g0 = __byte_perm(f[0], f[1], 0x7531u) & 0x80808080u;
+                const uint32_t g1 = __byte_perm(f[2], f[3], 0x7531u) & 0x80808080u;
+                bits = ((g0 * 0x00204081u) >> 28) | (((g1 * 0x00204081u) >> 28) << 4);
+            }
+            bits &= (1u << hi) - (1u << lo);
+        }
+        if (own) {
+            uint8_t *o = w.out - w.off + 16 * static_cast<int64_t>(c);
+            if (lo == 0 && hi == CS && w.vec) {
+                __stcs(reinterpret_cast<uint4 *>(o), make_uint4(ww[0], ww[1], ww[2], ww[3]));
+            } else if (BITS == 8) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (j >= lo && j < hi) o[j] = static_cast<uint8_t>(ww[j >> 2] >> ((j & 3) * 8));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (j >= lo && j < hi) reinterpret_cast<uint16_t *>(o)[j] = static_cast<uint16_t>(ww[j >> 1] >> ((j & 1) * 16));
+            }
+        }
+    }
+    const uint32_t nb = __shfl_down_sync(0xFFFFFFFFu, bits, 1);
+    if (w.mask && own && c * CS < w.n) {
+        const uint32_t piece = (bits >> offs) | (nb << (CS - offs));
+        if (BITS == 8) reinterpret_cast<uint16_t *>(w.mask)[c] = static_cast<uint16_t>(piece);
+        else reinterpret_cast<uint8_t *>(w.mask)[c] = static_cast<uint8_t>(piece);
+    }
+    return own ? bits : 0u;
+}
+
+// Mask pieces past the window's last sample.
+template <int BITS>
+__device__ __forceinline__ void mask_padding(const Win &w, int i, int nt) {
+    constexpr int CS = Geo<BITS>::kChunkSamples;
+    if (!w.mask) return;
+    for (int h = (w.n + CS - 1) / CS + i; h < w.mask_words * (32 / CS); h += nt) {
+        if (BITS == 8) reinterpret_cast<uint16_t *>(w.mask)[h] = 0;
+        else reinterpret_cast<uint8_t *>(w.mask)[h] = 0;
+    }
+}
+
+template <int BITS, int MODE, int T, class K>
+__device__ __forceinline__ uint32_t phase_replace_any(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
+                                                      uint32_t *nlc, Pow &pw, const RepShared *rsrc) {
+    constexpr int BPS = Geo<BITS>::kBps, CS = Geo<BITS>::kChunkSamples;
+    const int lane = tid & 31, warp = tid >> 5;
+    const int nch = (w.off + w.n * BPS + 15) >> 4;
+    uint32_t flagged = 0;
+    for (int base = warp * 31; base < nch; base += (T / 32) * 31) {
+        const uint32_t bits = replace_round_any<BITS, MODE>(w, r, rsrc, base, lane);
+        flagged += __popc(bits);
+        if (MODE == 3) {
+            if (BITS == 8) noise_note8(sm, lane, base + lane, bits, nlc);
+            else noise_append<12, false, K>(sm, w, r, p, lane, (base + lane) * CS - w.off / BPS, bits, nlc, pw);
+        }
+    }
+    mask_padding<BITS>(w, tid, T);
     return flagged;
 }
 
@@ -1234,6 +1376,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     constexpr bool COPIES = (MODE & kModeCopies) != 0;
     constexpr int OUTF = (MODE & kModeF16) ? 1 : ((MODE & kModeBF16) ? 2 : 0);
     constexpr int RMODE = MODE & 3;
+    constexpr bool ANY = (MODE & kModeAny) != 0;
     const int lane = tid & 31;
     if (STATS) {
         // Estimation only (the first pass of Eq. 3): M and D of the window. Nothing reads the
@@ -1242,7 +1385,10 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         // the stage's descriptor, which the copy warp rewrites once the stage is released: its
         // output pointers are taken first.
         int32_t *const med = sg.med, *const mad = sg.mad;
-        if (stage_ok) phase_histogram<BITS, T, ROWB>(sm, w, tid, par);
+        if (stage_ok) {
+            if constexpr (ANY) phase_histogram_any<BITS, T>(sm, w, tid, par);
+            else phase_histogram<BITS, T, ROWB>(sm, w, tid, par);
+        }
         if (named_bar_or(sm.bar_id, T, !stage_ok)) return false;
         if (tid == 0 && release_bar) mbar_arrive(release_bar);
         // int8: the counts go to one warp, which scans them and searches while the other warps
@@ -1262,7 +1408,10 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         return true;
     }
     if (!APPLY) {
-        if (stage_ok) phase_histogram<BITS, T, ROWB>(sm, w, tid, par);
+        if (stage_ok) {
+            if constexpr (ANY) phase_histogram_any<BITS, T>(sm, w, tid, par);
+            else phase_histogram<BITS, T, ROWB>(sm, w, tid, par);
+        }
         if (named_bar_or(sm.bar_id, T, !stage_ok)) return false;
         if (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
         else phase_reduce_scan12<T>(sm, tid, w.n);
@@ -1284,7 +1433,9 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     uint32_t f = 0;
     Pow pw = {0u, 0u};
     const KeysPre key{p};
-    if (!STATS && !COPIES)
+    if constexpr (ANY && !STATS)
+        f = phase_replace_any<BITS, RMODE, T, KeysPre>(sm, w, r, key, tid, &sm.ctl->ncount[par], pw, &sm.ctl->rep);
+    else if (!STATS && !COPIES)
         f = phase_replace<BITS, RMODE, T, PW, KeysPre, OUTF, (MODE & kModeFlaggedOnly) != 0>(
             sm, w, r, key, tid, &sm.ctl->ncount[par], pw, &sm.ctl->rep);
     if (!STATS && !COPIES && RMODE == 3) {
@@ -1405,18 +1556,7 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
     for (int c0 = warp * 32; c0 < nchunks; c0 += T) {
         const int k = c0 >> lcw;
         const RepShared &rk = reps[k];
-        const uint4 *rq = reinterpret_cast<const uint4 *>(&rk);
-        const uint4 q2 = rq[2], q3 = rq[3], q4 = rq[4];
-        Rep8 k8;
-        k8.mb4 = q2.x;
-        k8.tlo7 = q2.y;
-        k8.tsmall = q2.z;
-        k8.c4 = q2.w;
-        k8.hi4 = q3.x;
-        k8.lo4 = q3.y;
-        k8.ulo7 = q3.z;
-        k8.usmall = q3.w;
-        k8.unone = q4.x;
+        const Rep8 k8 = load_rep8(&rk);
         const int c = c0 + lane;
         uint4 v = d4[c];
         uint32_t bits = 0;
@@ -1613,6 +1753,105 @@ __device__ bool process_tile_multi8(const Shm &sm, const uint8_t *stage, const S
     if (STATS) return true;
     named_bar(sm.bar_id, T);
     replace_tile8<MODE & 3, T>(sm, stage, sg, w0, nw, lw, sm.mt->rep, sm.mt->count, p, tid, par, release_bar);
+    return true;
+}
+
+// ------------------------------------------------------------------ multi-window tiles of any windows
+// nw (1 <= nw <= K) windows of up to 8192 samples each, of any length at any alignment: window slot g
+// starts off + g * W bytes into the stage, the last one may be shorter. As process_tile_multi8 with
+// the histogram and replace rounds of the any-window form; a warp's replace round is 31 chunks of
+// one window. A noise-list entry's chunk number holds the slot above bit 10 (a window of 8192
+// samples has at most 514 chunks).
+template <int MODE, int T, int K>
+__device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, const Seg &sg, uint32_t w0, int nw,
+                                  const Params &p, int tid, int par, uint32_t release_bar) {
+    constexpr bool STATS = (MODE & kModeStats) != 0;
+    constexpr int RMODE = MODE & 3;
+    constexpr int NW = T / 32, LPS = 32 / K, TS = T / K;
+    static_assert(TS >= 32, "hist_chunks needs 32 threads per window");
+    const int lane = tid & 31, warp = tid >> 5;
+    int32_t *const med = sg.med, *const mad = sg.mad;  // sg lives in the stage descriptor
+    const int W = sg.W;
+    const int64_t left = sg.len - static_cast<int64_t>(w0) * W;
+    auto window = [&](int g) {
+        Win w;
+        const int64_t k = static_cast<int64_t>(w0) + g;
+        const int64_t left = sg.len - k * W;
+        const int at = off + g * W;
+        w.data = stage + (at & ~15);
+        w.off = at & 15;
+        w.n = static_cast<int32_t>(left < W ? left : W);
+        w.out = sg.out + k * W;
+        w.mask = sg.mask ? sg.mask + k * sg.mask_words : nullptr;
+        w.mask_words = sg.mask_words;
+        w.abs_idx = sg.abs0 + k * W;
+        w.sid = sg.stream_id;
+        w.vec = ((reinterpret_cast<uintptr_t>(w.out) - w.off) & 15u) == 0u;
+        return w;
+    };
+    if (lane / LPS < nw) {
+        const Win w = window(lane / LPS);
+        const uint32_t lb = sm.hist_s + 4u * lane;
+        hist_chunks<8>(w, warp * LPS + lane % LPS, TS, [&](uint32_t v) { hist8_word<128>(lb, v); },
+                       [&](int at) { red_add_shared(lb + (static_cast<uint32_t>(w.data[at]) << 7), 1u); });
+    }
+    if (named_bar_or(sm.bar_id, T, false)) return false;
+    if (STATS && tid == 0 && release_bar) mbar_arrive(release_bar);
+    reduce8_multi<T, K>(sm, tid);
+    named_bar(sm.bar_id, T);
+    for (int g = warp; g < nw; g += NW) {
+        RepShared *rep = &sm.mt->rep[g];
+        const int64_t lg = left - static_cast<int64_t>(g) * W;
+        scan_search8(reinterpret_cast<uint16_t *>(sm.cum) + g * Geo<8>::kCumWords, static_cast<int>(lg < W ? lg : W), lane,
+                     p.kq, p.cval, rep);
+        __syncwarp();
+        if (lane == 0) {
+            if (med) med[w0 + g] = rep->M;
+            if (mad) mad[w0 + g] = rep->D;
+        }
+    }
+    if (STATS) return true;
+    named_bar(sm.bar_id, T);
+    if constexpr (!STATS) {
+        const RepShared *reps = sm.mt->rep;
+        const int rpw = ((15 + W + 15) / 16 + 30) / 31;  // rounds of a window
+        for (int q = warp; q < nw * rpw; q += NW) {
+            const int g = q / rpw, base = (q - g * rpw) * 31;
+            const Win w = window(g);
+            const uint32_t bits = replace_round_any<8, RMODE>(w, load_rep(reps[g]), &reps[g], base, lane);
+            if (RMODE == 3) noise_note8(sm, lane, (g << 10) + base + lane, bits, &sm.ctl->ncount[par]);
+            const uint32_t wf = __reduce_add_sync(0xFFFFFFFFu, __popc(bits));
+            if (lane == 0 && wf) atomicAdd(&sm.mt->count[g], wf);
+            if (base == 0) mask_padding<8>(w, lane, 32);
+        }
+        if (RMODE == 3) {
+            named_bar(sm.bar_id, T);  // every entry of the windows is in the list
+            const KeysPre key{p};
+            noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t at) {
+                const int g = static_cast<int>(at >> 14);
+                const int64_t i = (static_cast<int64_t>(w0) + g) * W + static_cast<int>(at & 16383u) - ((off + g * W) & 15);
+                sg.out[i] = static_cast<uint8_t>(noise_value<8>(reps[g].M, reps[g].D, key, sg.stream_id, sg.abs0 + i));
+            });
+        }
+        if (lane == 0) {
+            __threadfence_block();
+            if (atomicAdd(&sm.ctl->done[par], 1u) == NW - 1) {
+                // last warp: every count is in and every read of the stage is done
+                __threadfence_block();
+                sm.ctl->done[par] = 0u;
+                if (RMODE == 3) sm.ctl->ncount[par] = 0u;  // every warp has read it
+                unsigned long long tot = 0ull;
+                for (int g = 0; g < nw; ++g) {
+                    const uint32_t cg = sm.mt->count[g];
+                    sm.mt->count[g] = 0u;
+                    if (sg.counts) sg.counts[w0 + g] = cg;
+                    tot += cg;
+                }
+                sm.ctl->flagged += tot;
+                if (release_bar) mbar_arrive(release_bar);
+            }
+        }
+    }
     return true;
 }
 

@@ -45,6 +45,42 @@ constexpr int kModeFlaggedOnly = 512;
 // mbarriers. Its own instantiation, chosen by the launch shape (Shape::warp_split == 2).
 constexpr int kModeWarpSplit = 1024;
 
+// Flag bit of the any-window form (plain excision, the estimation pass and the apply passes; one
+// group of 8 consumer warps): the copy warp stages a tile's bytes as they lie in global memory,
+// rounded out to 16-byte chunks, and the window phases take windows that start and end anywhere in
+// a chunk; several 8-bit windows of up to kMultiMaxWindow samples of any length share a histogram
+// table as in the multi-window form. For plans with windows that the aligned forms serve badly
+// (needs_any_form). 24 int8 streams of 2^18..2^22 samples in windows of 1000..40000, threshold: 200 -> 65
+// us a call (host included); 24 x 2466361 int8 samples in 2000-sample windows: 126 -> 77 us; 1.04 G
+// 12-bit samples in 829-sample windows, noise: 28.8 -> 14.7 ms.
+constexpr int kModeAny = 2048;
+constexpr int kMultiMaxWindow = 8192;  // largest window that shares a table (16-bit counts, list entries)
+
+// Windows of 2^l = 512..8192 int8 samples share a table in the multi-window form.
+inline bool multi_window(int bits, int32_t W) {
+    return bits == 8 && W >= 512 && W <= kMultiMaxWindow && (W & (W - 1)) == 0;
+}
+// Whether the aligned forms serve a stream of windows W badly: windows whose bytes are no multiple
+// of 16 are loaded byte by byte by the consumers with no copy in flight and stored byte by byte,
+// one window a tile; int8 windows of up to 8192 samples that are no power of two go one at a time
+// through the histogram's reduce and the barriers.
+inline bool needs_any_form(int bits, int32_t W, int64_t len) {
+    const int bps = bits == 8 ? 1 : 2;
+    if (static_cast<int64_t>(W) * bps % 16 != 0) return len > 16;
+    return bits == 8 && W <= kMultiMaxWindow && !multi_window(bits, W) && len >= 2 * static_cast<int64_t>(W);
+}
+// Windows per tile of a stage: as many whole ones as fit (the any-window form keeps 16 bytes for
+// the tile's distance to the 16-byte boundary before it).
+inline int64_t tile_windows(int bits, int mode, int32_t W, int stage_bytes) {
+    const int64_t wb = static_cast<int64_t>(W) * (bits == 8 ? 1 : 2);
+    if (mode & kModeAny) return (stage_bytes - 16) / wb > 1 ? (stage_bytes - 16) / wb : 1;
+    return wb % 16 == 0 && stage_bytes / wb > 1 ? stage_bytes / wb : 1;
+}
+// Smallest stage for windows of up to wb bytes.
+inline int min_stage_bytes(int mode, int64_t wb) {
+    return static_cast<int>((wb + ((mode & kModeAny) ? 16 : 0) + 127) / 128 * 128);
+}
+
 // One variant of a digital-copy pass.
 struct Variant {
     int64_t kq;     // round(k * 1.4826 * 2^16)

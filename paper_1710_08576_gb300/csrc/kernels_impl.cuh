@@ -63,7 +63,8 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     Layout L;
     L.grp = (mode & kModeApply) ? 0 : align_up(Geo<BITS>::hist_bytes(ncopies, groups), 128);
     // multi-window tiles: 8-bit, one group, plain excision or the estimation pass
-    const bool multi = BITS == 8 && groups == 1 && (mode & kModeMulti) != 0;
+    const bool multi = BITS == 8 && groups == 1 &&
+                       ((mode & kModeMulti) != 0 || ((mode & kModeAny) != 0 && (mode & kModeApply) == 0));
     L.cum = 0;
     // (multi-window tiles: up to kMultiMax slots of 16-bit counts)
     L.ctl = align_up(multi ? Geo<BITS>::kCumWords * 2 * kMultiMax : Geo<BITS>::kCumWords * 4, 128);
@@ -79,7 +80,8 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     // then each consumer warp's ring of kNoiseRing 32-bit positions (multi-window tiles keep the
     // rings in their cumulative-count area, which is idle by then and large enough); 12-bit: the
     // position list
-    const int list_bytes = align_up(stage_bytes / 4 > 128 ? stage_bytes / 4 : 128, 128);
+    // (any-window tiles: a chunk that two windows share has an entry for each)
+    const int list_bytes = align_up(stage_bytes / 4 > 128 ? stage_bytes / 4 : 128, 128) + ((mode & kModeAny) ? 128 : 0);
     const int ring_bytes = multi ? 0 : cw * kNoiseRing * 4;
     static_assert(kNoiseRing * 4 * 16 <= Geo<8>::kCumWords * 2 * kMultiMax, "rings of 16 warps fit the multi-window counts");
     const int noise_bytes = BITS == 8 ? list_bytes + ring_bytes : kNoiseList * 2;
@@ -138,6 +140,17 @@ __device__ __forceinline__ Win make_win(const Seg &sg, int64_t w, const uint8_t 
     win.abs_idx = sg.abs0 + s0;
     win.sid = sg.stream_id;
     win.vec = sg.vec != 0;
+    win.off = 0;
+    return win;
+}
+
+// Any-window form: window w of a tile whose first window w0 starts `off` bytes into the stage.
+__device__ __forceinline__ Win make_win_any(const Seg &sg, int64_t w, uint32_t w0, const uint8_t *stage, int off, int bps) {
+    Win win = make_win(sg, w, stage, bps);
+    const int at = off + static_cast<int>(w - w0) * sg.W * bps;
+    win.data = stage + (at & ~15);
+    win.off = at & 15;
+    win.vec = ((reinterpret_cast<uintptr_t>(win.out) - win.off) & 15u) == 0u;
     return win;
 }
 
@@ -356,6 +369,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
         constexpr int kLaneIn = 4 + offsetof(Seg, in) / 4, kLaneMed = 4 + offsetof(Seg, med) / 4;
         constexpr int kLaneMad = 4 + offsetof(Seg, mad) / 4, kLaneW = 4 + offsetof(Seg, W) / 4;
         constexpr int kLaneVec = 4 + offsetof(Seg, vec) / 4;
+        [[maybe_unused]] constexpr int kLaneLen = 4 + offsetof(Seg, len) / 4;
         const uint32_t *tile_w = reinterpret_cast<const uint32_t *>(tiles);
         const uint32_t *seg_w = reinterpret_cast<const uint32_t *>(segs);
         auto grab = [&](int i) -> int {  // lane 0: the group's tile of iteration i
@@ -428,13 +442,38 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                 }
             }
             const uint8_t *src = in + static_cast<int64_t>(w0) * W * BPS;
-            const uint32_t bulk = vec ? (tbytes & ~15u) : 0u, rem = tbytes & 15u;
-            if (vec && static_cast<uint32_t>(lane) < rem) stage[bulk + lane] = src[bulk + lane];
-            __syncwarp();
-            if (lane == 0) {
-                meta[s].tidx = t;
-                mbar_arrive_tx(full_bar(s), bulk);
-                if (bulk) bulk_g2s(smem_addr(stage), src, bulk, full_bar(s));
+            if constexpr ((MODE & kModeAny) != 0) {
+                // the tile's bytes at their distance from the 16-byte boundary before them: the whole
+                // chunks inside the run by one bulk copy (a chunk may hold bytes of the windows
+                // before or after), the bytes of partial chunks at the run's ends by the lanes
+                const uint64_t len = static_cast<uint64_t>(__shfl_sync(kAll, dw, kLaneLen)) |
+                                     (static_cast<uint64_t>(__shfl_sync(kAll, dw, kLaneLen + 1)) << 32);
+                const uint64_t lo = reinterpret_cast<uint64_t>(src), hi = lo + tbytes;
+                const uint64_t in0 = reinterpret_cast<uint64_t>(in), in1 = in0 + len * BPS;
+                uint8_t *const at = stage - (lo & ~15ull);  // address a goes to at + a
+                uint64_t b0 = lo & ~15ull, b1 = (hi + 15) & ~15ull;
+                if (b0 < in0) b0 += 16;
+                if (b1 > in1) b1 -= 16;
+                const uint32_t bulk = b1 > b0 ? static_cast<uint32_t>(b1 - b0) : 0u;
+                // at most 15 bytes before b0 and 15 from b1 on; without a whole chunk, at most 30
+                const uint64_t a = bulk == 0u ? lo + lane : (lane < 16 ? lo + lane : b1 + (lane - 16));
+                if (bulk == 0u ? a < hi : (lane < 16 ? a < b0 : a < hi)) at[a] = *reinterpret_cast<const uint8_t *>(a);
+                __syncwarp();
+                if (lane == 0) {
+                    meta[s].tidx = t;
+                    mbar_arrive_tx(full_bar(s), bulk);
+                    if (bulk) bulk_g2s(smem_addr(stage) + static_cast<uint32_t>(b0 - (lo & ~15ull)),
+                                       reinterpret_cast<const void *>(b0), bulk, full_bar(s));
+                }
+            } else {
+                const uint32_t bulk = vec ? (tbytes & ~15u) : 0u, rem = tbytes & 15u;
+                if (vec && static_cast<uint32_t>(lane) < rem) stage[bulk + lane] = src[bulk + lane];
+                __syncwarp();
+                if (lane == 0) {
+                    meta[s].tidx = t;
+                    mbar_arrive_tx(full_bar(s), bulk);
+                    if (bulk) bulk_g2s(smem_addr(stage), src, bulk, full_bar(s));
+                }
             }
             // advance the descriptor pipeline by one iteration
             dw = desc_word(t1, tw1);
@@ -486,7 +525,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
         const Tile tl = meta[s].tile;
         const Seg &sg = meta[s].seg;
         uint8_t *stage = stage0 + s * stage_bytes;
-        if (!sg.vec) {
+        if ((MODE & kModeAny) == 0 && !sg.vec) {
             const uint8_t *src = sg.in + static_cast<int64_t>(tl.w0) * sg.W * BPS;
             for (int i = tid; i < static_cast<int>(tl.bytes); i += T) stage[i] = src[i];
             if (named_bar_or(sm.bar_id, T, false)) {
@@ -544,9 +583,45 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
             }
             dirty = true;
         }
+        // any-window form: the tile's distance from the 16-byte boundary before it
+        const int toff = (MODE & kModeAny)
+                             ? static_cast<int>((reinterpret_cast<uint64_t>(sg.in) + static_cast<uint64_t>(tl.w0) * sg.W * BPS) & 15u)
+                             : 0;
+        if constexpr (BITS == 8 && G == 1 && CW == 8 && (MODE & kModeAny) != 0 && (MODE & kModeApply) == 0) {
+            // several windows of up to 8192 samples: four or eight at a time share the histogram
+            // table, the reduce, the barriers and the searches
+            if (tl.nw >= 2u && sg.W <= kMultiMaxWindow) {
+                if (dirty) {
+                    zero_shared(sm.hist, 32768, tid, T);
+                    named_bar(sm.bar_id, T);
+                    dirty = false;
+                }
+                const uint32_t K = tl.nw > 4u ? 8u : 4u;
+                for (uint32_t k0 = 0; k0 < tl.nw && alive; k0 += K) {
+                    const int nwk = static_cast<int>(tl.nw - k0 < K ? tl.nw - k0 : K);
+                    const uint32_t rel = k0 + K >= tl.nw ? empty_bar(s) : 0u;
+                    const int at = toff + static_cast<int>(k0) * sg.W;
+                    if (K == 8u)
+                        alive = process_tile_any8<MODE & ~kModeAny, T, 8>(sm, stage + (at & ~15), at & 15, sg, tl.w0 + k0, nwk, p,
+                                                                          tid, par, rel);
+                    else
+                        alive = process_tile_any8<MODE & ~kModeAny, T, 4>(sm, stage + (at & ~15), at & 15, sg, tl.w0 + k0, nwk, p,
+                                                                          tid, par, rel);
+                    par ^= 1;
+                }
+                rs = {{0u, 0u}};  // the reduce left the table zero
+                if (!alive) {
+                    timed_out = true;
+                    break;
+                }
+                continue;
+            }
+            dirty = true;
+        }
         for (uint32_t k = 0; k < tl.nw && alive; ++k) {
             const int64_t widx = static_cast<int64_t>(tl.w0) + k;
-            const Win win = make_win(sg, widx, stage + k * sg.W * BPS, (MODE & (kModeF16 | kModeBF16)) ? 2 : BPS);
+            const Win win = (MODE & kModeAny) ? make_win_any(sg, widx, tl.w0, stage, toff, BPS)
+                                              : make_win(sg, widx, stage + k * sg.W * BPS, (MODE & (kModeF16 | kModeBF16)) ? 2 : BPS);
             const int2 *amd = ((MODE & kModeApply) && tl.nw <= kApplyTileWindows)
                                   ? reinterpret_cast<const int2 *>(gb + L.amd) + s * kApplyTileWindows + k
                                   : nullptr;

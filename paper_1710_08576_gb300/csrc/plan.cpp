@@ -49,7 +49,7 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
         maxwb = std::max<int64_t>(maxwb, first);
         if (P->W[i] != P->W[0]) uniform = false;
     }
-    const int min_stage = static_cast<int>((maxwb + 127) / 128 * 128);
+    const int min_stage = min_stage_bytes(plan_tile_mode(P), maxwb);
     s.consumer_warps = (req && req->consumer_warps) ? req->consumer_warps : 8;
     s.groups = (req && req->groups) ? req->groups : 1;
     if (P->out_format != RFI_OUT_SAME) {  // the output formats are built for one group of 8 warps
@@ -85,7 +85,7 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
     s.ctas_per_sm = std::min(want_ctas, occ);
     P->grid_apply = 0;
     if (P->kmom >= 2) {
-        const int occ_apply = persistent_occupancy(P->bits, kModeApply + (P->fill ? 0 : P->mode), s);
+        const int occ_apply = persistent_occupancy(P->bits, plan_apply_mode(P), s);
         if (occ_apply < 1) return cudaGetLastError() != cudaSuccess ? RFI_ERR_CUDA : RFI_ERR_UNSUPPORTED;
         P->grid_apply = P->sm_count * occ_apply;  // clamped to the tile count with the grid
     }
@@ -105,8 +105,7 @@ rfi_status plan_build_tiles(rfi_plan_s *P) {
     const int bps = P->bits == 8 ? 1 : 2;
     std::vector<Tile> tiles;
     for (int i = 0; i < P->S; ++i) {
-        const int64_t wb = static_cast<int64_t>(P->W[i]) * bps;
-        int64_t per = (wb % 16 == 0) ? std::max<int64_t>(1, P->shape.stage_bytes / wb) : 1;
+        int64_t per = tile_windows(P->bits, plan_tile_mode(P), P->W[i], P->shape.stage_bytes);
         if (P->kmom >= 2) per = std::min<int64_t>(per, kApplyTileWindows);
         for (int64_t w0 = 0; w0 < P->nwin[i]; w0 += per) {
             const int64_t nw = std::min<int64_t>(per, P->nwin[i] - w0);
@@ -251,7 +250,7 @@ rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st) {
     RFI_CUDA(launch_mom(P->bits, P->d_mchunks, static_cast<int>(P->mchunks.size()), P->d_mad, P->d_mom, P->kmom,
                         st));
     RFI_CUDA(cudaMemsetAsync(&P->d_ctr->tile_counter, 0, sizeof(unsigned), st));
-    RFI_CUDA(launch_persistent(P->bits, kModeApply + (P->fill ? 0 : P->mode), P->shape, P->grid_apply, P->d_segs + P->S,
+    RFI_CUDA(launch_persistent(P->bits, plan_apply_mode(P), P->shape, P->grid_apply, P->d_segs + P->S,
                                P->d_tiles, P->ntiles, p, &P->d_ctr->tile_counter, 0, st));
     // the apply segments hold each window's M and its MoM: the noise spread of Eq. 3
     if (P->fill)
@@ -459,13 +458,24 @@ static rfi_status plan_create(const rfi_plan_desc *d, int32_t nvar, const rfi_va
     P->write_flagged = (P->flags & RFI_PLAN_WRITE_FLAGGED) != 0;
     P->fill = (P->flags & RFI_PLAN_NOISE_PASS) && P->mode == RFI_REPLACE_NOISE && !(P->flags & RFI_PLAN_PER_STREAM) &&
               !P->power && P->ncopy == 0 && P->out_format == RFI_OUT_SAME && short_segs && !P->write_flagged;
-    // small windows of 2^l samples: the multi-window form of the 8-bit kernel (several windows
-    // per histogram, reduce and set of barriers)
-    if (P->bits == 8 && P->ncopy == 0 && !P->power && P->out_format == RFI_OUT_SAME &&
-        !(P->flags & RFI_PLAN_PER_STREAM) && !P->write_flagged) {
-        for (int i = 0; i < P->S && !P->multi; ++i) {
-            const int32_t W = P->W[i];
-            P->multi = W >= 512 && W <= 8192 && (W & (W - 1)) == 0 && P->len[i] >= 2 * static_cast<int64_t>(W);
+    if (P->ncopy == 0 && !P->power && P->out_format == RFI_OUT_SAME && !(P->flags & RFI_PLAN_PER_STREAM) &&
+        !P->write_flagged) {
+        // small windows of 2^l samples: the multi-window form of the 8-bit kernel (several windows
+        // per histogram, reduce and set of barriers)
+        for (int i = 0; i < P->S && !P->multi; ++i)
+            P->multi = multi_window(P->bits, P->W[i]) && P->len[i] >= 2 * static_cast<int64_t>(P->W[i]);
+        // windows that the aligned forms serve badly: the any-window form (built for one group of 8
+        // consumer warps), where they are enough of the plan: it takes their byte-wise loads from
+        // about 8 to 1 times an aligned window's time and the small ones from 1.6 to 1, and costs the
+        // plan's other windows up to a tenth (31 of 32 lanes own a chunk; no split-warp form)
+        const rfi_launch_shape *q = d->shape;
+        if (!q || ((q->consumer_warps == 0 || q->consumer_warps == 8) && q->groups <= 1 && q->warp_split <= 1)) {
+            uint64_t bytewise = 0, small = 0;
+            for (int i = 0; i < P->S; ++i) {
+                if (!needs_any_form(P->bits, P->W[i], P->len[i])) continue;
+                (static_cast<int64_t>(P->W[i]) * (P->bits == 8 ? 1 : 2) % 16 ? bytewise : small) += P->len[i];
+            }
+            P->any = 70 * bytewise + 7 * small > total_s;
         }
     }
 

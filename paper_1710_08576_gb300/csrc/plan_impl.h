@@ -57,6 +57,8 @@ struct rfi_plan_s {
     bool power = false;
     // some stream has windows of 2^l samples, 512 <= 2^l <= 8192: the multi-window form
     bool multi = false;
+    // windows that the aligned forms serve badly: the any-window form (needs_any_form)
+    bool any = false;
     // RFI_PLAN_WRITE_FLAGGED: in place, only changed chunks are stored
     bool write_flagged = false;
     uint64_t *d_pow = nullptr;
@@ -126,9 +128,18 @@ inline int plan_kernel_mode(const rfi_plan_s *P) {
     if (P->ncopy > 0) return kModeCopies;
     const int m = (P->fill && P->kmom < 2 ? 0 : P->mode) | (P->power ? kModePower : 0) | fmt;
     if (P->write_flagged) return m | kModeFlaggedOnly;
+    if (P->any) return m | kModeAny;
     return m | (P->multi && m < 4 ? kModeMulti : 0);
 }
 // Kernel mode of the estimation pass of a Median-of-MAD plan.
-inline int plan_stats_mode(const rfi_plan_s *P) { return kModeStats | (P->multi ? kModeMulti : 0); }
+inline int plan_stats_mode(const rfi_plan_s *P) {
+    return kModeStats | (P->any ? kModeAny : (P->multi ? kModeMulti : 0));
+}
+// Kernel mode of the apply pass of a Median-of-MAD plan.
+inline int plan_apply_mode(const rfi_plan_s *P) {
+    return (kModeApply + (P->fill ? 0 : P->mode)) | (P->any ? kModeAny : 0);
+}
+// The mode that the plan's stages and tiles are sized for.
+inline int plan_tile_mode(const rfi_plan_s *P) { return P->any ? kModeAny : 0; }
 
 }  // namespace rfi

@@ -45,6 +45,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -175,6 +176,7 @@ struct KeysSeed {
 // second product (of the stream) and round 2's first product (of a word that holds no idx_lo).
 struct NoiseKey {
     uint32_t a, b, c;  // round 2: z = a ^ (low product of round 1), x = b ^ ...; round 3: z = c ^ ...
+    NoiseKey() = default;
     template <class K>
     __device__ __forceinline__ NoiseKey(const K &key, uint32_t sid, uint32_t idx_hi) {
         const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * sid;
@@ -243,13 +245,50 @@ struct NoiseScale {
     }
 };
 
+// A tile's noise words, computed by the copy warp when it stages the tile: every thread of the
+// group computing them per window costs as much as they save on a window with few flags.
+struct TileNoise {
+    NoiseKey nk;
+    uint32_t one_hi;  // every index of the tile has the same high word
+};
+
+// Noise over a run of samples of one stream starting at absolute index abs0: value(pos, sig2, moff)
+// for sample abs0 + pos. The words that the samples share are computed once where the run's
+// indices have one high word (every run but one across a multiple of 2^32).
 template <int BITS, class K>
-__device__ __forceinline__ int32_t noise_value(int32_t M, uint32_t D, const K &key, uint32_t sid, int64_t idx) {
-    const uint64_t i = static_cast<uint64_t>(idx);
-    const NoiseKey nk(key, sid, static_cast<uint32_t>(i >> 32));
-    return NoiseScale<BITS>::value(noise_sum(nk, key, static_cast<uint32_t>(i)), NoiseScale<BITS>::kSig2 * static_cast<int32_t>(D),
-                                   M - NoiseScale<BITS>::kOff);
-}
+struct NoiseRun {
+    const K &key;
+    NoiseKey nk;
+    uint64_t abs0;
+    uint32_t sid;
+    bool one_hi;
+    __device__ __forceinline__ NoiseRun(const K &k, uint32_t stream, uint64_t a0, uint64_t n)
+        : key(k), nk(k, stream, static_cast<uint32_t>(a0 >> 32)), abs0(a0), sid(stream),
+          one_hi(((a0 ^ (a0 + n - 1)) >> 32) == 0) {}
+    // the words as the tile's copy warp left them (TileNoise)
+    __device__ __forceinline__ NoiseRun(const K &k, uint32_t stream, uint64_t a0, const TileNoise &t)
+        : key(k), nk(t.nk), abs0(a0), sid(stream), one_hi(t.one_hi != 0u) {}
+    __device__ __forceinline__ uint32_t sum(uint32_t pos) const {
+        if (one_hi) return noise_sum(nk, key, static_cast<uint32_t>(abs0) + pos);
+        const uint64_t idx = abs0 + pos;
+        return noise_sum(NoiseKey(key, sid, static_cast<uint32_t>(idx >> 32)), key, static_cast<uint32_t>(idx));
+    }
+    __device__ __forceinline__ int32_t value(uint32_t pos, int32_t sig2, int32_t moff) const {
+        return NoiseScale<BITS>::value(sum(pos), sig2, moff);
+    }
+    // two samples at a time: their Philox chains are independent and interleave
+    __device__ __forceinline__ int2 value2(uint32_t pa, uint32_t pb, int32_t sig2, int32_t moff) const {
+        uint32_t a, b;
+        if (one_hi) {
+            a = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pa);
+            b = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pb);
+        } else {
+            a = sum(pa);
+            b = sum(pb);
+        }
+        return make_int2(NoiseScale<BITS>::value(a, sig2, moff), NoiseScale<BITS>::value(b, sig2, moff));
+    }
+};
 
 // ------------------------------------------------------------------ shared-memory layout
 template <int BITS>
@@ -285,7 +324,8 @@ __device__ __forceinline__ int pad32(int b) { return b + (b >> 5); }
 
 struct __align__(16) RepShared {
     int32_t M, D, t, hiv, lov;
-    uint32_t active, pad[2];
+    uint32_t active;
+    int32_t sig2, moff;  // digital noise (NoiseScale)
     // int8 replace constants (see Rep8)
     uint32_t mb4, tlo7, tsmall, c4, hi4, lo4, ulo7, usmall;
     uint32_t unone;
@@ -379,6 +419,15 @@ struct Win {
     uint32_t sid;
     bool vec;             // out is 16-byte aligned: vector stores
     int32_t off;          // any-window form: bytes of data before sample 0 (0..15); else 0
+    const TileNoise *tn;  // the tile's noise words (digital noise with the kernel's own key; else null)
+    // noise of this window
+    template <int BITS, class K>
+    __device__ __forceinline__ NoiseRun<BITS, K> noise(const K &key) const {
+        if constexpr (std::is_same<K, KeysPre>::value) {
+            if (tn) return NoiseRun<BITS, K>(key, sid, static_cast<uint64_t>(abs_idx), *tn);
+        }
+        return NoiseRun<BITS, K>(key, sid, static_cast<uint64_t>(abs_idx), static_cast<uint64_t>(n));
+    }
 };
 
 // ------------------------------------------------------------------ phase 1: histogram
@@ -665,6 +714,7 @@ struct Rep {
     int32_t cval;     // constant replacement (saturated)
     int32_t t;        // min(ceil(Kq*D / 2^16), sample span + 1)
     int32_t hiv, lov; // threshold replacement above / below (saturated)
+    int32_t sig2, moff;  // digital noise (NoiseScale)
     bool active;      // some sample can be flagged
 };
 
@@ -687,7 +737,8 @@ __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, 
     r.hiv = sat_to(static_cast<int64_t>(r.M) + c, Geo<BITS>::kLo, Geo<BITS>::kHi);
     r.lov = sat_to(static_cast<int64_t>(r.M) - c, Geo<BITS>::kLo, Geo<BITS>::kHi);
     r.active = (d > 0 && t <= SPAN) ? 1u : 0u;  // |x - M| never exceeds the sample span
-    r.pad[0] = r.pad[1] = 0u;
+    r.sig2 = NoiseScale<BITS>::kSig2 * d;
+    r.moff = M - NoiseScale<BITS>::kOff;
     r.cval = cval;
     if (BITS == 8) {
         const uint32_t tt = static_cast<uint32_t>(r.t > 255 ? 255 : r.t);
@@ -741,6 +792,8 @@ __device__ __forceinline__ Rep load_rep(const RepShared &s) {
     r.hiv = s.hiv;
     r.lov = s.lov;
     r.active = s.active != 0u;
+    r.sig2 = s.sig2;
+    r.moff = s.moff;
     return r;
 }
 
@@ -797,20 +850,19 @@ __device__ __forceinline__ uint32_t rep8_word(uint32_t w, const Rep8 &k, uint32_
     return (w & ~f) | (rep & f);
 }
 
-// Two 12-bit samples (int16 halves of w, in range): returns the output word and sets fm to the
-// flag bits (bit 15 / bit 31). With u = x + 2048 (12 bits) per half and bounds lo = M + 2048 - t,
+// Two 12-bit samples (int16 halves of w, in range): returns the output word and sets m to 0xFFFF in
+// flagged halves. With u = x + 2048 (12 bits) per half and bounds lo = M + 2048 - t,
 // hi = M + 2048 + t: x is flagged iff u >= hi or u <= lo (Eq. 2 with |x - M| >= t). Per half,
 // (u | 0x8000) - hi has bit 15 set iff u >= hi, and (0x8000 + lo) - u iff u <= lo; no borrow
 // crosses the halves because every operand is below 2^13. A flag moved down to bit 0 / 16 and
 // multiplied by 0xFFFF gives the half's select mask.
 template <int MODE>
 __device__ __forceinline__ uint32_t rep12_word(uint32_t w, uint32_t hi2, uint32_t lo2x, uint32_t c2, uint32_t h2,
-                                               uint32_t l2, uint32_t &fm) {
+                                               uint32_t l2, uint32_t &m) {
     const uint32_t u = (w ^ 0x08000800u) & 0x0FFF0FFFu;
     const uint32_t up = (u | 0x80008000u) - hi2;   // bit 15 / 31: u >= hi
     const uint32_t dn = lo2x - u;                   // bit 15 / 31: u <= lo
-    fm = (up | dn) & 0x80008000u;
-    const uint32_t m = (fm >> 15) * 0xFFFFu;  // 0xFFFF in a flagged half
+    m = (((up | dn) & 0x80008000u) >> 15) * 0xFFFFu;
     uint32_t z = 0u;
     if (MODE == 1) z = c2;
     if (MODE == 2) {
@@ -818,6 +870,13 @@ __device__ __forceinline__ uint32_t rep12_word(uint32_t w, uint32_t hi2, uint32_
         z = (h2 & ma) | (l2 & ~ma);
     }
     return (w & ~m) | (z & m);
+}
+
+// Mask bits of a chunk of eight 12-bit samples from its four flag words (0x0000/0xFFFF halves): one
+// byte of each flag, then the signed byte dot product of chunk_bits.
+__device__ __forceinline__ uint32_t chunk_bits12(uint32_t f0, uint32_t f1, uint32_t f2, uint32_t f3) {
+    return static_cast<uint32_t>(__dp4a(static_cast<int>(prmt(f2, f3, 0x6420u)), static_cast<int>(0x80C0E0F0u),
+                                        __dp4a(static_cast<int>(prmt(f0, f1, 0x6420u)), static_cast<int>(0xF8FCFEFFu), 0)));
 }
 
 // Mask bits of a 16-sample chunk from its four flag words (0x00/0xFF bytes), sample j -> bit j.
@@ -926,6 +985,7 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
     }
     const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
     const uint32_t excl = inc - cnt;
+    const NoiseRun<BITS, K> run = w.template noise<BITS>(p);
     for (uint32_t q0 = 0; q0 < total; q0 += 32) {
         const uint32_t q = q0 + lane;
         // owner: the last lane whose first index is <= q (lanes without flags share the next
@@ -941,7 +1001,7 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
         const int sL = __shfl_sync(0xFFFFFFFFu, s0, L);
         if (q < total) {
             const int pos = sL + nth_set_bit(bL, static_cast<int>(q - eL));
-            const int32_t z = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pos);
+            const int32_t z = run.value(static_cast<uint32_t>(pos), r.sig2, r.moff);
             store_sample<BITS, OUTF>(w.out, pos, z);
             if (PW) pw.z += static_cast<uint32_t>(z * z);
         }
@@ -971,7 +1031,12 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
     if (base + total <= static_cast<uint32_t>(kNoiseList)) {
         uint32_t off = base + inc - cnt;
-        for (uint32_t m = bits; m; m &= m - 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 + __ffs(m) - 1);
+        // one predicated store per sample of the chunk: with a quarter of the samples flagged in
+        // bursts some lane has all eight, and a loop over the set bits costs more per step (with the
+        // noise words shared over a tile, 60 streams of 2^25 samples in 8192-sample windows: 4.54 -> 4.27 ms)
+#pragma unroll
+        for (int j = 0; j < Geo<BITS>::kChunkSamples; ++j)
+            if ((bits >> j) & 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 + j);
         return;
     }
     for (uint32_t i = base + lane; i < static_cast<uint32_t>(kNoiseList); i += 32) sm.nlist[i] = kNoiseSkip;
@@ -986,29 +1051,30 @@ __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Re
                                            uint32_t *nlc, Pow &pw) {
     if (sm.nlist == nullptr) return;
     const uint32_t n = min(*nlc, static_cast<uint32_t>(kNoiseList));
+    const NoiseRun<BITS, K> run = w.template noise<BITS>(p);
     uint32_t i = static_cast<uint32_t>(tid);
     // two entries at a time: the two Philox chains are independent, so their rounds interleave
     // and fill each other's dependency stalls (60 streams of 2^25 12-bit samples in 8192-sample
     // windows, a quarter of them flagged: 4.60 -> 4.53 ms per call)
     for (; i + T < n; i += 2 * T) {
         const uint32_t pa = sm.nlist[i], pb = sm.nlist[i + T];
-        const int32_t za = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pa);
-        const int32_t zb = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pb);
+        const int2 z = run.value2(pa, pb, r.sig2, r.moff);
         if (pa != kNoiseSkip) {
-            store_sample<BITS, OUTF>(w.out, pa, za);
-            if (PW) pw.z += static_cast<uint32_t>(za * za);
+            store_sample<BITS, OUTF>(w.out, pa, z.x);
+            if (PW) pw.z += static_cast<uint32_t>(z.x * z.x);
         }
         if (pb != kNoiseSkip) {
-            store_sample<BITS, OUTF>(w.out, pb, zb);
-            if (PW) pw.z += static_cast<uint32_t>(zb * zb);
+            store_sample<BITS, OUTF>(w.out, pb, z.y);
+            if (PW) pw.z += static_cast<uint32_t>(z.y * z.y);
         }
     }
-    for (; i < n; i += T) {
+    if (i < n) {
         const uint32_t pos = sm.nlist[i];
-        if (pos == kNoiseSkip) continue;
-        const int32_t z = noise_value<BITS>(r.M, r.D, p, w.sid, w.abs_idx + pos);
-        store_sample<BITS, OUTF>(w.out, pos, z);
-        if (PW) pw.z += static_cast<uint32_t>(z * z);
+        if (pos != kNoiseSkip) {
+            const int32_t z = run.value(pos, r.sig2, r.moff);
+            store_sample<BITS, OUTF>(w.out, pos, z);
+            if (PW) pw.z += static_cast<uint32_t>(z * z);
+        }
     }
 }
 
@@ -1074,10 +1140,11 @@ template <int T, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_deferred8(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
                                                 const uint32_t *nlc, Pow &pw) {
     named_bar(sm.bar_id, T);  // every entry of the window is in the list
+    const NoiseRun<8, K> run = w.template noise<8>(p);
     noise_expand8<T>(sm, *nlc, tid, [&](uint32_t at) {
         const uint32_t pos = at - static_cast<uint32_t>(w.off);
         if (pos >= static_cast<uint32_t>(w.n)) return;
-        const int32_t z = noise_value<8>(r.M, r.D, p, w.sid, w.abs_idx + pos);
+        const int32_t z = run.value(pos, r.sig2, r.moff);
         store_sample<8, OUTF>(w.out, static_cast<int>(pos), z);
         if (PW) pw.z += static_cast<uint32_t>(z * z);
     });
@@ -1201,10 +1268,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
 #pragma unroll
                         for (int q = 0; q < 4; ++q) ww[q] = rep12_word<MODE>(ww[q], k12.mb4, k12.tlo7, k12.c4, k12.hi4,
                                                                              k12.lo4, f[q]);
-                        // flag bits 15 / 31 of the four words -> bits 0..7 (sample order)
-                        const uint32_t g0 = __byte_perm(f[0], f[1], 0x7531u) & 0x80808080u;
-                        const uint32_t g1 = __byte_perm(f[2], f[3], 0x7531u) & 0x80808080u;
-                        bits = ((g0 * 0x00204081u) >> 28) | (((g1 * 0x00204081u) >> 28) << 4);
+                        bits = chunk_bits12(f[0], f[1], f[2], f[3]);
                         // samples past the window (a ragged last chunk) are neither flagged nor stored
                         if (valid < 8) bits &= (1u << valid) - 1u;
                     }
@@ -1290,9 +1354,7 @@ __device__ __forceinline__ uint32_t replace_round_any(const Win &w, const Rep &r
                 const RepShared &k = *rsrc;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) ww[q] = rep12_word<MODE>(ww[q], k.mb4, k.tlo7, k.c4, k.hi4, k.lo4, f[q]);
-                const uint32_t g0 = __byte_perm(f[0], f[1], 0x7531u) & 0x80808080u;
-                const uint32_t g1 = __byte_perm(f[2], f[3], 0x7531u) & 0x80808080u;
-                bits = ((g0 * 0x00204081u) >> 28) | (((g1 * 0x00204081u) >> 28) << 4);
+                bits = chunk_bits12(f[0], f[1], f[2], f[3]);
             }
             bits &= (1u << hi) - (1u << lo);
         }
@@ -1544,7 +1606,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
 template <int RMODE, int T>
 __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg, uint32_t w0, int nw, int lw,
                               const RepShared *reps, uint32_t *cnt, const Params &p, int tid, int par,
-                              uint32_t release_bar) {
+                              uint32_t release_bar, const TileNoise &tn) {
     constexpr int NW = T / 32;
     const int lane = tid & 31, warp = tid >> 5;
     const int lcw = lw - 4;  // log2 of the chunks per window
@@ -1578,11 +1640,10 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
     if (RMODE == 3) {
         named_bar(sm.bar_id, T);  // every entry of the tile is in the list
         const KeysPre key{p};
-        const int64_t abs0 = sg.abs0 + (static_cast<int64_t>(w0) << lw);
+        const NoiseRun<8, KeysPre> run(key, sg.stream_id, static_cast<uint64_t>(sg.abs0 + (static_cast<int64_t>(w0) << lw)), tn);
         noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t pos) {
             const RepShared &rk = reps[pos >> lw];
-            const int32_t z = noise_value<8>(rk.M, rk.D, key, sg.stream_id, abs0 + pos);
-            out[pos] = static_cast<uint8_t>(z);
+            out[pos] = static_cast<uint8_t>(run.value(pos, rk.sig2, rk.moff));
         });
     }
 
@@ -1616,7 +1677,7 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
 template <int MODE, int T>
 __device__ bool process_tile_apply8(const Shm &sm, const uint8_t *stage, const Tile &tl, const Seg &sg,
                                     const int2 *amd, const Params &p, int tid, int par, int lw,
-                                    uint32_t release_bar, bool stage_ok) {
+                                    uint32_t release_bar, bool stage_ok, const TileNoise &tn) {
     const int nw = static_cast<int>(tl.nw);
     // every thread has finished the previous tile or window (its thresholds, counts, noise
     // work area) before this barrier
@@ -1624,7 +1685,7 @@ __device__ bool process_tile_apply8(const Shm &sm, const uint8_t *stage, const T
     RepShared *reps = sm.at->rep;
     if (tid < nw) reps[tid] = make_rep<8>(amd[tid].x, amd[tid].y, p.kq, p.cval);
     named_bar(sm.bar_id, T);
-    replace_tile8<MODE & 3, T>(sm, stage, sg, tl.w0, nw, lw, reps, sm.at->count, p, tid, par, release_bar);
+    replace_tile8<MODE & 3, T>(sm, stage, sg, tl.w0, nw, lw, reps, sm.at->count, p, tid, par, release_bar, tn);
     return true;
 }
 
@@ -1731,7 +1792,8 @@ __device__ __forceinline__ void scan_search8(uint16_t *cum, int n, int lane, int
 // windows) releases the stage: after the histogram for kModeStats, else after the replace pass.
 template <int MODE, int T, int K>
 __device__ bool process_tile_multi8(const Shm &sm, const uint8_t *stage, const Seg &sg, uint32_t w0, int nw, int lw,
-                                    const Params &p, int tid, int par, uint32_t release_bar, bool stage_ok) {
+                                    const Params &p, int tid, int par, uint32_t release_bar, bool stage_ok,
+                                    const TileNoise &tn) {
     constexpr bool STATS = (MODE & kModeStats) != 0;
     constexpr int NW = T / 32;
     const int lane = tid & 31, warp = tid >> 5;
@@ -1752,7 +1814,7 @@ __device__ bool process_tile_multi8(const Shm &sm, const uint8_t *stage, const S
     }
     if (STATS) return true;
     named_bar(sm.bar_id, T);
-    replace_tile8<MODE & 3, T>(sm, stage, sg, w0, nw, lw, sm.mt->rep, sm.mt->count, p, tid, par, release_bar);
+    replace_tile8<MODE & 3, T>(sm, stage, sg, w0, nw, lw, sm.mt->rep, sm.mt->count, p, tid, par, release_bar, tn);
     return true;
 }
 
@@ -1764,7 +1826,7 @@ __device__ bool process_tile_multi8(const Shm &sm, const uint8_t *stage, const S
 // samples has at most 514 chunks).
 template <int MODE, int T, int K>
 __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, const Seg &sg, uint32_t w0, int nw,
-                                  const Params &p, int tid, int par, uint32_t release_bar) {
+                                  const Params &p, int tid, int par, uint32_t release_bar, const TileNoise &tn) {
     constexpr bool STATS = (MODE & kModeStats) != 0;
     constexpr int RMODE = MODE & 3;
     constexpr int NW = T / 32, LPS = 32 / K, TS = T / K;
@@ -1786,6 +1848,7 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
         w.mask_words = sg.mask_words;
         w.abs_idx = sg.abs0 + k * W;
         w.sid = sg.stream_id;
+        w.tn = &tn;
         w.vec = ((reinterpret_cast<uintptr_t>(w.out) - w.off) & 15u) == 0u;
         return w;
     };
@@ -1827,10 +1890,12 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
         if (RMODE == 3) {
             named_bar(sm.bar_id, T);  // every entry of the windows is in the list
             const KeysPre key{p};
+            uint8_t *const out = sg.out + static_cast<int64_t>(w0) * W;
+            const NoiseRun<8, KeysPre> run(key, sg.stream_id, static_cast<uint64_t>(sg.abs0 + static_cast<int64_t>(w0) * W), tn);
             noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t at) {
                 const int g = static_cast<int>(at >> 14);
-                const int64_t i = (static_cast<int64_t>(w0) + g) * W + static_cast<int>(at & 16383u) - ((off + g * W) & 15);
-                sg.out[i] = static_cast<uint8_t>(noise_value<8>(reps[g].M, reps[g].D, key, sg.stream_id, sg.abs0 + i));
+                const uint32_t pos = static_cast<uint32_t>(g * W + static_cast<int>(at & 16383u) - ((off + g * W) & 15));
+                out[pos] = static_cast<uint8_t>(run.value(pos, reps[g].sig2, reps[g].moff));
             });
         }
         if (lane == 0) {

@@ -91,33 +91,24 @@ __global__ void __launch_bounds__(kFillThreads) noise_fill_kernel(const Seg *__r
         }
         __syncwarp();
         const int lg = (mw & (mw - 1u)) == 0u ? __ffs(static_cast<int>(mw)) - 1 : -1;  // log2 mw, or -1
-        const NoiseKey nk(key, g.stream_id, static_cast<uint32_t>(static_cast<uint64_t>(g.abs0) >> 32));
-        const bool one_hi = ((static_cast<uint64_t>(g.abs0) ^ static_cast<uint64_t>(g.abs0 + g.len - 1)) >> 32) == 0;
-        const uint64_t abs0 = static_cast<uint64_t>(g.abs0);
+        const NoiseRun<BITS, KeysPre> run(key, g.stream_id, static_cast<uint64_t>(g.abs0), static_cast<uint64_t>(g.len));
         uint8_t *const out = g.out;
         auto emit = [&](uint32_t code) {
             const uint4 e = a.win[code >> 5];
             const uint32_t pos = e.x + (code & 31u);
-            uint32_t sum;
-            if (one_hi) {
-                sum = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pos);
-            } else {
-                const uint64_t idx = abs0 + pos;
-                sum = noise_sum(NoiseKey(key, g.stream_id, static_cast<uint32_t>(idx >> 32)), key, static_cast<uint32_t>(idx));
-            }
-            fill_store<BITS>(out, pos, NoiseScale<BITS>::value(sum, static_cast<int32_t>(e.y), static_cast<int32_t>(e.z)));
+            fill_store<BITS>(out, pos, run.value(pos, static_cast<int32_t>(e.y), static_cast<int32_t>(e.z)));
         };
         // two entries of a lane at a time: their Philox chains are independent and interleave
         auto emit2 = [&](uint32_t c0, uint32_t c1) {
-            if (!one_hi) {
+            if (!run.one_hi) {
                 emit(c0);
                 emit(c1);
                 return;
             }
             const uint4 e0 = a.win[c0 >> 5], e1 = a.win[c1 >> 5];
             const uint32_t p0 = e0.x + (c0 & 31u), p1 = e1.x + (c1 & 31u);
-            const uint32_t s0 = noise_sum(nk, key, static_cast<uint32_t>(abs0) + p0);
-            const uint32_t s1 = noise_sum(nk, key, static_cast<uint32_t>(abs0) + p1);
+            const uint32_t lo = static_cast<uint32_t>(run.abs0);
+            const uint32_t s0 = noise_sum(run.nk, key, lo + p0), s1 = noise_sum(run.nk, key, lo + p1);
             fill_store<BITS>(out, p0, NoiseScale<BITS>::value(s0, static_cast<int32_t>(e0.y), static_cast<int32_t>(e0.z)));
             fill_store<BITS>(out, p1, NoiseScale<BITS>::value(s1, static_cast<int32_t>(e1.y), static_cast<int32_t>(e1.z)));
         };

@@ -114,7 +114,7 @@ struct Seg {
     int32_t vec;          // in/out 16-byte aligned and W * bytes_per_sample % 16 == 0
     uint64_t *power;      // detected power of window 0: {sum x^2, sum z^2} (nullable)
     uint32_t nwords;      // mask words of the run (set for the digital-noise pass)
-    uint32_t pad;
+    int32_t tidx;         // not of the table: a stage descriptor's tile index
 };
 
 // Work-list entry of the persistent kernel: windows [w0, w0 + nw) of segment seg.

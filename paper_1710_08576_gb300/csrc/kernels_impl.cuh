@@ -19,10 +19,10 @@ __host__ __device__ constexpr int align_up(int v, int a) { return (v + a - 1) / 
 // Per-stage descriptor written by the copy warp: the tile, its segment and the tile index.
 struct StageMeta {
     Tile tile;
-    Seg seg;
-    int32_t tidx;   // tile index, -1: no more tiles
-    int32_t pad[3];
+    Seg seg;        // seg.tidx: tile index, -1: no more tiles
+    TileNoise tn;   // digital noise
 };
+static_assert(sizeof(StageMeta) == 128, "no padding");
 
 // Split-warp form: a window handed from the histogram warps to the replace warps. Slot j is
 // filled by histogram warp 0 (lane 0) after waiting for its empty mbarrier, announced through its
@@ -141,6 +141,7 @@ __device__ __forceinline__ Win make_win(const Seg &sg, int64_t w, const uint8_t 
     win.sid = sg.stream_id;
     win.vec = sg.vec != 0;
     win.off = 0;
+    win.tn = nullptr;
     return win;
 }
 
@@ -203,7 +204,7 @@ __device__ bool split_consumers(const Shm &sm, uint8_t *gb, const Layout &L, Sta
                 tmo = true;
                 break;
             }
-            if (meta[s].tidx < 0) break;  // the end of the work list, seen alike by every thread
+            if (meta[s].seg.tidx < 0) break;  // the end of the work list, seen alike by every thread
             const Tile tl = meta[s].tile;
             const Seg &sg = meta[s].seg;
             uint8_t *stage = stage0 + s * stage_bytes;
@@ -370,6 +371,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
         constexpr int kLaneMad = 4 + offsetof(Seg, mad) / 4, kLaneW = 4 + offsetof(Seg, W) / 4;
         constexpr int kLaneVec = 4 + offsetof(Seg, vec) / 4;
         [[maybe_unused]] constexpr int kLaneLen = 4 + offsetof(Seg, len) / 4;
+        [[maybe_unused]] constexpr int kLaneAbs = 4 + offsetof(Seg, abs0) / 4, kLaneSid = 4 + offsetof(Seg, stream_id) / 4;
         const uint32_t *tile_w = reinterpret_cast<const uint32_t *>(tiles);
         const uint32_t *seg_w = reinterpret_cast<const uint32_t *>(segs);
         auto grab = [&](int i) -> int {  // lane 0: the group's tile of iteration i
@@ -419,7 +421,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
             issued = it + 1;
             if (t >= ntiles) {
                 if (lane == 0) {
-                    meta[s].tidx = -1;
+                    meta[s].seg.tidx = -1;
                     mbar_arrive(full_bar(s));
                 }
                 break;
@@ -432,6 +434,13 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
             uint32_t *md = reinterpret_cast<uint32_t *>(&meta[s]);
             if (lane < 28) md[lane] = dw;
             uint8_t *stage = stage0 + s * stage_bytes;
+            if constexpr ((MODE & 3) == 3 && (MODE & (kModeStats | kModeCopies)) == 0) {
+                // the tile's noise words (every lane computes them, one stores them)
+                const uint64_t a0 = ptr(dw, kLaneAbs) + static_cast<uint64_t>(w0) * static_cast<uint64_t>(W);
+                const uint64_t a1 = a0 + tbytes / BPS - 1;
+                const NoiseKey nk(KeysPre{p}, __shfl_sync(kAll, dw, kLaneSid), static_cast<uint32_t>(a0 >> 32));
+                if (lane == 0) meta[s].tn = TileNoise{nk, ((a0 ^ a1) >> 32) == 0u ? 1u : 0u};
+            }
             if (MODE & kModeApply) {
                 // the centre and dispersion of the tile's windows ride along with the stage
                 const int32_t *med = reinterpret_cast<const int32_t *>(ptr(dw, kLaneMed));
@@ -460,7 +469,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                 if (bulk == 0u ? a < hi : (lane < 16 ? a < b0 : a < hi)) at[a] = *reinterpret_cast<const uint8_t *>(a);
                 __syncwarp();
                 if (lane == 0) {
-                    meta[s].tidx = t;
+                    meta[s].seg.tidx = t;
                     mbar_arrive_tx(full_bar(s), bulk);
                     if (bulk) bulk_g2s(smem_addr(stage) + static_cast<uint32_t>(b0 - (lo & ~15ull)),
                                        reinterpret_cast<const void *>(b0), bulk, full_bar(s));
@@ -470,7 +479,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                 if (vec && static_cast<uint32_t>(lane) < rem) stage[bulk + lane] = src[bulk + lane];
                 __syncwarp();
                 if (lane == 0) {
-                    meta[s].tidx = t;
+                    meta[s].seg.tidx = t;
                     mbar_arrive_tx(full_bar(s), bulk);
                     if (bulk) bulk_g2s(smem_addr(stage), src, bulk, full_bar(s));
                 }
@@ -517,7 +526,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
         // after the wait is always a bar.red.or, so a thread that timed out and the others
         // agree on leaving.
         const bool ok = mbar_wait_bounded(full_bar(s), u & 1, kWaitTimeoutNs);
-        const int t = ok ? meta[s].tidx : -2;
+        const int t = ok ? meta[s].seg.tidx : -2;
         if (t < 0) {  // end of the work list (-1, seen alike by every thread) or a timeout (-2)
             timed_out = named_bar_or(sm.bar_id, T, t == -2);
             break;
@@ -541,7 +550,7 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                 tl.bytes == tl.nw * W) {
                 const int2 *amd = reinterpret_cast<const int2 *>(gb + L.amd) + s * kApplyTileWindows;
                 alive = process_tile_apply8<MODE, T>(sm, stage, tl, sg, amd, p, tid, par, 31 - __clz(static_cast<int>(W)),
-                                                     empty_bar(s), true);
+                                                     empty_bar(s), true, meta[s].tn);
                 par ^= 1;
                 if (!alive) {
                     timed_out = true;
@@ -568,10 +577,10 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                     const uint32_t rel = k0 + K >= tl.nw ? empty_bar(s) : 0u;
                     if (K == 8u)
                         alive = process_tile_multi8<MODE & ~kModeMulti, T, 8>(sm, stage + (k0 << lw), sg, tl.w0 + k0,
-                                                                              nwk, lw, p, tid, par, rel, true);
+                                                                              nwk, lw, p, tid, par, rel, true, meta[s].tn);
                     else
                         alive = process_tile_multi8<MODE & ~kModeMulti, T, 4>(sm, stage + (k0 << lw), sg, tl.w0 + k0,
-                                                                              nwk, lw, p, tid, par, rel, true);
+                                                                              nwk, lw, p, tid, par, rel, true, meta[s].tn);
                     par ^= 1;
                 }
                 rs = {{0u, 0u}};  // the reduce left the table zero
@@ -603,10 +612,10 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
                     const int at = toff + static_cast<int>(k0) * sg.W;
                     if (K == 8u)
                         alive = process_tile_any8<MODE & ~kModeAny, T, 8>(sm, stage + (at & ~15), at & 15, sg, tl.w0 + k0, nwk, p,
-                                                                          tid, par, rel);
+                                                                          tid, par, rel, meta[s].tn);
                     else
                         alive = process_tile_any8<MODE & ~kModeAny, T, 4>(sm, stage + (at & ~15), at & 15, sg, tl.w0 + k0, nwk, p,
-                                                                          tid, par, rel);
+                                                                          tid, par, rel, meta[s].tn);
                     par ^= 1;
                 }
                 rs = {{0u, 0u}};  // the reduce left the table zero
@@ -620,8 +629,9 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
         }
         for (uint32_t k = 0; k < tl.nw && alive; ++k) {
             const int64_t widx = static_cast<int64_t>(tl.w0) + k;
-            const Win win = (MODE & kModeAny) ? make_win_any(sg, widx, tl.w0, stage, toff, BPS)
+            Win win = (MODE & kModeAny) ? make_win_any(sg, widx, tl.w0, stage, toff, BPS)
                                               : make_win(sg, widx, stage + k * sg.W * BPS, (MODE & (kModeF16 | kModeBF16)) ? 2 : BPS);
+            win.tn = &meta[s].tn;
             const int2 *amd = ((MODE & kModeApply) && tl.nw <= kApplyTileWindows)
                                   ? reinterpret_cast<const int2 *>(gb + L.amd) + s * kApplyTileWindows + k
                                   : nullptr;

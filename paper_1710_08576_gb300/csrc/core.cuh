@@ -268,25 +268,24 @@ struct NoiseRun {
     // the words as the tile's copy warp left them (TileNoise)
     __device__ __forceinline__ NoiseRun(const K &k, uint32_t stream, uint64_t a0, const TileNoise &t)
         : key(k), nk(t.nk), abs0(a0), sid(stream), one_hi(t.one_hi != 0u) {}
+    // one_hi runs; a branch to the general form here costs 2 % of a call, so the loops below have a
+    // general twin instead
     __device__ __forceinline__ uint32_t sum(uint32_t pos) const {
-        if (one_hi) return noise_sum(nk, key, static_cast<uint32_t>(abs0) + pos);
-        const uint64_t idx = abs0 + pos;
-        return noise_sum(NoiseKey(key, sid, static_cast<uint32_t>(idx >> 32)), key, static_cast<uint32_t>(idx));
+        return noise_sum(nk, key, static_cast<uint32_t>(abs0) + pos);
     }
     __device__ __forceinline__ int32_t value(uint32_t pos, int32_t sig2, int32_t moff) const {
         return NoiseScale<BITS>::value(sum(pos), sig2, moff);
     }
     // two samples at a time: their Philox chains are independent and interleave
     __device__ __forceinline__ int2 value2(uint32_t pa, uint32_t pb, int32_t sig2, int32_t moff) const {
-        uint32_t a, b;
-        if (one_hi) {
-            a = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pa);
-            b = noise_sum(nk, key, static_cast<uint32_t>(abs0) + pb);
-        } else {
-            a = sum(pa);
-            b = sum(pb);
-        }
+        const uint32_t a = sum(pa), b = sum(pb);
         return make_int2(NoiseScale<BITS>::value(a, sig2, moff), NoiseScale<BITS>::value(b, sig2, moff));
+    }
+    // any run
+    __device__ __forceinline__ int32_t value_any(uint32_t pos, int32_t sig2, int32_t moff) const {
+        const uint64_t idx = abs0 + pos;
+        return NoiseScale<BITS>::value(
+            noise_sum(NoiseKey(key, sid, static_cast<uint32_t>(idx >> 32)), key, static_cast<uint32_t>(idx)), sig2, moff);
     }
 };
 
@@ -298,18 +297,13 @@ struct Geo {
     static constexpr int kBps = BITS == 8 ? 1 : 2;          // bytes per sample
     static constexpr int kLo = BITS == 8 ? -128 : -2048;
     static constexpr int kHi = BITS == 8 ? 127 : 2047;
-    // cumulative counts, laid out against bank conflicts: 8-bit padded, b + b/32; 12-bit
-    // swizzled in place: within each row of 16 bins the 16-byte group q sits at q ^ (row/2 mod 4),
-    // so that both a warp's consecutive 16-byte writes and its threads' reads of their own rows
-    // touch 8 distinct bank groups per 8 lanes
+    // 8-bit: cumulative counts, padded (pad32); 12-bit: the histogram's second table
     static constexpr int kCumWords = BITS == 8 ? kBins + kBins / 32 : kBins;
-    __host__ __device__ static constexpr int cum_index(int b) {
-        return BITS == 8 ? b + (b >> 5) : (b & ~15) | ((((b >> 2) ^ (b >> 5)) & 3) << 2) | (b & 3);
-    }
     static constexpr int kChunkSamples = 16 / kBps;          // samples per 16-byte chunk
     // 8-bit, one consumer group: a 32 KiB table of 128-byte rows (raw byte u -> row u, lane l
     // -> word l). 8-bit, two groups: one 64 KiB table of 256-byte rows shared by both (group g
-    // owns bytes [128g, 128g + 128) of every row). 12-bit: ncopies tables of 4096 words per group.
+    // owns bytes [128g, 128g + 128) of every row). 12-bit: ncopies tables of 4096 words per group
+    // (copy 0 of the even windows, then the other copies).
     __host__ __device__ static constexpr int hist_bytes(int ncopies, int groups) {
         return BITS == 8 ? (groups == 2 ? 65536 : 32768) : kBins * 4 * ncopies * groups;
     }
@@ -337,7 +331,7 @@ struct __align__(16) RepShared {
 struct CopyShared {
     RepShared vrep[kMaxCopies];        // threshold and replacement values per variant
     uint32_t vcount[kMaxCopies][2];    // flagged samples, by variant and window parity
-    uint32_t ncount[2 * kMaxCopies];   // 12-bit digital-noise list entries, by variant and parity
+    uint32_t ncount[4 * kMaxCopies];   // digital-noise list entries, by variant, parity and slice
 };
 
 // Apply passes over whole tiles: the thresholds and flag counts of the tile's windows.
@@ -363,7 +357,7 @@ struct Ctl {
     uint32_t count[2];   // flagged samples, by window parity
     uint32_t done[2];    // warps finished with the window, by window parity
     uint32_t err[2];     // 12-bit range error seen in the window, by window parity
-    uint32_t ncount[2];  // 12-bit digital-noise list entries, by window parity
+    uint32_t ncount[4];  // digital-noise list entries, by window parity (and slice of the window, 12-bit)
     unsigned long long pw[2][2];  // power-metered excision: {sum x^2, sum z^2}, by window parity
     uint32_t abort;      // set when any warp gave up on a bounded wait
     int32_t mb;          // median bin of the current window (written by its owner thread)
@@ -381,14 +375,15 @@ struct Shm {
     uint8_t *hist;       // histogram (generic pointer; 8-bit: the 64 KiB table)
     uint32_t hist_s;     // histogram (shared address)
     uint32_t grp;        // 8-bit: byte offset of this group's half row (0 or 128)
-    uint32_t *cum;       // padded cumulative counts
+    uint32_t *cum;       // padded cumulative counts; 12-bit: the histogram's second table (table12)
+    uint32_t *coarse;    // 12-bit estimation pass: the rows' cumulative counts (or null: see rows12)
     Ctl *ctl;
     int ncopies;         // 12-bit only
     int bar_id;          // named barrier of this consumer group
     CopyShared *cp;      // digital copy: per-variant state (or null)
     uint16_t *nlist;     // digital noise work area (or null): int8, the entries of the chunks that
                          // hold flagged samples (32-bit); 12-bit, the positions of flagged samples
-    uint32_t *nring;     // int8 digital noise: kNoiseRing positions per consumer warp (or null)
+    uint32_t *nring;     // int8 digital noise: noise_ring(mode) positions per consumer warp (or null)
     ApplyTile *at;       // apply passes: the current tile's thresholds and counts (or null)
     struct MultiTile *mt;  // 8-bit, one group: state of a multi-window tile (or null)
 };
@@ -398,9 +393,16 @@ struct Shm {
 // the per-warp path.
 constexpr int kNoiseList = 4096;
 constexpr uint16_t kNoiseSkip = 0xFFFFu;
-// Positions a warp's ring holds: fewer than 32 wait between two batches, and one expansion step
-// adds at most 32.
-constexpr int kNoiseRing = 64;
+// 12-bit digital noise goes through a window in slices of this many chunks (8192 samples; in the
+// any-window form 33 rounds of 31 chunks), so that the list serves slices with up to half their samples
+// flagged whatever the window's length.
+constexpr int kNoiseSlice = 1024, kNoiseSliceAny = 1023;
+// Positions a warp's ring holds: fewer than a batch wait between two batches (64 positions where a lane
+// takes two at a time, else 32), and one expansion step adds at most 32. Two at a time: the plain
+// kernel and the output formats; in the kernels with multi-window tiles or several variants the
+// registers it takes cost more than the overlap gives.
+__host__ __device__ constexpr bool noise_pairs(int mode) { return (mode & (kModeMulti | kModeAny | kModeApply | kModeCopies | kModePower)) == 0; }
+__host__ __device__ constexpr int noise_ring(int mode) { return noise_pairs(mode) ? 128 : 64; }
 
 // Per-thread sums of x^2 and z^2 of the power-metered excision. A thread sees at most
 // 65536 / 128 samples of a window, each below 2^22, so 32 bits hold its sums.
@@ -462,6 +464,16 @@ __device__ __forceinline__ void hist8_word(uint32_t lp, uint32_t w) {
     }
 }
 
+// 12-bit histogram tables: copy 0 has one for the even and one for the odd windows, so that a window's
+// table can be cleared while the next one's is in use; the other copies are folded into copy 0 and
+// cleared before the next window.
+__device__ __forceinline__ uint32_t *table12(const Shm &sm, int par) {
+    return par ? sm.cum : reinterpret_cast<uint32_t *>(sm.hist);
+}
+__device__ __forceinline__ uint32_t copy12(const Shm &sm, int c, int par) {
+    return c == 0 ? smem_addr(table12(sm, par)) : sm.hist_s + static_cast<uint32_t>(c) * 16384u;
+}
+
 // Two 12-bit samples in int16 halves. The bin x + 2048 of an in-range sample is its low 12 bits
 // with bit 11 flipped; a half is in range iff its bits 15..11 are all equal, which the caller
 // accumulates as (w ^ (w << 1)) & 0xF000F000.
@@ -497,7 +509,7 @@ __device__ __forceinline__ void phase_histogram(const Shm &sm, const Win &w, int
             else red_add_shared(lb + (u << 7), 1u);
         }
     } else {
-        const uint32_t cb = sm.hist_s + static_cast<uint32_t>(lane & (sm.ncopies - 1)) * 16384u;
+        const uint32_t cb = copy12(sm, lane & (sm.ncopies - 1), par);
         uint32_t bad = 0;
         for (int c = tid; c < nfull; c += T) {
             const uint4 a = d4[c];
@@ -550,7 +562,7 @@ __device__ __forceinline__ void phase_histogram_any(const Shm &sm, const Win &w,
         hist_chunks<8>(w, tid, T, [&](uint32_t v) { hist8_word<128>(lb, v); },
                        [&](int at) { red_add_shared(lb + (static_cast<uint32_t>(w.data[at]) << 7), 1u); });
     } else {
-        const uint32_t cb = sm.hist_s + static_cast<uint32_t>(lane & (sm.ncopies - 1)) * 16384u;
+        const uint32_t cb = copy12(sm, lane & (sm.ncopies - 1), par);
         uint32_t bad = 0;
         hist_chunks<12>(w, tid, T,
                         [&](uint32_t v) {
@@ -567,22 +579,6 @@ __device__ __forceinline__ void phase_histogram_any(const Shm &sm, const Win &w,
 }
 
 // ------------------------------------------------------------------ phases 2-3: reduce + scan
-// Block exclusive offsets of per-thread totals `run` (named barrier inside).
-template <int T>
-__device__ __forceinline__ uint32_t block_offsets(const Shm &sm, uint32_t run, int tid) {
-    const int lane = tid & 31, warp = tid >> 5;
-    uint32_t inc = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    if (lane == 31) sm.ctl->warp_tot[warp] = inc;
-    named_bar(sm.bar_id, T);
-    const uint32_t pre = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sm.ctl->warp_tot[lane] : 0u);
-    return pre + inc - run;
-}
-
 // 8-bit estimation pass: each thread's bins' counts for this window (the differences of its
 // running row sums) into the cumulative-count array, for one warp to scan.
 template <int T, int ROWB>
@@ -610,8 +606,7 @@ __device__ __forceinline__ void phase_reduce8_counts(const Shm &sm, int tid, Row
 // One warp, after phase_reduce8_counts and a group barrier: the inclusive scan of the 256 counts
 // in place (8 consecutive bins per lane) and the median bin, the lowest whose cumulative count
 // reaches ceil(n/2), into the control block.
-__device__ __forceinline__ void phase_scan8_warp(const Shm &sm, int n, int lane) {
-    uint32_t *cum = sm.cum;
+__device__ __forceinline__ void phase_scan8_warp(const Shm &sm, uint32_t *cum, int n, int lane) {
     uint32_t c[8];
     uint32_t run = 0;
 #pragma unroll
@@ -639,58 +634,45 @@ __device__ __forceinline__ void phase_scan8_warp(const Shm &sm, int n, int lane)
     __syncwarp();
 }
 
-// 12-bit: fold the copies into padded totals (conflict-free strided pass), then scan
-// contiguous bins per thread.
+// 12-bit: the 4096 bins as 256 rows of 16. Each row's total goes into coarse (padded), for one warp
+// to scan as the 256 counts of an 8-bit window; the copies are folded into copy 0 on the way. The
+// table of the window before is cleared. coarse is the first kCoarse words of that table (its words
+// are zeroed by the search, search12) or, in the estimation pass, whose other warps go on to the
+// next window's histogram during the search, a region of its own. Eight lanes of a row's
+// 16-byte read touch all banks (the pieces are taken in an order rotated by row pairs).
+// A full scan of the 4096 bins, which this replaces, took the group two more passes over the
+// table, a block-wide offset exchange and a fourth barrier: about 1400 instructions of its warps per
+// window against 350 (60 streams of 2^22 samples in 2048-sample windows, threshold, 2 CTAs: 1024 -> 991 us;
+// with one histogram copy and 3 CTAs, for which there was no room in the old default: 651 us).
+constexpr int kCoarse = 264;
 template <int T>
-__device__ __forceinline__ void phase_reduce_scan12(const Shm &sm, int tid, int n) {
-    constexpr int B = 4096;
-    constexpr int BPT = B / T;  // consecutive bins per thread in the scan
-    static_assert(BPT % 4 == 0, "whole 16-byte groups of bins per thread");
-    uint4 *h4 = reinterpret_cast<uint4 *>(sm.hist);
-    uint32_t *cum = sm.cum;
+__device__ __forceinline__ void phase_rows12(const Shm &sm, int tid, int par, uint32_t *coarse) {
+    uint32_t *const old = table12(sm, par ^ 1);
+    for (int i4 = tid + (coarse == old ? kCoarse / 4 : 0); i4 < 1024; i4 += T)
+        reinterpret_cast<uint4 *>(old)[i4] = make_uint4(0u, 0u, 0u, 0u);
     const int nc = sm.ncopies;
-    // fold the copies (and clear them) four bins at a time, coalesced
-    for (int i4 = tid; i4 < B / 4; i4 += T) {
-        uint4 s = h4[i4];
-        h4[i4] = make_uint4(0u, 0u, 0u, 0u);
-        for (int c = 1; c < nc; ++c) {
-            const uint4 a = h4[c * (B / 4) + i4];
-            h4[c * (B / 4) + i4] = make_uint4(0u, 0u, 0u, 0u);
-            s.x += a.x;
-            s.y += a.y;
-            s.z += a.z;
-            s.w += a.w;
+    for (int r = tid; r < 256; r += T) {
+        uint4 *const row = reinterpret_cast<uint4 *>(table12(sm, par)) + 4 * r;
+        const int rot = (r >> 1) & 3;
+        uint32_t s = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint4 v = row[q ^ rot];
+            if (nc > 1) {
+                for (int c = 1; c < nc; ++c) {
+                    uint4 *const o = reinterpret_cast<uint4 *>(sm.hist + c * 16384) + 4 * r + (q ^ rot);
+                    const uint4 a = *o;
+                    *o = make_uint4(0u, 0u, 0u, 0u);
+                    v.x += a.x;
+                    v.y += a.y;
+                    v.z += a.z;
+                    v.w += a.w;
+                }
+                row[q ^ rot] = v;
+            }
+            s += v.x + v.y + v.z + v.w;
         }
-        *reinterpret_cast<uint4 *>(cum + Geo<12>::cum_index(4 * i4)) = s;
-    }
-    named_bar(sm.bar_id, T);
-    uint32_t v[BPT];
-    uint32_t run = 0;
-#pragma unroll
-    for (int q = 0; q < BPT / 4; ++q) {
-        const uint4 a = *reinterpret_cast<const uint4 *>(cum + Geo<12>::cum_index(tid * BPT + 4 * q));
-        run += a.x;
-        v[4 * q] = run;
-        run += a.y;
-        v[4 * q + 1] = run;
-        run += a.z;
-        v[4 * q + 2] = run;
-        run += a.w;
-        v[4 * q + 3] = run;
-    }
-    const uint32_t excl = block_offsets<T>(sm, run, tid);
-    const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
-    uint32_t prev = excl;
-#pragma unroll
-    for (int q = 0; q < BPT / 4; ++q) {
-        uint32_t c[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            c[k] = v[4 * q + k] + excl;
-            if (c[k] >= half && prev < half) sm.ctl->mb = tid * BPT + 4 * q + k;
-            prev = c[k];
-        }
-        *reinterpret_cast<uint4 *>(cum + Geo<12>::cum_index(tid * BPT + 4 * q)) = make_uint4(c[0], c[1], c[2], c[3]);
+        coarse[pad32(r)] = s;
     }
 }
 
@@ -768,19 +750,62 @@ __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, 
 
 // One warp: lower median bin, then the MAD, then the threshold and replacement values, written
 // to the shared control block.
-template <int BITS>
-__device__ __forceinline__ void phase_search(const Shm &sm, int n, int lane, int64_t kq, int32_t cval) {
-    constexpr int B = Geo<BITS>::kBins;
+__device__ __forceinline__ void phase_search8(const Shm &sm, int n, int lane, int64_t kq, int32_t cval) {
+    constexpr int B = Geo<8>::kBins;
     const uint32_t *cum = sm.cum;
     const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
     const int mb = sm.ctl->mb;  // found by its owner thread during the scan
     const int d = warp_search<B>(lane, [&](int dd) {
         const int hi = mb + dd < B - 1 ? mb + dd : B - 1;
         const int lo = mb - dd - 1;
-        const uint32_t f = cum[Geo<BITS>::cum_index(hi)] - (lo >= 0 ? cum[Geo<BITS>::cum_index(lo)] : 0u);
+        const uint32_t f = cum[pad32(hi)] - (lo >= 0 ? cum[pad32(lo)] : 0u);
         return f >= half;
     });
-    if (lane == 0) sm.ctl->rep = make_rep<BITS>(mb - Geo<BITS>::kOffset, d, kq, cval);
+    if (lane == 0) sm.ctl->rep = make_rep<8>(mb - Geo<8>::kOffset, d, kq, cval);
+}
+
+// One warp, 12-bit: after phase_rows12 and a group barrier, the scan of the rows' totals (cc), the
+// median M in its row R, then the MAD. With F(d) the samples within d of M:
+//  - the smallest s for which the rows R - s .. R + s hold half the window puts D into 16(s - 1) + 1 ..
+//    16 s + 15 (those rows lie within 16 s + 15 of M and hold everything within 16 s of it),
+//  - F(16(s - 1)) comes from the rows' cumulative counts and parts of two rows,
+//  - lane j adds the bins at distance 16(s - 1) + 1 + j on either side, and a prefix sum gives the first
+//    distance that reaches half the window.
+__device__ __forceinline__ void phase_search12(const Shm &sm, const uint32_t *tab, uint32_t *cc, bool zero_cc, int n,
+                                               int lane, int64_t kq, int32_t cval) {
+    const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
+    auto prefix = [&](uint32_t v) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, v, o);
+            if (lane >= o) v += y;
+        }
+        return v;
+    };
+    auto upto = [&](int r) { return r >= 0 ? cc[pad32(r)] : 0u; };  // samples in rows 0 .. r
+    phase_scan8_warp(sm, cc, n, lane);
+    const int R = sm.ctl->mb;
+    const uint32_t in_row = prefix(lane < 16 ? tab[16 * R + lane] : 0u);
+    const int M = 16 * R + __ffs(__ballot_sync(0xFFFFFFFFu, upto(R - 1) + in_row >= half)) - 1;
+    const int s = warp_search<256>(lane, [&](int x) { return upto(min(R + x, 255)) - upto(R - x - 1) >= half; });
+    const int d0 = 16 * (s - 1);
+    uint32_t base = 0u;  // F(d0)
+    if (s > 0) {
+        const int b1 = min(M + d0, 4095), b2 = M - d0 - 1;
+        const int b = lane < 16 ? b1 : b2;
+        const uint32_t v = b >= 0 && (lane & 15) <= (b & 15) ? tab[(b & ~15) + (lane & 15)] : 0u;
+        base = upto((b1 >> 4) - 1) - (b2 >= 0 ? upto((b2 >> 4) - 1) : 0u) + __reduce_add_sync(0xFFFFFFFFu, lane < 16 ? v : 0u - v);
+    }
+    const int d = d0 + 1 + lane;
+    uint32_t add = 0u;
+    if (d >= 0 && M + d <= 4095) add = tab[M + d];
+    if (d > 0 && M - d >= 0) add += tab[M - d];
+    const int D = d0 + __ffs(__ballot_sync(0xFFFFFFFFu, base + prefix(add) >= half));
+    if (lane == 0) sm.ctl->rep = make_rep<12>(M - Geo<12>::kOffset, D, kq, cval);
+    if (zero_cc) {
+        __syncwarp();
+        for (int i = lane; i < kCoarse / 4; i += 32) reinterpret_cast<uint4 *>(cc)[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 __device__ __forceinline__ Rep load_rep(const RepShared &s) {
@@ -1001,21 +1026,21 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
         const int sL = __shfl_sync(0xFFFFFFFFu, s0, L);
         if (q < total) {
             const int pos = sL + nth_set_bit(bL, static_cast<int>(q - eL));
-            const int32_t z = run.value(static_cast<uint32_t>(pos), r.sig2, r.moff);
+            const int32_t z = run.value_any(static_cast<uint32_t>(pos), r.sig2, r.moff);
             store_sample<BITS, OUTF>(w.out, pos, z);
             if (PW) pw.z += static_cast<uint32_t>(z * z);
         }
     }
 }
 
-// Digital noise, replace pass: the warp numbers its flagged samples of this round, reserves that
-// many list entries with one shared atomic, and each lane writes its positions. Windows of
-// 65536 samples (position 65535 would equal the skip mark) and rounds that do not fit in the
-// list take the per-warp path at once; list entries reserved beyond the written ones are
-// marked skipped. Called by all lanes of the warp with the flags of samples s0, s0 + 1, ...
+// Digital noise, replace pass (12-bit): the warp numbers its flagged samples of this round, reserves
+// that many list entries with one shared atomic, and each lane writes its positions, counted from
+// the slice's first sample. Rounds that do not fit in the list take the per-warp path at once;
+// list entries reserved beyond the written ones are marked skipped. Called by all lanes of the warp
+// with the flags of samples s0, s0 + 1, ...
 template <int BITS, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const Rep &r, const K &p, int lane,
-                                             int s0, uint32_t bits, uint32_t *nlc, Pow &pw) {
+                                             int s0, int slice0, uint32_t bits, uint32_t *nlc, Pow &pw) {
     if (!__any_sync(0xFFFFFFFFu, bits != 0u)) return;
     const uint32_t cnt = __popc(bits);
     uint32_t inc = cnt;
@@ -1025,9 +1050,8 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
         if (lane >= o) inc += y;
     }
     const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
-    const bool listed = sm.nlist != nullptr && w.n < 65536;
     uint32_t base = kNoiseList;
-    if (listed && lane == 31) base = atomicAdd(nlc, total);
+    if (sm.nlist != nullptr && lane == 31) base = atomicAdd(nlc, total);
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
     if (base + total <= static_cast<uint32_t>(kNoiseList)) {
         uint32_t off = base + inc - cnt;
@@ -1036,7 +1060,7 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
         // noise words shared over a tile, 60 streams of 2^25 samples in 8192-sample windows: 4.54 -> 4.27 ms)
 #pragma unroll
         for (int j = 0; j < Geo<BITS>::kChunkSamples; ++j)
-            if ((bits >> j) & 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 + j);
+            if ((bits >> j) & 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 - slice0 + j);
         return;
     }
     for (uint32_t i = base + lane; i < static_cast<uint32_t>(kNoiseList); i += 32) sm.nlist[i] = kNoiseSkip;
@@ -1048,32 +1072,34 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
 // group evaluates Philox for a share of the list and stores the value over the chunk's output.
 template <int BITS, int T, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
-                                           uint32_t *nlc, Pow &pw) {
+                                           int slice0, const uint32_t *nlc, Pow &pw) {
     if (sm.nlist == nullptr) return;
     const uint32_t n = min(*nlc, static_cast<uint32_t>(kNoiseList));
     const NoiseRun<BITS, K> run = w.template noise<BITS>(p);
+    auto put = [&](uint32_t l, uint32_t pos, int32_t z) {
+        if (l == kNoiseSkip) return;
+        store_sample<BITS, OUTF>(w.out, static_cast<int>(pos), z);
+        if (PW) pw.z += static_cast<uint32_t>(z * z);
+    };
     uint32_t i = static_cast<uint32_t>(tid);
-    // two entries at a time: the two Philox chains are independent, so their rounds interleave
-    // and fill each other's dependency stalls (60 streams of 2^25 12-bit samples in 8192-sample
-    // windows, a quarter of them flagged: 4.60 -> 4.53 ms per call)
-    for (; i + T < n; i += 2 * T) {
-        const uint32_t pa = sm.nlist[i], pb = sm.nlist[i + T];
-        const int2 z = run.value2(pa, pb, r.sig2, r.moff);
-        if (pa != kNoiseSkip) {
-            store_sample<BITS, OUTF>(w.out, pa, z.x);
-            if (PW) pw.z += static_cast<uint32_t>(z.x * z.x);
+    if (run.one_hi) {
+        // two entries at a time: the two Philox chains are independent, so their rounds interleave
+        // and fill each other's dependency stalls (60 streams of 2^25 12-bit samples in 8192-sample
+        // windows, a quarter of them flagged: 4.60 -> 4.53 ms per call)
+        for (; i + T < n; i += 2 * T) {
+            const uint32_t la = sm.nlist[i], lb = sm.nlist[i + T];
+            const int2 z = run.value2(slice0 + la, slice0 + lb, r.sig2, r.moff);
+            put(la, slice0 + la, z.x);
+            put(lb, slice0 + lb, z.y);
         }
-        if (pb != kNoiseSkip) {
-            store_sample<BITS, OUTF>(w.out, pb, z.y);
-            if (PW) pw.z += static_cast<uint32_t>(z.y * z.y);
+        if (i < n) {
+            const uint32_t l = sm.nlist[i];
+            put(l, slice0 + l, run.value(slice0 + l, r.sig2, r.moff));
         }
-    }
-    if (i < n) {
-        const uint32_t pos = sm.nlist[i];
-        if (pos != kNoiseSkip) {
-            const int32_t z = run.value(pos, r.sig2, r.moff);
-            store_sample<BITS, OUTF>(w.out, pos, z);
-            if (PW) pw.z += static_cast<uint32_t>(z * z);
+    } else {  // a window across a multiple of 2^32
+        for (; i < n; i += T) {
+            const uint32_t l = sm.nlist[i];
+            if (l != kNoiseSkip) put(l, slice0 + l, run.value_any(slice0 + l, r.sig2, r.moff));
         }
     }
 }
@@ -1097,21 +1123,24 @@ __device__ __forceinline__ void noise_note8(const Shm &sm, int lane, int c, uint
 // noise_note8, in any order (a sample's noise depends only on its absolute index). Warp w
 // expands entries 2w and 2w + 1, then 2w + 2NW and 2w + 2NW + 1, and so on: each half-warp
 // takes one entry and its lane j tests flag bit j. The flagged positions go into the warp's
-// ring, compacted by a ballot and a prefix popcount, and whenever 32 are waiting every lane
-// takes one and emit(pos) evaluates and stores its noise. Fewer than 32 are left for the end.
-// Every lane does Philox work in every batch but the last, however the flags are spread over
-// the chunks, and the chunks are shared out evenly between the warps.
-template <int T, class Emit>
-__device__ __forceinline__ void noise_expand8(const Shm &sm, uint32_t n, int tid, Emit &&emit) {
-    constexpr uint32_t NW = T / 32;
-    constexpr uint32_t RM = kNoiseRing - 1;
+// ring, compacted by a ballot and a prefix popcount, and whenever 32 (PAIR: 64) are waiting every
+// lane takes one (two, whose Philox chains interleave) and emit evaluates and stores its noise.
+// Fewer are left for the end. Every lane does Philox work in every batch but the last, however
+// the flags are spread over the chunks, and the chunks are shared out evenly between the warps.
+// PAIR (60 streams of 2^22 samples, noise): 16384-sample windows 260 -> 257 us, 65536 385 -> 357,
+// fp16 output 281 -> 275.
+template <int T, bool PAIR, class Emit, class Emit2>
+__device__ __forceinline__ void noise_expand8(const Shm &sm, uint32_t n, int tid, Emit &&emit, Emit2 &&emit2) {
+    constexpr uint32_t NW = T / 32, B = PAIR ? 64 : 32, RING = 2 * B;
+    constexpr uint32_t RM = RING - 1;
     const int lane = tid & 31;
     const uint32_t warp = static_cast<uint32_t>(tid >> 5);
     const uint32_t *list = reinterpret_cast<const uint32_t *>(sm.nlist);
-    uint32_t *ring = sm.nring + warp * kNoiseRing;
+    uint32_t *ring = sm.nring + warp * RING;
     const uint32_t j = static_cast<uint32_t>(lane & 15);
     const uint32_t below = (1u << lane) - 1u;
-    uint32_t head = 0u, tail = 0u;  // positions taken / queued so far (tail - head < 32 between steps)
+    uint32_t head = 0u, tail = 0u;  // positions taken / queued so far (tail - head < B between steps)
+    auto at = [&](uint32_t i) { return ring[(head + i + static_cast<uint32_t>(lane)) & RM]; };
     for (uint32_t e0 = 2u * warp; e0 < n; e0 += 2u * NW) {
         const uint32_t e = e0 + static_cast<uint32_t>(lane >> 4);
         const uint32_t ent = e < n ? list[e] : 0u;
@@ -1119,35 +1148,67 @@ __device__ __forceinline__ void noise_expand8(const Shm &sm, uint32_t n, int tid
         const uint32_t bal = __ballot_sync(0xFFFFFFFFu, fl);
         if (fl) ring[(tail + static_cast<uint32_t>(__popc(bal & below))) & RM] = (ent >> 16) * 16u + j;
         tail += static_cast<uint32_t>(__popc(bal));
-        if (tail - head >= 32u) {
+        if (tail - head >= B) {
             __syncwarp();
-            const uint32_t pos = ring[(head + static_cast<uint32_t>(lane)) & RM];
-            __syncwarp();  // read before the next step refills the slot
-            head += 32u;
-            emit(pos);
+            if constexpr (PAIR) {
+                const uint32_t pa = at(0), pb = at(32);
+                __syncwarp();  // read before the next step refills the slots
+                head += B;
+                emit2(pa, pb);
+            } else {
+                const uint32_t pos = at(0);
+                __syncwarp();  // read before the next step refills the slot
+                head += B;
+                emit(pos);
+            }
         }
+    }
+    if (PAIR && tail - head > 32u) {
+        __syncwarp();
+        emit(at(0));
+        head += 32u;
     }
     if (tail != head) {
         __syncwarp();
-        if (static_cast<uint32_t>(lane) < tail - head) emit(ring[(head + static_cast<uint32_t>(lane)) & RM]);
+        if (static_cast<uint32_t>(lane) < tail - head) emit(at(0));
+    }
+}
+
+// The same for a run whose indices have two high words (a tile across a multiple of 2^32): one entry
+// per thread, its samples one after the other.
+template <int T, class Emit>
+__device__ __forceinline__ void noise_expand8_any(const Shm &sm, uint32_t n, int tid, Emit &&emit) {
+    for (uint32_t e = static_cast<uint32_t>(tid); e < n; e += T) {
+        const uint32_t ent = reinterpret_cast<const uint32_t *>(sm.nlist)[e];
+        for (uint32_t m = ent & 0xFFFFu; m; m &= m - 1u) emit((ent >> 16) * 16u + static_cast<uint32_t>(__ffs(m) - 1));
     }
 }
 
 // Digital noise (int8) of one window, after its replace pass noted its chunks in the list (*nlc
 // entries): one group barrier, then noise_expand8. Every store is checked against the window's
 // length.
-template <int T, bool PW, class K, int OUTF = 0>
+template <int T, bool PW, bool PAIR, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_deferred8(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
                                                 const uint32_t *nlc, Pow &pw) {
     named_bar(sm.bar_id, T);  // every entry of the window is in the list
     const NoiseRun<8, K> run = w.template noise<8>(p);
-    noise_expand8<T>(sm, *nlc, tid, [&](uint32_t at) {
-        const uint32_t pos = at - static_cast<uint32_t>(w.off);
+    auto put = [&](uint32_t pos, int32_t z) {
         if (pos >= static_cast<uint32_t>(w.n)) return;
-        const int32_t z = run.value(pos, r.sig2, r.moff);
         store_sample<8, OUTF>(w.out, static_cast<int>(pos), z);
         if (PW) pw.z += static_cast<uint32_t>(z * z);
-    });
+    };
+    const uint32_t off = static_cast<uint32_t>(w.off);
+    if (run.one_hi) {
+        noise_expand8<T, PAIR>(
+            sm, *nlc, tid, [&](uint32_t at) { put(at - off, run.value(at - off, r.sig2, r.moff)); },
+            [&](uint32_t a, uint32_t b) {
+                const int2 z = run.value2(a - off, b - off, r.sig2, r.moff);
+                put(a - off, z.x);
+                put(b - off, z.y);
+            });
+    } else {
+        noise_expand8_any<T>(sm, *nlc, tid, [&](uint32_t at) { put(at - off, run.value_any(at - off, r.sig2, r.moff)); });
+    }
 }
 
 // Sum of squares of the bytes of w kept by keep (0xFF per kept byte), as signed int8 samples.
@@ -1162,7 +1223,8 @@ __device__ __forceinline__ uint32_t sq4(uint32_t w, uint32_t keep) {
 // full rounds go two at a time.
 template <int BITS, int MODE, int T, bool PW, class K, int OUTF = 0, bool FO = false, bool PAIR = false>
 __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, const Rep &r, const K &p,
-                                                  int tid, uint32_t *nlc, Pow &pw, const RepShared *rsrc) {
+                                                  int tid, uint32_t *nlc, Pow &pw, const RepShared *rsrc,
+                                                  int slice = 0) {
     constexpr int BPS = Geo<BITS>::kBps;
     const int lane = tid & 31, warp = tid >> 5;
     const int nbytes = w.n * BPS;
@@ -1255,10 +1317,11 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
         uint8_t *mk = reinterpret_cast<uint8_t *>(w.mask);
         const int32_t t = r.t;
         const RepShared k12 = *rsrc;
-        for (int base = warp * 32; base < nchunks; base += T) {
+        const int cend = MODE == 3 ? min(nchunks, slice + kNoiseSlice) : nchunks;  // slice: its first chunk
+        for (int base = slice + warp * 32; base < cend; base += T) {
             const int c = base + lane;
             uint32_t bits = 0;
-            if (c < nchunks) {
+            if (c < cend) {
                 const uint4 v = d4[c];
                 uint32_t ww[4] = {v.x, v.y, v.z, v.w};
                 const int valid = c < nfull ? 8 : ((nbytes - c * 16) >> 1);  // samples in the window
@@ -1313,9 +1376,9 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
                 }
                 if (mk) mk[c] = static_cast<uint8_t>(bits);
             }
-            if (MODE == 3) noise_append<12, PW, K, OUTF>(sm, w, r, p, lane, c * 8, bits, nlc, pw);
+            if (MODE == 3) noise_append<12, PW, K, OUTF>(sm, w, r, p, lane, c * 8, slice * 8, bits, nlc, pw);
         }
-        if (mk) {
+        if (mk && cend == nchunks) {
             for (int c = nchunks + tid; c < 4 * w.mask_words; c += T) mk[c] = 0;
         }
     }
@@ -1395,28 +1458,48 @@ __device__ __forceinline__ void mask_padding(const Win &w, int i, int nt) {
 
 template <int BITS, int MODE, int T, class K>
 __device__ __forceinline__ uint32_t phase_replace_any(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
-                                                      uint32_t *nlc, Pow &pw, const RepShared *rsrc) {
+                                                      uint32_t *nlc, Pow &pw, const RepShared *rsrc, int slice = 0) {
     constexpr int BPS = Geo<BITS>::kBps, CS = Geo<BITS>::kChunkSamples;
     const int lane = tid & 31, warp = tid >> 5;
     const int nch = (w.off + w.n * BPS + 15) >> 4;
+    const int cend = BITS == 12 && MODE == 3 ? min(nch, slice + kNoiseSliceAny) : nch;
     uint32_t flagged = 0;
-    for (int base = warp * 31; base < nch; base += (T / 32) * 31) {
+    for (int base = slice + warp * 31; base < cend; base += (T / 32) * 31) {
         const uint32_t bits = replace_round_any<BITS, MODE>(w, r, rsrc, base, lane);
         flagged += __popc(bits);
         if (MODE == 3) {
             if (BITS == 8) noise_note8(sm, lane, base + lane, bits, nlc);
-            else noise_append<12, false, K>(sm, w, r, p, lane, (base + lane) * CS - w.off / BPS, bits, nlc, pw);
+            else noise_append<12, false, K>(sm, w, r, p, lane, (base + lane) * CS - w.off / BPS, slice * CS - w.off / BPS,
+                                             bits, nlc, pw);
         }
     }
-    mask_padding<BITS>(w, tid, T);
+    if (cend == nch) mask_padding<BITS>(w, tid, T);
     return flagged;
 }
 
+// 12-bit digital noise of one window, in slices: replace(counter, first chunk) lists a slice's flagged
+// samples and gives the thread's flag count, list(first sample, counter) evaluates them. nlc: two
+// counters, both zero on entry, used in turn; the one of the slice before is zeroed between the two
+// barriers around a slice's evaluation, when no thread reads it any more.
+template <int T, bool ANY, class Replace, class List>
+__device__ __forceinline__ uint32_t noise_slices12(const Shm &sm, const Win &w, uint32_t *nlc, int tid, Replace &&replace,
+                                                   List &&list) {
+    constexpr int STEP = ANY ? kNoiseSliceAny : kNoiseSlice;
+    const int nch = (w.off + 2 * w.n + 15) >> 4;
+    uint32_t f = 0;
+    for (int c = 0, k = 0;; c += STEP, k ^= 1) {
+        f += replace(nlc + k, c);
+        named_bar(sm.bar_id, T);  // every flagged position of the slice is in the list
+        if (c + STEP < nch && tid == 0) nlc[k ^ 1] = 0u;
+        list(c * 8 - w.off / 2, nlc + k);
+        if (c + STEP >= nch) return f;
+        named_bar(sm.bar_id, T);  // the list is free again
+    }
+}
+
 // ------------------------------------------------------------------ one window
-// All T threads of the group call this; the histogram must be zero on entry and is zero again
-// when the first warp leaves the reduce phase. Uses the group's named barrier three times
-// (after the histogram, inside the scan, after the cumulative counts) plus once after the
-// search. There is no barrier at the end: each warp adds its flag count and marks itself done,
+// All T threads of the group call this. The 12-bit tables must be zero at a group's first window.
+// Uses the group's named barrier after the histogram, after the reduce and after the search. There is no barrier at the end: each warp adds its flag count and marks itself done,
 // and the last warp of the window (window parity `par`) writes the count, median and MAD to
 // slot `widx` of the segment and, when release_bar != 0, releases the stage through it.
 // `stage_ok` is this thread's result of waiting for the stage (false: timed out); the first
@@ -1455,12 +1538,16 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         if (tid == 0 && release_bar) mbar_arrive(release_bar);
         // int8: the counts go to one warp, which scans them and searches while the other warps
         // start the next window (one group barrier fewer than a block-wide scan)
-        if (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
-        else phase_reduce_scan12<T>(sm, tid, w.n);
+        if constexpr (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
+        else phase_rows12<T>(sm, tid, par, sm.coarse);
         named_bar(sm.bar_id, T);
         if (tid < 32) {
-            if (BITS == 8) phase_scan8_warp(sm, w.n, lane);
-            phase_search<BITS>(sm, w.n, lane, p.kq, p.cval);
+            if constexpr (BITS == 8) {
+                phase_scan8_warp(sm, sm.cum, w.n, lane);
+                phase_search8(sm, w.n, lane, p.kq, p.cval);
+            } else {
+                phase_search12(sm, table12(sm, par), sm.coarse, false, w.n, lane, p.kq, p.cval);
+            }
             if (lane == 0) {  // the lane that wrote the record
                 if (med) med[widx] = sm.ctl->rep.M;
                 if (mad) mad[widx] = sm.ctl->rep.D;
@@ -1475,12 +1562,16 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             else phase_histogram<BITS, T, ROWB>(sm, w, tid, par);
         }
         if (named_bar_or(sm.bar_id, T, !stage_ok)) return false;
-        if (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
-        else phase_reduce_scan12<T>(sm, tid, w.n);
+        if constexpr (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
+        else phase_rows12<T>(sm, tid, par, table12(sm, par ^ 1));
         named_bar(sm.bar_id, T);
         if (tid < 32) {
-            if (BITS == 8) phase_scan8_warp(sm, w.n, lane);
-            phase_search<BITS>(sm, w.n, lane, p.kq, p.cval);
+            if constexpr (BITS == 8) {
+                phase_scan8_warp(sm, sm.cum, w.n, lane);
+                phase_search8(sm, w.n, lane, p.kq, p.cval);
+            } else {
+                phase_search12(sm, table12(sm, par), table12(sm, par ^ 1), true, w.n, lane, p.kq, p.cval);
+            }
         }
     } else {
         // every thread has read the previous window's values before this barrier
@@ -1495,17 +1586,21 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     uint32_t f = 0;
     Pow pw = {0u, 0u};
     const KeysPre key{p};
-    if constexpr (ANY && !STATS)
-        f = phase_replace_any<BITS, RMODE, T, KeysPre>(sm, w, r, key, tid, &sm.ctl->ncount[par], pw, &sm.ctl->rep);
-    else if (!STATS && !COPIES)
-        f = phase_replace<BITS, RMODE, T, PW, KeysPre, OUTF, (MODE & kModeFlaggedOnly) != 0>(
-            sm, w, r, key, tid, &sm.ctl->ncount[par], pw, &sm.ctl->rep);
-    if (!STATS && !COPIES && RMODE == 3) {
-        if (BITS == 8) {
-            noise_deferred8<T, PW, KeysPre, OUTF>(sm, w, r, key, tid, &sm.ctl->ncount[par], pw);
+    // the replace pass, and the digital noise of the samples it listed
+    auto replace = [&](uint32_t *nlc, int slice) {
+        if constexpr (ANY) return phase_replace_any<BITS, RMODE, T, KeysPre>(sm, w, r, key, tid, nlc, pw, &sm.ctl->rep, slice);
+        else return phase_replace<BITS, RMODE, T, PW, KeysPre, OUTF, (MODE & kModeFlaggedOnly) != 0>(sm, w, r, key, tid, nlc, pw,
+                                                                                                    &sm.ctl->rep, slice);
+    };
+    if constexpr (!STATS && !COPIES) {
+        uint32_t *const nlc = &sm.ctl->ncount[2 * par];
+        if constexpr (BITS == 12 && RMODE == 3) {
+            f = noise_slices12<T, ANY>(sm, w, nlc, tid, replace, [&](int slice0, const uint32_t *c) {
+                noise_list<12, T, PW, KeysPre, OUTF>(sm, w, r, key, tid, slice0, c, pw);
+            });
         } else {
-            named_bar(sm.bar_id, T);  // every flagged position of the window is in the list
-            noise_list<BITS, T, PW, KeysPre, OUTF>(sm, w, r, key, tid, &sm.ctl->ncount[par], pw);
+            f = replace(nlc, 0);
+            if constexpr (RMODE == 3) noise_deferred8<T, PW, noise_pairs(MODE), KeysPre, OUTF>(sm, w, r, key, tid, nlc, pw);
         }
     }
     if (COPIES) {
@@ -1524,19 +1619,23 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             wv.vec = sv.vec != 0;
             const Rep rv = load_rep(sm.cp->vrep[v]);
             const KeysSeed vkey{static_cast<uint32_t>(vr.seed), static_cast<uint32_t>(vr.seed >> 32)};
-            uint32_t *nc = &sm.cp->ncount[2 * v + par];
+            uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
             uint32_t fv;
             switch (vr.mode) {
                 case 0: fv = phase_replace<BITS, 0, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]); break;
                 case 1: fv = phase_replace<BITS, 1, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]); break;
                 case 2: fv = phase_replace<BITS, 2, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]); break;
                 default:
-                    fv = phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]);
-                    if (BITS == 8) {
-                        noise_deferred8<T, false>(sm, wv, rv, vkey, tid, nc, pw);
+                    if constexpr (BITS == 12) {
+                        fv = noise_slices12<T, false>(
+                            sm, wv, nc, tid,
+                            [&](uint32_t *c, int slice) {
+                                return phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, c, pw, &sm.cp->vrep[v], slice);
+                            },
+                            [&](int slice0, const uint32_t *c) { noise_list<BITS, T, false>(sm, wv, rv, vkey, tid, slice0, c, pw); });
                     } else {
-                        named_bar(sm.bar_id, T);
-                        noise_list<BITS, T, false>(sm, wv, rv, vkey, tid, nc, pw);
+                        fv = phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]);
+                        noise_deferred8<T, false, false>(sm, wv, rv, vkey, tid, nc, pw);
                     }
                     // the noise work area and the first indices are reused by the next variant
                     if (v + 1 < params_nvar(p)) named_bar(sm.bar_id, T);
@@ -1566,11 +1665,15 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             __threadfence_block();
             const uint32_t cnt = atomicExch(&sm.ctl->count[par], 0u);
             sm.ctl->done[par] = 0u;
-            if (RMODE == 3 && !COPIES) sm.ctl->ncount[par] = 0u;  // every warp has read it
+            if (RMODE == 3 && !COPIES) {  // every warp has read them
+                sm.ctl->ncount[2 * par] = 0u;
+                if (BITS == 12) sm.ctl->ncount[2 * par + 1] = 0u;
+            }
             if (COPIES) {
                 for (int v = 0; v < params_nvar(p); ++v) {
                     const uint32_t cv = atomicExch(&sm.cp->vcount[v][par], 0u);
-                    sm.cp->ncount[2 * v + par] = 0u;
+                    sm.cp->ncount[4 * v + 2 * par] = 0u;
+                    sm.cp->ncount[4 * v + 2 * par + 1] = 0u;
                     const Seg &sv = vsegs[static_cast<int64_t>(v) * params_seg_stride(p)];
                     if (sv.counts) sv.counts[widx] = cv;
                     sm.ctl->flagged += cv;
@@ -1632,7 +1735,7 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
         }
         store_chunk8<0>(out, c, v, true);
         if (mk) mk[c] = static_cast<uint16_t>(bits);
-        if (RMODE == 3) noise_note8(sm, lane, c, bits, &sm.ctl->ncount[par]);
+        if (RMODE == 3) noise_note8(sm, lane, c, bits, &sm.ctl->ncount[2 * par]);
         const uint32_t wf = __reduce_add_sync(0xFFFFFFFFu, __popc(bits));
         if (lane == 0 && wf) atomicAdd(&cnt[k], wf);
     }
@@ -1641,10 +1744,21 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
         named_bar(sm.bar_id, T);  // every entry of the tile is in the list
         const KeysPre key{p};
         const NoiseRun<8, KeysPre> run(key, sg.stream_id, static_cast<uint64_t>(sg.abs0 + (static_cast<int64_t>(w0) << lw)), tn);
-        noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t pos) {
-            const RepShared &rk = reps[pos >> lw];
-            out[pos] = static_cast<uint8_t>(run.value(pos, rk.sig2, rk.moff));
-        });
+        const uint32_t n = sm.ctl->ncount[2 * par];
+        if (run.one_hi) {
+            noise_expand8<T, false>(
+                sm, n, tid,
+                [&](uint32_t pos) {
+                    const RepShared &rk = reps[pos >> lw];
+                    out[pos] = static_cast<uint8_t>(run.value(pos, rk.sig2, rk.moff));
+                },
+                [](uint32_t, uint32_t) {});
+        } else {
+            noise_expand8_any<T>(sm, n, tid, [&](uint32_t pos) {
+                const RepShared &rk = reps[pos >> lw];
+                out[pos] = static_cast<uint8_t>(run.value_any(pos, rk.sig2, rk.moff));
+            });
+        }
     }
 
     if (lane == 0) {
@@ -1653,7 +1767,7 @@ __device__ void replace_tile8(const Shm &sm, const uint8_t *stage, const Seg &sg
             // last warp of the tile: every count is in and every read of the stage is done
             __threadfence_block();
             sm.ctl->done[par] = 0u;
-            if (RMODE == 3) sm.ctl->ncount[par] = 0u;  // every warp has read it
+            if (RMODE == 3) sm.ctl->ncount[2 * par] = 0u;  // every warp has read it
             unsigned long long tot = 0ull;
             for (int k = 0; k < nw; ++k) {
                 const uint32_t ck = cnt[k];
@@ -1882,7 +1996,7 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
             const int g = q / rpw, base = (q - g * rpw) * 31;
             const Win w = window(g);
             const uint32_t bits = replace_round_any<8, RMODE>(w, load_rep(reps[g]), &reps[g], base, lane);
-            if (RMODE == 3) noise_note8(sm, lane, (g << 10) + base + lane, bits, &sm.ctl->ncount[par]);
+            if (RMODE == 3) noise_note8(sm, lane, (g << 10) + base + lane, bits, &sm.ctl->ncount[2 * par]);
             const uint32_t wf = __reduce_add_sync(0xFFFFFFFFu, __popc(bits));
             if (lane == 0 && wf) atomicAdd(&sm.mt->count[g], wf);
             if (base == 0) mask_padding<8>(w, lane, 32);
@@ -1892,11 +2006,26 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
             const KeysPre key{p};
             uint8_t *const out = sg.out + static_cast<int64_t>(w0) * W;
             const NoiseRun<8, KeysPre> run(key, sg.stream_id, static_cast<uint64_t>(sg.abs0 + static_cast<int64_t>(w0) * W), tn);
-            noise_expand8<T>(sm, sm.ctl->ncount[par], tid, [&](uint32_t at) {
-                const int g = static_cast<int>(at >> 14);
-                const uint32_t pos = static_cast<uint32_t>(g * W + static_cast<int>(at & 16383u) - ((off + g * W) & 15));
-                out[pos] = static_cast<uint8_t>(run.value(pos, reps[g].sig2, reps[g].moff));
-            });
+            const uint32_t n = sm.ctl->ncount[2 * par];
+            auto where = [&](uint32_t at, int g) {  // entry position -> sample of the tile
+                return static_cast<uint32_t>(g * W + static_cast<int>(at & 16383u) - ((off + g * W) & 15));
+            };
+            if (run.one_hi) {
+                noise_expand8<T, false>(
+                    sm, n, tid,
+                    [&](uint32_t at) {
+                        const int g = static_cast<int>(at >> 14);
+                        const uint32_t pos = where(at, g);
+                        out[pos] = static_cast<uint8_t>(run.value(pos, reps[g].sig2, reps[g].moff));
+                    },
+                    [](uint32_t, uint32_t) {});
+            } else {
+                noise_expand8_any<T>(sm, n, tid, [&](uint32_t at) {
+                    const int g = static_cast<int>(at >> 14);
+                    const uint32_t pos = where(at, g);
+                    out[pos] = static_cast<uint8_t>(run.value_any(pos, reps[g].sig2, reps[g].moff));
+                });
+            }
         }
         if (lane == 0) {
             __threadfence_block();
@@ -1904,7 +2033,7 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
                 // last warp: every count is in and every read of the stage is done
                 __threadfence_block();
                 sm.ctl->done[par] = 0u;
-                if (RMODE == 3) sm.ctl->ncount[par] = 0u;  // every warp has read it
+                if (RMODE == 3) sm.ctl->ncount[2 * par] = 0u;  // every warp has read it
                 unsigned long long tot = 0ull;
                 for (int g = 0; g < nw; ++g) {
                     const uint32_t cg = sm.mt->count[g];

@@ -96,7 +96,8 @@ __global__ void __launch_bounds__(kFillThreads) noise_fill_kernel(const Seg *__r
         auto emit = [&](uint32_t code) {
             const uint4 e = a.win[code >> 5];
             const uint32_t pos = e.x + (code & 31u);
-            fill_store<BITS>(out, pos, run.value(pos, static_cast<int32_t>(e.y), static_cast<int32_t>(e.z)));
+            const int32_t sig2 = static_cast<int32_t>(e.y), moff = static_cast<int32_t>(e.z);
+            fill_store<BITS>(out, pos, run.one_hi ? run.value(pos, sig2, moff) : run.value_any(pos, sig2, moff));
         };
         // two entries of a lane at a time: their Philox chains are independent and interleave
         auto emit2 = [&](uint32_t c0, uint32_t c1) {
@@ -107,8 +108,7 @@ __global__ void __launch_bounds__(kFillThreads) noise_fill_kernel(const Seg *__r
             }
             const uint4 e0 = a.win[c0 >> 5], e1 = a.win[c1 >> 5];
             const uint32_t p0 = e0.x + (c0 & 31u), p1 = e1.x + (c1 & 31u);
-            const uint32_t lo = static_cast<uint32_t>(run.abs0);
-            const uint32_t s0 = noise_sum(run.nk, key, lo + p0), s1 = noise_sum(run.nk, key, lo + p1);
+            const uint32_t s0 = run.sum(p0), s1 = run.sum(p1);
             fill_store<BITS>(out, p0, NoiseScale<BITS>::value(s0, static_cast<int32_t>(e0.y), static_cast<int32_t>(e0.z)));
             fill_store<BITS>(out, p1, NoiseScale<BITS>::value(s1, static_cast<int32_t>(e1.y), static_cast<int32_t>(e1.z)));
         };

@@ -188,6 +188,11 @@ size_t stream_smem_bytes(int bits, int mode, int consumer_warps, int ncopies, in
 // Maximum resident CTAs per SM of the persistent kernel for this shape (0 if it cannot run).
 int persistent_occupancy(int bits, int mode, const Shape &s);
 
+// 12-bit histogram copies where nothing asks for a number: more copies spread a warp's same-bin
+// atomics, but take 16 KiB each from the CTAs (60 streams of 2^22 samples, noise, 8192-sample windows: 618
+// us a call with 1, 3 CTAs per SM, 746 with 2, 1186 with 4; 65536-sample windows, one CTA: 960, 969, 998).
+constexpr int kDefaultHistCopies = 1;
+
 // Persistent batched kernel over a device work list. counter: one zeroed uint32 (dynamic tiles).
 cudaError_t launch_persistent(int bits, int mode, const Shape &s, int grid, const Seg *segs,
                               const Tile *tiles, int ntiles, const Params &p, unsigned *counter,

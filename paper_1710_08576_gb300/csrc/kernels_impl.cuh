@@ -41,8 +41,8 @@ struct __align__(16) SplitSlot {
 
 // Dynamic shared memory: the histogram at offset 0 (8-bit: one table for all groups; 12-bit:
 // per group; none for the apply passes of Eq. 3), then one block per consumer group
-// (cumulative counts, control block, mbarriers, stage descriptors), then the stage buffers of
-// every group.
+// (cumulative counts or the 12-bit histogram's second table, control block, mbarriers, stage
+// descriptors), then the stage buffers of every group.
 struct Layout {
     int grp;        // first group block
     int grp_size;   // bytes per group block
@@ -54,6 +54,7 @@ struct Layout {
     int cps;                  // digital copy: per-variant state inside a group block (0: none)
     int mt;                   // 8-bit plain excision and estimation: multi-window tile state (0: none)
     int split;                // split-warp form: the hand-over slots (0: none)
+    int coarse;               // 12-bit estimation pass: the rows' cumulative counts (0: none)
     int stage;      // first stage buffer; group g stage s at stage + (g * stages + s) * stage_bytes
     int total;
 };
@@ -77,13 +78,13 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     const bool noise = ((mode & 3) == 3 || (mode & kModeCopies) != 0) && (mode & kModeStats) == 0;
     L.nlist = noise ? meta_end : 0;
     // int8: a 32-bit entry for every 16-byte chunk of a stage that may hold a flagged sample,
-    // then each consumer warp's ring of kNoiseRing 32-bit positions (multi-window tiles keep the
+    // then each consumer warp's ring of noise_ring(mode) 32-bit positions (multi-window tiles keep the
     // rings in their cumulative-count area, which is idle by then and large enough); 12-bit: the
     // position list
     // (any-window tiles: a chunk that two windows share has an entry for each)
     const int list_bytes = align_up(stage_bytes / 4 > 128 ? stage_bytes / 4 : 128, 128) + ((mode & kModeAny) ? 128 : 0);
-    const int ring_bytes = multi ? 0 : cw * kNoiseRing * 4;
-    static_assert(kNoiseRing * 4 * 16 <= Geo<8>::kCumWords * 2 * kMultiMax, "rings of 16 warps fit the multi-window counts");
+    const int ring_bytes = multi ? 0 : cw * noise_ring(mode) * 4;
+    static_assert(noise_ring(kModeMulti) * 4 * 16 <= Geo<8>::kCumWords * 2 * kMultiMax, "rings of 16 warps fit the multi-window counts");
     const int noise_bytes = BITS == 8 ? list_bytes + ring_bytes : kNoiseList * 2;
     L.nring = (noise && BITS == 8) ? (multi ? L.cum : meta_end + list_bytes) : 0;
     const int list_end = noise ? align_up(meta_end + noise_bytes, 128) : meta_end;
@@ -96,6 +97,9 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     const int cps_end = copies ? align_up(amd_end + static_cast<int>(sizeof(CopyShared)), 128) : amd_end;
     L.mt = multi ? cps_end : 0;
     L.grp_size = multi ? align_up(cps_end + static_cast<int>(sizeof(MultiTile)), 128) : cps_end;
+    const bool coarse = BITS == 12 && (mode & kModeStats) != 0;
+    L.coarse = coarse ? L.grp_size : 0;
+    if (coarse) L.grp_size = align_up(L.grp_size + kCoarse * 4, 128);
     L.split = split ? L.grp_size : 0;
     if (split) L.grp_size = align_up(L.grp_size + kSplitSlots * static_cast<int>(sizeof(SplitSlot)), 128);
     L.stage = L.grp + groups * L.grp_size;
@@ -112,6 +116,7 @@ __device__ __forceinline__ Shm group_view(uint8_t *smem, const Layout &L, int g,
     sm.hist_s = smem_addr(sm.hist);
     sm.grp = BITS == 8 ? 128u * static_cast<uint32_t>(g) : 0u;
     sm.cum = reinterpret_cast<uint32_t *>(gb + L.cum);
+    sm.coarse = L.coarse ? reinterpret_cast<uint32_t *>(gb + L.coarse) : nullptr;
     sm.ctl = reinterpret_cast<Ctl *>(gb + L.ctl);
     sm.ncopies = ncopies;
     sm.bar_id = 1 + g;
@@ -226,12 +231,12 @@ __device__ bool split_consumers(const Shm &sm, uint8_t *gb, const Layout &L, Sta
                 phase_reduce8_counts<TH, 128>(sm, tid, rs);
                 named_bar(1, TH);
                 if (tid < 32) {
-                    phase_scan8_warp(sm, win.n, lane);
+                    phase_scan8_warp(sm, sm.cum, win.n, lane);
                     const int j = seq % kSplitSlots, use = seq / kSplitSlots;
                     int okj = 1;
                     if (use > 0 && lane == 0) okj = mbar_wait_bounded(slot_empty(j), (use - 1) & 1, kWaitTimeoutNs);
                     okj = __shfl_sync(0xFFFFFFFFu, okj, 0);
-                    phase_search<8>(sm, win.n, lane, p.kq, p.cval);
+                    phase_search8(sm, win.n, lane, p.kq, p.cval);
                     __syncwarp();
                     if (lane == 0) {
                         if (okj) {
@@ -291,7 +296,7 @@ __device__ bool split_consumers(const Shm &sm, uint8_t *gb, const Layout &L, Sta
             const Rep r = load_rep(sl.rep);
             Pow pw = {0u, 0u};
             uint32_t f = phase_replace<8, RMODE, TR, false, KeysPre, 0, (MODE & kModeFlaggedOnly) != 0, true>(
-                sr, win, r, key, rtid, &sm.ctl->ncount[par], pw, &sl.rep);
+                sr, win, r, key, rtid, &sm.ctl->ncount[2 * par], pw, &sl.rep);
             f = __reduce_add_sync(0xFFFFFFFFu, f);
             if (lane == 0) {
                 if (f) atomicAdd(&sm.ctl->count[par], f);

@@ -146,7 +146,7 @@ extern "C" rfi_status rfi_excise_noalloc(const rfi_plan_desc *d, const void *con
     Shape sh{};
     sh.consumer_warps = 8;
     sh.groups = 1;
-    sh.hist_copies = bps == 1 ? 1 : 2;
+    sh.hist_copies = kDefaultHistCopies;
     sh.dynamic_tiles = 1;
     const int min_stage = static_cast<int>((maxwb + 127) / 128 * 128);
     // work list: grow the stage (windows per tile) until the list fits the scratch area

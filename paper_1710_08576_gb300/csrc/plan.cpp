@@ -70,7 +70,7 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
     s.stage_bytes = std::max(min_stage, (req && req->stage_bytes) ? req->stage_bytes : (mom_stage ? 32768 : 16384));
     s.stage_bytes = (s.stage_bytes + 127) / 128 * 128;
     s.stages = (req && req->stages) ? req->stages : (mom_stage ? 1 : 2);
-    s.hist_copies = P->bits == 8 ? 1 : ((req && req->hist_copies) ? req->hist_copies : 2);
+    s.hist_copies = P->bits == 8 ? 1 : ((req && req->hist_copies) ? req->hist_copies : kDefaultHistCopies);
     s.dynamic_tiles = (req && req->dynamic_tiles) ? req->dynamic_tiles : (uniform ? 2 : 1);
     const int want_ctas = (req && req->ctas_per_sm) ? req->ctas_per_sm : 4;  // as many as fit, up to 4
     // the shape is sized for the kernel with the histogram (the MoM stats pass)

@@ -186,7 +186,7 @@ Params server_params(const rfi_server_s *s, DevCounters *ctr) {  // ctr: the ser
     p.kq = s->kq;
     p.seed = s->seed;
     p.cval = s->cval;
-    p.ncopies = s->bits == 8 ? 1 : 2;
+    p.ncopies = kDefaultHistCopies;
     p.status = &ctr->status;
     p.flagged = &ctr->flagged;
     set_round_keys(p);
@@ -560,7 +560,7 @@ rfi_status rfi_server_step(rfi_server_t s, int32_t *launched) {
     Shape sh{};
     sh.consumer_warps = 8;
     sh.groups = 1;
-    sh.hist_copies = s->bits == 8 ? 1 : 2;
+    sh.hist_copies = kDefaultHistCopies;
     sh.dynamic_tiles = 2;  // static round robin: no work-list cursor to reset between passes
     sh.stage_bytes = (max_wb + 127) / 128 * 128;
     sh.stages = 2;

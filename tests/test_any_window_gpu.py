@@ -122,3 +122,45 @@ def test_median_of_mad(cuda, rfi, bits, noise_pass):
                 assert np.array_equal(counts[i].cpu().numpy().view(np.uint32), r["counts"]), i
         finally:
             plan.close()
+
+
+@pytest.mark.parametrize("bits,W", [(8, 1000), (8, 12500), (12, 1000), (12, 12500)])
+def test_noise_of_windows_across_two_to_the_32(cuda, rfi, bits, W):
+    """A stream of 2^32 samples and some, all zero but the last 100000: the noise of a window (and, in
+    windows of 1000, of a tile of several) whose sample indices pass 2^32."""
+    import torch
+    n = (1 << 32) + 50_000
+    w0 = ((1 << 32) - 50_000) // W  # first window compared
+    x = torch.zeros(n, dtype=torch.int8 if bits == 8 else torch.int16, device="cuda")
+    tail = _streams(bits, [n - w0 * W], 12, 2e-2)[0]
+    x[w0 * W:] = torch.from_numpy(tail).cuda()
+    z = torch.empty_like(x)
+    plan = rfi.Plan(bits, [n], [W], 3.0, 3, 0, 99)
+    try:
+        plan.excise([x], [z])
+        assert plan.stats()[0] == 0
+    finally:
+        plan.close()
+    ref = oracle.excise(tail, W, 3.0, 3, seed=99, abs0=w0 * W, bits=bits)
+    assert np.array_equal(z[w0 * W:].cpu().numpy(), ref["z"])
+    assert not z[:w0 * W].any()
+
+
+@pytest.mark.parametrize("bits", [8, 12])
+def test_served_noise_across_two_to_the_32(cuda, rfi, bits):
+    """Aligned windows that pass 2^32 (a served stream may start there)."""
+    import torch
+    W, start = 10000, ((1 << 32) // 10000 - 1) * 10000
+    x = _streams(bits, [4 * W], 13, 2e-2)[0]
+    sv = rfi.Server(bits, [W], 8 * W, 3.0, 3, 0, 21, memory_budget=64 << 20, stream_start=[start])
+    try:
+        t = torch.from_numpy(x).cuda()
+        torch.cuda.synchronize()
+        assert sv.push(0, t)[0] == 0
+        sv.drain(10.0)
+        z = torch.zeros_like(t)
+        assert sv.read(0, start, x.size, z) == 0
+        ref = oracle.excise(x, W, 3.0, 3, seed=21, abs0=start, bits=bits)
+        assert np.array_equal(z.cpu().numpy(), ref["z"])
+    finally:
+        sv.close()

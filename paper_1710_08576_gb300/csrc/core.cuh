@@ -1198,7 +1198,12 @@ __device__ __forceinline__ void noise_deferred8(const Shm &sm, const Win &w, con
         if (PW) pw.z += static_cast<uint32_t>(z * z);
     };
     const uint32_t off = static_cast<uint32_t>(w.off);
-    if (run.one_hi) {
+    if constexpr (!std::is_same<K, KeysPre>::value) {
+        // a variant's own key: no tile words, and its window's flags are too few to pay for them
+        noise_expand8<T, false>(
+            sm, *nlc, tid, [&](uint32_t at) { put(at - off, run.value_any(at - off, r.sig2, r.moff)); },
+            [](uint32_t, uint32_t) {});
+    } else if (run.one_hi) {
         noise_expand8<T, PAIR>(
             sm, *nlc, tid, [&](uint32_t at) { put(at - off, run.value(at - off, r.sig2, r.moff)); },
             [&](uint32_t a, uint32_t b) {

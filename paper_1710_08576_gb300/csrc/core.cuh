@@ -343,8 +343,8 @@ struct ApplyTile {
 // Multi-window tiles (8-bit, one consumer group): up to K (4 or 8) small windows are
 // histogrammed at once, window slot g in lanes (32/K)g .. (32/K)(g+1)-1 of the lane-striped
 // table, so that one reduce, one set of barriers and parallel searches serve them all. Their
-// cumulative counts (at most 8192, the largest window of this form) are 16-bit: slot g's
-// kCumWords entries at (uint16_t *)cum + g * kCumWords.
+// cumulative counts (at most 8192, the largest window of this form) are 16-bit: slot g's 256
+// entries at (uint16_t *)cum + g * kCumWords.
 constexpr int kMultiMax = 8;
 struct MultiTile {
     RepShared rep[kMultiMax];
@@ -705,51 +705,67 @@ __device__ __forceinline__ int32_t sat_to(int64_t v, int32_t lo, int32_t hi) {
 }
 
 // Threshold and replacement values of a window with median M and dispersion D (Eq. 1; D is the
-// window's MAD, or the median of MADs of Eq. 3).
-template <int BITS>
+// window's MAD, or the median of MADs of Eq. 3): those that replacement mode MODE reads (kModeStats:
+// none but M and D; kModeCopies: none, the variants have records of their own; kRepAll: those of every
+// mode). One lane computes them between the search and the replace pass, while the window's other
+// threads wait (all values for every mode: 60 streams of 2^26 int8 samples, zero, 1.609 ms; now 1.592).
+constexpr int kRepAll = 1 << 20;
+template <int BITS, int MODE>
 __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, int32_t cval) {
     constexpr int SPAN = Geo<BITS>::kHi - Geo<BITS>::kLo;
-    RepShared r;
+    constexpr bool NONE = (MODE & (kModeStats | kModeCopies)) != 0;
+    constexpr int RMODE = MODE & 3;
+    constexpr bool ALL = (MODE & kRepAll) != 0;
+    RepShared r = {};
     r.M = M;
     r.D = d;
+    if constexpr (NONE) return r;
     const int64_t kd = kq * static_cast<int64_t>(d);
     const int64_t t = (kd + 65535) >> 16;
-    const int64_t c = kd >> 16;
     r.t = static_cast<int32_t>(t < SPAN + 1 ? t : SPAN + 1);
-    r.hiv = sat_to(static_cast<int64_t>(r.M) + c, Geo<BITS>::kLo, Geo<BITS>::kHi);
-    r.lov = sat_to(static_cast<int64_t>(r.M) - c, Geo<BITS>::kLo, Geo<BITS>::kHi);
     r.active = (d > 0 && t <= SPAN) ? 1u : 0u;  // |x - M| never exceeds the sample span
-    r.sig2 = NoiseScale<BITS>::kSig2 * d;
-    r.moff = M - NoiseScale<BITS>::kOff;
-    r.cval = cval;
-    if (BITS == 8) {
+    if constexpr (ALL || RMODE == 1) r.cval = cval;
+    if constexpr (ALL || RMODE == 2) {
+        const int64_t c = kd >> 16;
+        r.hiv = sat_to(static_cast<int64_t>(r.M) + c, Geo<BITS>::kLo, Geo<BITS>::kHi);
+        r.lov = sat_to(static_cast<int64_t>(r.M) - c, Geo<BITS>::kLo, Geo<BITS>::kHi);
+    }
+    if constexpr (ALL || RMODE == 3) {
+        r.sig2 = NoiseScale<BITS>::kSig2 * d;
+        r.moff = M - NoiseScale<BITS>::kOff;
+    }
+    if constexpr (BITS == 8) {
         const uint32_t tt = static_cast<uint32_t>(r.t > 255 ? 255 : r.t);
-        const uint32_t ub = static_cast<uint32_t>(r.M + 129);  // smallest biased value above M
         r.mb4 = static_cast<uint32_t>(r.M + 128) * 0x01010101u;
         r.tlo7 = (tt & 0x7Fu) * 0x01010101u;
         r.tsmall = tt < 128u ? ~0u : 0u;
-        r.c4 = (static_cast<uint32_t>(cval) & 0xFFu) * 0x01010101u;
-        r.hi4 = (static_cast<uint32_t>(r.hiv) & 0xFFu) * 0x01010101u;
-        r.lo4 = (static_cast<uint32_t>(r.lov) & 0xFFu) * 0x01010101u;
-        r.ulo7 = (ub & 0x7Fu) * 0x01010101u;
-        r.usmall = ub < 128u ? ~0u : 0u;
-        r.unone = ub > 255u ? 1u : 0u;
+        if constexpr (ALL || RMODE == 1) r.c4 = (static_cast<uint32_t>(cval) & 0xFFu) * 0x01010101u;
+        if constexpr (ALL || RMODE == 2) {
+            const uint32_t ub = static_cast<uint32_t>(r.M + 129);  // smallest biased value above M
+            r.hi4 = (static_cast<uint32_t>(r.hiv) & 0xFFu) * 0x01010101u;
+            r.lo4 = (static_cast<uint32_t>(r.lov) & 0xFFu) * 0x01010101u;
+            r.ulo7 = (ub & 0x7Fu) * 0x01010101u;
+            r.usmall = ub < 128u ? ~0u : 0u;
+            r.unone = ub > 255u ? 1u : 0u;
+        }
     } else {
         // 12-bit, two samples per word (see rep12_word): u = x + 2048 per 16-bit half
         const uint32_t mb = static_cast<uint32_t>(r.M + 2048);
         const uint32_t tt = static_cast<uint32_t>(r.t);  // <= 4096
         r.mb4 = (mb + tt) * 0x00010001u;                  // upper bound, u >= it flags
         r.tlo7 = (0x8000u + mb - tt) * 0x00010001u;       // 0x8000 + lower bound, u <= it flags
-        r.c4 = (static_cast<uint32_t>(cval) & 0xFFFFu) * 0x00010001u;
-        r.hi4 = (static_cast<uint32_t>(r.hiv) & 0xFFFFu) * 0x00010001u;
-        r.lo4 = (static_cast<uint32_t>(r.lov) & 0xFFFFu) * 0x00010001u;
-        r.tsmall = r.ulo7 = r.usmall = r.unone = 0u;
+        if constexpr (ALL || RMODE == 1) r.c4 = (static_cast<uint32_t>(cval) & 0xFFFFu) * 0x00010001u;
+        if constexpr (ALL || RMODE == 2) {
+            r.hi4 = (static_cast<uint32_t>(r.hiv) & 0xFFFFu) * 0x00010001u;
+            r.lo4 = (static_cast<uint32_t>(r.lov) & 0xFFFFu) * 0x00010001u;
+        }
     }
     return r;
 }
 
 // One warp: lower median bin, then the MAD, then the threshold and replacement values, written
 // to the shared control block.
+template <int MODE>
 __device__ __forceinline__ void phase_search8(const Shm &sm, int n, int lane, int64_t kq, int32_t cval) {
     constexpr int B = Geo<8>::kBins;
     const uint32_t *cum = sm.cum;
@@ -761,7 +777,7 @@ __device__ __forceinline__ void phase_search8(const Shm &sm, int n, int lane, in
         const uint32_t f = cum[pad32(hi)] - (lo >= 0 ? cum[pad32(lo)] : 0u);
         return f >= half;
     });
-    if (lane == 0) sm.ctl->rep = make_rep<8>(mb - Geo<8>::kOffset, d, kq, cval);
+    if (lane == 0) sm.ctl->rep = make_rep<8, MODE>(mb - Geo<8>::kOffset, d, kq, cval);
 }
 
 // One warp, 12-bit: after phase_rows12 and a group barrier, the scan of the rows' totals (cc), the
@@ -771,6 +787,7 @@ __device__ __forceinline__ void phase_search8(const Shm &sm, int n, int lane, in
 //  - F(16(s - 1)) comes from the rows' cumulative counts and parts of two rows,
 //  - lane j adds the bins at distance 16(s - 1) + 1 + j on either side, and a prefix sum gives the first
 //    distance that reaches half the window.
+template <int MODE>
 __device__ __forceinline__ void phase_search12(const Shm &sm, const uint32_t *tab, uint32_t *cc, bool zero_cc, int n,
                                                int lane, int64_t kq, int32_t cval) {
     const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
@@ -801,7 +818,7 @@ __device__ __forceinline__ void phase_search12(const Shm &sm, const uint32_t *ta
     if (d >= 0 && M + d <= 4095) add = tab[M + d];
     if (d > 0 && M - d >= 0) add += tab[M - d];
     const int D = d0 + __ffs(__ballot_sync(0xFFFFFFFFu, base + prefix(add) >= half));
-    if (lane == 0) sm.ctl->rep = make_rep<12>(M - Geo<12>::kOffset, D, kq, cval);
+    if (lane == 0) sm.ctl->rep = make_rep<12, MODE>(M - Geo<12>::kOffset, D, kq, cval);
     if (zero_cc) {
         __syncwarp();
         for (int i = lane; i < kCoarse / 4; i += 32) reinterpret_cast<uint4 *>(cc)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -1549,9 +1566,9 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         if (tid < 32) {
             if constexpr (BITS == 8) {
                 phase_scan8_warp(sm, sm.cum, w.n, lane);
-                phase_search8(sm, w.n, lane, p.kq, p.cval);
+                phase_search8<MODE>(sm, w.n, lane, p.kq, p.cval);
             } else {
-                phase_search12(sm, table12(sm, par), sm.coarse, false, w.n, lane, p.kq, p.cval);
+                phase_search12<MODE>(sm, table12(sm, par), sm.coarse, false, w.n, lane, p.kq, p.cval);
             }
             if (lane == 0) {  // the lane that wrote the record
                 if (med) med[widx] = sm.ctl->rep.M;
@@ -1573,9 +1590,9 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         if (tid < 32) {
             if constexpr (BITS == 8) {
                 phase_scan8_warp(sm, sm.cum, w.n, lane);
-                phase_search8(sm, w.n, lane, p.kq, p.cval);
+                phase_search8<MODE>(sm, w.n, lane, p.kq, p.cval);
             } else {
-                phase_search12(sm, table12(sm, par), table12(sm, par ^ 1), true, w.n, lane, p.kq, p.cval);
+                phase_search12<MODE>(sm, table12(sm, par), table12(sm, par ^ 1), true, w.n, lane, p.kq, p.cval);
             }
         }
     } else {
@@ -1583,7 +1600,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         if (named_bar_or(sm.bar_id, T, !stage_ok)) return false;
         if (tid == 0) {  // from the stage's copy (amd) when the copy warp brought it along
             const int2 md = amd ? *amd : make_int2(sg.med[widx], sg.mad[widx]);
-            sm.ctl->rep = make_rep<BITS>(md.x, md.y, p.kq, p.cval);
+            sm.ctl->rep = make_rep<BITS, MODE>(md.x, md.y, p.kq, p.cval);
         }
     }
     named_bar(sm.bar_id, T);
@@ -1612,7 +1629,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         // every variant's values from the window's M and D, then its replace pass
         if (tid < params_nvar(p)) {
             const Variant vr = params_var(p)[tid];
-            sm.cp->vrep[tid] = make_rep<BITS>(r.M, r.D, vr.kq, vr.cval);
+            sm.cp->vrep[tid] = make_rep<BITS, kRepAll>(r.M, r.D, vr.kq, vr.cval);
         }
         named_bar(sm.bar_id, T);
         for (int v = 0; v < params_nvar(p); ++v) {
@@ -1802,7 +1819,7 @@ __device__ bool process_tile_apply8(const Shm &sm, const uint8_t *stage, const T
     // work area) before this barrier
     if (named_bar_or(sm.bar_id, T, !stage_ok)) return false;
     RepShared *reps = sm.at->rep;
-    if (tid < nw) reps[tid] = make_rep<8>(amd[tid].x, amd[tid].y, p.kq, p.cval);
+    if (tid < nw) reps[tid] = make_rep<8, MODE>(amd[tid].x, amd[tid].y, p.kq, p.cval);
     named_bar(sm.bar_id, T);
     replace_tile8<MODE & 3, T>(sm, stage, sg, tl.w0, nw, lw, reps, sm.at->count, p, tid, par, release_bar, tn);
     return true;
@@ -1839,8 +1856,8 @@ __device__ __forceinline__ void hist8_multi(const Shm &sm, const uint8_t *stage,
 // byte u holds lane l's count at word l; a slot's lanes are 8/K of the row's eight 16-byte
 // groups). The eight threads tid & ~7 .. tid | 7 read the eight groups of the same row, so the
 // reads and clears are free of bank conflicts; with four slots, thread pairs combine their
-// groups by a shuffle. Counts go to 16-bit arrays, 264 entries per slot (slot g's array starts
-// on bank 4g, so the stores of one row's slots do not collide either).
+// groups by a shuffle. Counts go to 16-bit arrays, 264 entries apart (slot g's array starts
+// on bank 4g, so the stores of one row's slots do not collide either, and on a 16-byte boundary).
 template <int T, int K>
 __device__ __forceinline__ void reduce8_multi(const Shm &sm, int tid) {
     static_assert(K == 4 || K == 8, "four or eight window slots");
@@ -1857,22 +1874,28 @@ __device__ __forceinline__ void reduce8_multi(const Shm &sm, int tid) {
         *a = make_uint4(0u, 0u, 0u, 0u);
         uint32_t sum = v.x + v.y + v.z + v.w;
         if (K == 4) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
-        if (K == 8 || (p & 1) == 0) cumg[pad32(row ^ 128)] = static_cast<uint16_t>(sum);
+        if (K == 8 || (p & 1) == 0) cumg[row ^ 128] = static_cast<uint16_t>(sum);
     }
 }
 
-// One warp: the inclusive scan of a slot's 256 counts in place (8 consecutive bins per lane),
-// then its lower median bin and MAD (the searches of phase_scan8_warp and phase_search), and the
-// threshold and replacement values into *rep (lane 0). The counts and cumulative counts are
-// 16-bit (a window of this form has at most 8192 samples).
+// One warp: the inclusive scan of a slot's 256 counts in place (8 consecutive bins per lane, one
+// 16-byte load and store), then its lower median bin and MAD (the searches of phase_scan8_warp and
+// phase_search8), and the threshold and replacement values into *rep (lane 0). The counts and
+// cumulative counts are 16-bit (a window of this form has at most 8192 samples).
+template <int MODE>
 __device__ __forceinline__ void scan_search8(uint16_t *cum, int n, int lane, int64_t kq, int32_t cval,
                                              RepShared *rep) {
+    uint4 *const own = reinterpret_cast<uint4 *>(cum) + lane;
+    const uint4 h = *own;
+    const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
     uint32_t c[8];
     uint32_t run = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        run += cum[pad32(lane * 8 + j)];
-        c[j] = run;
+    for (int j = 0; j < 4; ++j) {
+        run += hw[j] & 0xFFFFu;
+        c[2 * j] = run;
+        run += hw[j] >> 16;
+        c[2 * j + 1] = run;
     }
     uint32_t inc = run;
 #pragma unroll
@@ -1882,24 +1905,23 @@ __device__ __forceinline__ void scan_search8(uint16_t *cum, int n, int lane, int
     }
     const uint32_t excl = inc - run;
     const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
-    int found = 0;
+    // bins whose cumulative count stays below half the window lie below the median bin
+    uint32_t below = 0u;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const uint32_t v = c[j] + excl;
-        const uint32_t before = (j ? c[j - 1] : 0u) + excl;
-        cum[pad32(lane * 8 + j)] = static_cast<uint16_t>(v);
-        if (v >= half && before < half) found = lane * 8 + j + 1;
+        c[j] += excl;
+        below += c[j] < half ? 1u : 0u;
     }
-    // the median bin is the one lane that found it; the others hold 0
-    const int mb = static_cast<int>(__reduce_max_sync(0xFFFFFFFFu, static_cast<uint32_t>(found))) - 1;
+    *own = make_uint4(c[0] | (c[1] << 16), c[2] | (c[3] << 16), c[4] | (c[5] << 16), c[6] | (c[7] << 16));
+    const int mb = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, below));
     __syncwarp();
     const int d = warp_search<256>(lane, [&](int dd) {
         const int hi = mb + dd < 255 ? mb + dd : 255;
         const int lo = mb - dd - 1;
-        const uint32_t f = static_cast<uint32_t>(cum[pad32(hi)]) - (lo >= 0 ? static_cast<uint32_t>(cum[pad32(lo)]) : 0u);
+        const uint32_t f = static_cast<uint32_t>(cum[hi]) - (lo >= 0 ? static_cast<uint32_t>(cum[lo]) : 0u);
         return f >= half;
     });
-    if (lane == 0) *rep = make_rep<8>(mb - Geo<8>::kOffset, d, kq, cval);
+    if (lane == 0) *rep = make_rep<8, MODE>(mb - Geo<8>::kOffset, d, kq, cval);
 }
 
 // A tile of nw (1 <= nw <= K) full int8 windows of 2^lw samples, 16-byte aligned, in shared
@@ -1924,7 +1946,7 @@ __device__ bool process_tile_multi8(const Shm &sm, const uint8_t *stage, const S
     named_bar(sm.bar_id, T);
     for (int g = warp; g < nw; g += NW) {
         RepShared *rep = &sm.mt->rep[g];
-        scan_search8(reinterpret_cast<uint16_t *>(sm.cum) + g * Geo<8>::kCumWords, 1 << lw, lane, p.kq, p.cval, rep);
+        scan_search8<MODE>(reinterpret_cast<uint16_t *>(sm.cum) + g * Geo<8>::kCumWords, 1 << lw, lane, p.kq, p.cval, rep);
         __syncwarp();
         if (lane == 0) {
             if (med) med[w0 + g] = rep->M;
@@ -1984,7 +2006,7 @@ __device__ bool process_tile_any8(const Shm &sm, const uint8_t *stage, int off, 
     for (int g = warp; g < nw; g += NW) {
         RepShared *rep = &sm.mt->rep[g];
         const int64_t lg = left - static_cast<int64_t>(g) * W;
-        scan_search8(reinterpret_cast<uint16_t *>(sm.cum) + g * Geo<8>::kCumWords, static_cast<int>(lg < W ? lg : W), lane,
+        scan_search8<MODE>(reinterpret_cast<uint16_t *>(sm.cum) + g * Geo<8>::kCumWords, static_cast<int>(lg < W ? lg : W), lane,
                      p.kq, p.cval, rep);
         __syncwarp();
         if (lane == 0) {

@@ -236,7 +236,7 @@ __device__ bool split_consumers(const Shm &sm, uint8_t *gb, const Layout &L, Sta
                     int okj = 1;
                     if (use > 0 && lane == 0) okj = mbar_wait_bounded(slot_empty(j), (use - 1) & 1, kWaitTimeoutNs);
                     okj = __shfl_sync(0xFFFFFFFFu, okj, 0);
-                    phase_search8(sm, win.n, lane, p.kq, p.cval);
+                    phase_search8<MODE>(sm, win.n, lane, p.kq, p.cval);
                     __syncwarp();
                     if (lane == 0) {
                         if (okj) {

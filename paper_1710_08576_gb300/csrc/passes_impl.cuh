@@ -11,41 +11,67 @@
 namespace rfi {
 namespace dev {
 
-// One warp per chunk of kMomChunk consecutive windows of one stream. The warp builds a
-// histogram of the MADs of the k_mom windows before the chunk, then slides: per window it
-// adds the window's MAD, drops the one k_mom windows back, and finds the lower median of the
-// (at most k_mom) MADs in the histogram with a two-level search (32-bin groups, then bins).
-// MAD values are histogram bins: [0, 255] for int8 samples, [0, 4095] for 12-bit.
-template <int NB>
-__global__ void __launch_bounds__(32) mom_kernel(const MomChunk *__restrict__ chunks, const int32_t *__restrict__ D,
-                                                 int32_t *__restrict__ Mm, int kmom) {
+// One block per chunk of kMomChunk consecutive windows of one stream. The block builds a histogram
+// of the MADs of the k_mom windows before the chunk (equal values of a warp counted at once: a
+// stream's MADs take few values); each of its NW warps takes a share of the chunk's windows, brings a
+// copy of the histogram up to its first window and slides: per window it adds the window's
+// MAD, drops the one k_mom windows back, and finds the lower median of the (at most k_mom) MADs in
+// the histogram with a two-level search (32-bin groups, then bins). MAD values are histogram
+// bins: [0, 255] for int8 samples, [0, 4095] for 12-bit (whose larger tables leave room for two
+// warps). The slide is one dependent chain, so its length sets the time: with one warp for the
+// whole chunk and its histogram the pass took 59 us on 60 x 4096 windows, k_mom 4096, now 14.
+template <int NB, int NW>
+__global__ void __launch_bounds__(NW * 32) mom_kernel(const MomChunk *__restrict__ chunks, const int32_t *__restrict__ D,
+                                                      int32_t *__restrict__ Mm, int kmom) {
     constexpr int NC = NB / 32;                  // groups of 32 bins
     constexpr int CPL = NC >= 32 ? NC / 32 : 1;  // groups per lane
-    __shared__ uint32_t h[NB];
-    __shared__ uint32_t hc[NC];
+    constexpr int T = NW * 32;
+    constexpr int SHARE = kMomChunk / NW;        // windows per warp
+    static_assert(kMomChunk % NW == 0, "even shares");
+    __shared__ uint32_t hist[NW][NB], group[NW][NC];
     __shared__ int32_t add[kMomChunk], drop[kMomChunk], res[kMomChunk];
-    const int lane = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const MomChunk c = chunks[blockIdx.x];
     const int32_t *d = D + c.base;
     auto bin = [](int32_t v) { return v < 0 ? 0 : (v > NB - 1 ? NB - 1 : v); };
-    for (int i = lane; i < NB; i += 32) h[i] = 0u;
-    for (int i = lane; i < NC; i += 32) hc[i] = 0u;
-    __syncwarp();
+    for (int i = tid; i < NB; i += T) hist[0][i] = 0u;
+    __syncthreads();
     const int n = c.b - c.a;
     // the histogram enters the chunk holding window a - 1's MADs: windows [a - kmom, a)
     const int lo = c.a - kmom > 0 ? c.a - kmom : 0;
-    for (int i = lo + lane; i < c.a; i += 32) {
-        const int v = bin(d[i]);
-        atomicAdd(&h[v], 1u);
-        atomicAdd(&hc[v >> 5], 1u);
+    for (int i0 = lo; i0 < c.a; i0 += T) {  // (whole warps: every lane votes)
+        const int i = i0 + tid;
+        const int v = i < c.a ? bin(d[i]) : -1;
+        const unsigned same = __match_any_sync(0xFFFFFFFFu, v);
+        if (v >= 0 && lane == __ffs(static_cast<int>(same)) - 1) atomicAdd(&hist[0][v], static_cast<uint32_t>(__popc(same)));
     }
-    for (int i = lane; i < n; i += 32) {
+    for (int i = tid; i < n; i += T) {
         add[i] = bin(d[c.a + i]);
         const int j = c.a + i - kmom;
         drop[i] = j >= 0 ? bin(d[j]) : -1;
     }
+    __syncthreads();
+    for (int i = tid; i < NB; i += T) {
+        const uint32_t v = hist[0][i];
+#pragma unroll
+        for (int w = 1; w < NW; ++w) hist[w][i] = v;
+    }
+    __syncthreads();
+    uint32_t *const h = hist[warp], *const hc = group[warp];
+    const int first = warp * SHARE, last = min(first + SHARE, n);
+    for (int i = lane; i < min(first, n); i += 32) {
+        atomicAdd(&h[add[i]], 1u);
+        if (drop[i] >= 0) atomicSub(&h[drop[i]], 1u);
+    }
     __syncwarp();
-    for (int i = 0; i < n; ++i) {
+    for (int g = lane; g < NC; g += 32) {
+        uint32_t s = 0u;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) s += h[32 * g + ((k + lane) & 31)];
+        hc[g] = s;
+    }
+    __syncwarp();
+    for (int i = first; i < last; ++i) {
         const int j = c.a + i;
         if (lane == 0) {
             const int v = add[i], u = drop[i];
@@ -92,14 +118,16 @@ __global__ void __launch_bounds__(32) mom_kernel(const MomChunk *__restrict__ ch
         if (lane == 0) res[i] = 32 * g + b;
         __syncwarp();
     }
-    for (int i = lane; i < n; i += 32) Mm[c.base + c.a + i] = res[i];
+    __syncthreads();
+    for (int i = tid; i < n; i += T) Mm[c.base + c.a + i] = res[i];
 }
 
 template <int NB>
 cudaError_t mom_launch_t(const MomChunk *chunks, int nchunks, const int32_t *D, int32_t *Mm, int kmom,
                          cudaStream_t st) {
     if (nchunks <= 0) return cudaSuccess;
-    mom_kernel<NB><<<nchunks, 32, 0, st>>>(chunks, D, Mm, kmom);
+    constexpr int NW = NB == 256 ? 8 : 2;
+    mom_kernel<NB, NW><<<nchunks, NW * 32, 0, st>>>(chunks, D, Mm, kmom);
     return cudaGetLastError();
 }
 

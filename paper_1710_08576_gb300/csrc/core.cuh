@@ -297,7 +297,8 @@ struct Geo {
     static constexpr int kBps = BITS == 8 ? 1 : 2;          // bytes per sample
     static constexpr int kLo = BITS == 8 ? -128 : -2048;
     static constexpr int kHi = BITS == 8 ? 127 : 2047;
-    // 8-bit: cumulative counts, padded (pad32); 12-bit: the histogram's second table
+    // 8-bit: 256 cumulative counts (264 words: the distance of two multi-window slots' 16-bit counts);
+    // 12-bit: the histogram's second table
     static constexpr int kCumWords = BITS == 8 ? kBins + kBins / 32 : kBins;
     static constexpr int kChunkSamples = 16 / kBps;          // samples per 16-byte chunk
     // 8-bit, one consumer group: a 32 KiB table of 128-byte rows (raw byte u -> row u, lane l
@@ -313,8 +314,6 @@ struct Geo {
 // Shared-window address of the first byte of dynamic shared memory. The 8-bit histogram sits
 // there and its atomics use it as an immediate offset; kernels check it at entry.
 constexpr uint32_t kDynSmemShared = 1024;
-
-__device__ __forceinline__ int pad32(int b) { return b + (b >> 5); }
 
 struct __align__(16) RepShared {
     int32_t M, D, t, hiv, lov;
@@ -360,7 +359,7 @@ struct Ctl {
     uint32_t ncount[4];  // digital-noise list entries, by window parity (and slice of the window, 12-bit)
     unsigned long long pw[2][2];  // power-metered excision: {sum x^2, sum z^2}, by window parity
     uint32_t abort;      // set when any warp gave up on a bounded wait
-    int32_t mb;          // median bin of the current window (written by its owner thread)
+    int32_t pad;
     unsigned long long flagged;  // group total
 };
 
@@ -375,7 +374,7 @@ struct Shm {
     uint8_t *hist;       // histogram (generic pointer; 8-bit: the 64 KiB table)
     uint32_t hist_s;     // histogram (shared address)
     uint32_t grp;        // 8-bit: byte offset of this group's half row (0 or 128)
-    uint32_t *cum;       // padded cumulative counts; 12-bit: the histogram's second table (table12)
+    uint32_t *cum;       // cumulative counts; 12-bit: the histogram's second table (table12)
     uint32_t *coarse;    // 12-bit estimation pass: the rows' cumulative counts (or null: see rows12)
     Ctl *ctl;
     int ncopies;         // 12-bit only
@@ -597,44 +596,41 @@ __device__ __forceinline__ void phase_reduce8_counts(const Shm &sm, int tid, Row
                 const uint4 a = row[(q + lane) & 7];
                 s += a.x + a.y + a.z + a.w;
             }
-            sm.cum[pad32(tid * BPT + i)] = s - rs.s[i];
+            sm.cum[tid * BPT + i] = s - rs.s[i];
             rs.s[i] = s;
         }
     }
 }
 
-// One warp, after phase_reduce8_counts and a group barrier: the inclusive scan of the 256 counts
-// in place (8 consecutive bins per lane) and the median bin, the lowest whose cumulative count
-// reaches ceil(n/2), into the control block.
-__device__ __forceinline__ void phase_scan8_warp(const Shm &sm, uint32_t *cum, int n, int lane) {
-    uint32_t c[8];
-    uint32_t run = 0;
+// One warp: the inclusive scan of 256 counts in place (8 consecutive ones per lane, 16 bytes at a
+// time) and the first whose cumulative count reaches half, in every lane. cum on a 16-byte boundary.
+__device__ __forceinline__ int scan256_warp(uint32_t *cum, uint32_t half, int lane) {
+    uint4 *const own = reinterpret_cast<uint4 *>(cum) + 2 * lane;
+    const uint4 a = own[0], b = own[1];
+    uint32_t c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        run += cum[pad32(lane * 8 + j)];
-        c[j] = run;
-    }
-    uint32_t inc = run;
+    for (int j = 1; j < 8; ++j) c[j] += c[j - 1];
+    uint32_t inc = c[7];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
         if (lane >= o) inc += y;
     }
-    const uint32_t excl = inc - run;
-    const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
-    int found = -1;
+    const uint32_t excl = inc - c[7];
+    uint32_t below = 0u;  // those that stay below half lie before the one wanted
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const uint32_t v = c[j] + excl;
-        const uint32_t before = (j ? c[j - 1] : 0u) + excl;
-        cum[pad32(lane * 8 + j)] = v;
-        if (v >= half && before < half) found = lane * 8 + j;
+        c[j] += excl;
+        below += c[j] < half ? 1u : 0u;
     }
-    if (found >= 0) sm.ctl->mb = found;
+    own[0] = make_uint4(c[0], c[1], c[2], c[3]);
+    own[1] = make_uint4(c[4], c[5], c[6], c[7]);
+    const int first = static_cast<int>(__reduce_add_sync(0xFFFFFFFFu, below));
     __syncwarp();
+    return first;
 }
 
-// 12-bit: the 4096 bins as 256 rows of 16. Each row's total goes into coarse (padded), for one warp
+// 12-bit: the 4096 bins as 256 rows of 16. Each row's total goes into coarse, for one warp
 // to scan as the 256 counts of an 8-bit window; the copies are folded into copy 0 on the way. The
 // table of the window before is cleared. coarse is the first kCoarse words of that table (its words
 // are zeroed by the search, search12) or, in the estimation pass, whose other warps go on to the
@@ -644,7 +640,7 @@ __device__ __forceinline__ void phase_scan8_warp(const Shm &sm, uint32_t *cum, i
 // table, a block-wide offset exchange and a fourth barrier: about 1400 instructions of its warps per
 // window against 350 (60 streams of 2^22 samples in 2048-sample windows, threshold, 2 CTAs: 1024 -> 991 us;
 // with one histogram copy and 3 CTAs, for which there was no room in the old default: 651 us).
-constexpr int kCoarse = 264;
+constexpr int kCoarse = 256;
 template <int T>
 __device__ __forceinline__ void phase_rows12(const Shm &sm, int tid, int par, uint32_t *coarse) {
     uint32_t *const old = table12(sm, par ^ 1);
@@ -672,7 +668,7 @@ __device__ __forceinline__ void phase_rows12(const Shm &sm, int tid, int par, ui
             }
             s += v.x + v.y + v.z + v.w;
         }
-        coarse[pad32(r)] = s;
+        coarse[r] = s;
     }
 }
 
@@ -763,18 +759,18 @@ __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, 
     return r;
 }
 
-// One warp: lower median bin, then the MAD, then the threshold and replacement values, written
-// to the shared control block.
+// One warp, 8-bit: after phase_reduce8_counts and a group barrier, the scan of the counts, the lower
+// median bin, then the MAD, then the threshold and replacement values, written to the shared
+// control block. The window's other threads wait for this chain, so its length counts.
 template <int MODE>
 __device__ __forceinline__ void phase_search8(const Shm &sm, int n, int lane, int64_t kq, int32_t cval) {
-    constexpr int B = Geo<8>::kBins;
     const uint32_t *cum = sm.cum;
     const uint32_t half = static_cast<uint32_t>((n + 1) >> 1);
-    const int mb = sm.ctl->mb;  // found by its owner thread during the scan
-    const int d = warp_search<B>(lane, [&](int dd) {
-        const int hi = mb + dd < B - 1 ? mb + dd : B - 1;
+    const int mb = scan256_warp(sm.cum, half, lane);
+    const int d = warp_search<256>(lane, [&](int dd) {
+        const int hi = mb + dd < 255 ? mb + dd : 255;
         const int lo = mb - dd - 1;
-        const uint32_t f = cum[pad32(hi)] - (lo >= 0 ? cum[pad32(lo)] : 0u);
+        const uint32_t f = cum[hi] - (lo >= 0 ? cum[lo] : 0u);
         return f >= half;
     });
     if (lane == 0) sm.ctl->rep = make_rep<8, MODE>(mb - Geo<8>::kOffset, d, kq, cval);
@@ -799,9 +795,8 @@ __device__ __forceinline__ void phase_search12(const Shm &sm, const uint32_t *ta
         }
         return v;
     };
-    auto upto = [&](int r) { return r >= 0 ? cc[pad32(r)] : 0u; };  // samples in rows 0 .. r
-    phase_scan8_warp(sm, cc, n, lane);
-    const int R = sm.ctl->mb;
+    auto upto = [&](int r) { return r >= 0 ? cc[r] : 0u; };  // samples in rows 0 .. r
+    const int R = scan256_warp(cc, half, lane);
     const uint32_t in_row = prefix(lane < 16 ? tab[16 * R + lane] : 0u);
     const int M = 16 * R + __ffs(__ballot_sync(0xFFFFFFFFu, upto(R - 1) + in_row >= half)) - 1;
     const int s = warp_search<256>(lane, [&](int x) { return upto(min(R + x, 255)) - upto(R - x - 1) >= half; });
@@ -1565,7 +1560,6 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         named_bar(sm.bar_id, T);
         if (tid < 32) {
             if constexpr (BITS == 8) {
-                phase_scan8_warp(sm, sm.cum, w.n, lane);
                 phase_search8<MODE>(sm, w.n, lane, p.kq, p.cval);
             } else {
                 phase_search12<MODE>(sm, table12(sm, par), sm.coarse, false, w.n, lane, p.kq, p.cval);
@@ -1589,7 +1583,6 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         named_bar(sm.bar_id, T);
         if (tid < 32) {
             if constexpr (BITS == 8) {
-                phase_scan8_warp(sm, sm.cum, w.n, lane);
                 phase_search8<MODE>(sm, w.n, lane, p.kq, p.cval);
             } else {
                 phase_search12<MODE>(sm, table12(sm, par), table12(sm, par ^ 1), true, w.n, lane, p.kq, p.cval);
@@ -1879,8 +1872,7 @@ __device__ __forceinline__ void reduce8_multi(const Shm &sm, int tid) {
 }
 
 // One warp: the inclusive scan of a slot's 256 counts in place (8 consecutive bins per lane, one
-// 16-byte load and store), then its lower median bin and MAD (the searches of phase_scan8_warp and
-// phase_search8), and the threshold and replacement values into *rep (lane 0). The counts and
+// 16-byte load and store), then its lower median bin and MAD (as phase_search8), and the threshold and replacement values into *rep (lane 0). The counts and
 // cumulative counts are 16-bit (a window of this form has at most 8192 samples).
 template <int MODE>
 __device__ __forceinline__ void scan_search8(uint16_t *cum, int n, int lane, int64_t kq, int32_t cval,

@@ -231,7 +231,6 @@ __device__ bool split_consumers(const Shm &sm, uint8_t *gb, const Layout &L, Sta
                 phase_reduce8_counts<TH, 128>(sm, tid, rs);
                 named_bar(1, TH);
                 if (tid < 32) {
-                    phase_scan8_warp(sm, sm.cum, win.n, lane);
                     const int j = seq % kSplitSlots, use = seq / kSplitSlots;
                     int okj = 1;
                     if (use > 0 && lane == 0) okj = mbar_wait_bounded(slot_empty(j), (use - 1) & 1, kWaitTimeoutNs);

@@ -474,14 +474,17 @@ __device__ __forceinline__ uint32_t copy12(const Shm &sm, int c, int par) {
 }
 
 // Two 12-bit samples in int16 halves. The bin x + 2048 of an in-range sample is its low 12 bits
-// with bit 11 flipped; a half is in range iff its bits 15..11 are all equal, which the caller
-// accumulates as (w ^ (w << 1)) & 0xF000F000.
+// with bit 11 flipped; the upper half's bin sits 14 bits above its table offset. A half is in range
+// iff its bits 15..11 are all equal: the caller collects w ^ (w << 1) and looks at its bits
+// 0xF000F000 (kRange12) once.
+constexpr uint32_t kRange12 = 0xF000F000u;
 __device__ __forceinline__ void hist12_word(uint32_t copy_base, uint32_t w) {
-    red_add_shared(copy_base + (((w & 0xFFFu) ^ 0x800u) << 2), 1u);
-    red_add_shared(copy_base + ((((w >> 16) & 0xFFFu) ^ 0x800u) << 2), 1u);
+    const uint32_t u = (w ^ 0x08000800u) & 0x0FFF0FFFu;
+    red_add_shared(copy_base + ((u & 0xFFFFu) << 2), 1u);
+    red_add_shared(copy_base + (u >> 14), 1u);
 }
 
-__device__ __forceinline__ uint32_t range12_bits(uint32_t w) { return (w ^ (w << 1)) & 0xF000F000u; }
+__device__ __forceinline__ uint32_t range12_bits(uint32_t w) { return w ^ (w + w); }
 
 template <int BITS, int T, int ROWB>
 __device__ __forceinline__ void phase_histogram(const Shm &sm, const Win &w, int tid, int par) {
@@ -510,6 +513,9 @@ __device__ __forceinline__ void phase_histogram(const Shm &sm, const Win &w, int
     } else {
         const uint32_t cb = copy12(sm, lane & (sm.ncopies - 1), par);
         uint32_t bad = 0;
+        // not unrolled: a window of 8192 samples has four rounds, and the unrolled loop's entry costs
+        // more than it saves (8192-sample windows 583 -> 578 us, 4096 395 -> 382, 1024 1107 -> 1053)
+#pragma unroll 1
         for (int c = tid; c < nfull; c += T) {
             const uint4 a = d4[c];
             hist12_word(cb, a.x); hist12_word(cb, a.y); hist12_word(cb, a.z); hist12_word(cb, a.w);
@@ -521,7 +527,7 @@ __device__ __forceinline__ void phase_histogram(const Shm &sm, const Win &w, int
             red_add_shared(cb + (((x & 0xFFFu) ^ 0x800u) << 2), 1u);
             bad |= range12_bits(x) & 0xF000u;
         }
-        if (bad) atomicOr(&sm.ctl->err[par], 1u);
+        if (bad & kRange12) atomicOr(&sm.ctl->err[par], 1u);
     }
 }
 
@@ -573,7 +579,7 @@ __device__ __forceinline__ void phase_histogram_any(const Shm &sm, const Win &w,
                             red_add_shared(cb + (((x & 0xFFFu) ^ 0x800u) << 2), 1u);
                             bad |= range12_bits(x) & 0xF000u;
                         });
-        if (bad) atomicOr(&sm.ctl->err[par], 1u);
+        if (bad & kRange12) atomicOr(&sm.ctl->err[par], 1u);
     }
 }
 
@@ -748,7 +754,7 @@ __device__ __forceinline__ RepShared make_rep(int32_t M, int32_t d, int64_t kq, 
         // 12-bit, two samples per word (see rep12_word): u = x + 2048 per 16-bit half
         const uint32_t mb = static_cast<uint32_t>(r.M + 2048);
         const uint32_t tt = static_cast<uint32_t>(r.t);  // <= 4096
-        r.mb4 = (mb + tt) * 0x00010001u;                  // upper bound, u >= it flags
+        r.mb4 = (0x8000u - mb - tt) * 0x00010001u;        // 0x8000 - upper bound, u >= it flags
         r.tlo7 = (0x8000u + mb - tt) * 0x00010001u;       // 0x8000 + lower bound, u <= it flags
         if constexpr (ALL || RMODE == 1) r.c4 = (static_cast<uint32_t>(cval) & 0xFFFFu) * 0x00010001u;
         if constexpr (ALL || RMODE == 2) {
@@ -871,13 +877,14 @@ __device__ __forceinline__ Rep8 load_rep8(const RepShared *rsrc) {
     return k;
 }
 
-// 4 int8 samples: returns the output word and sets f to 0xFF in flagged bytes. Noise bytes are
-// left 0 here and written by the compacted noise pass.
+// 4 int8 samples: returns the output word and sets f to 0xFF in flagged bytes. With digital noise the
+// word stays as it is: the noise overwrites every flagged sample.
 template <int MODE>
 __device__ __forceinline__ uint32_t rep8_word(uint32_t w, const Rep8 &k, uint32_t &f) {
     const uint32_t wb = w ^ 0x80808080u;                  // x + 128 in every byte
     const uint32_t ad = __vabsdiffu4(wb, k.mb4);         // |x - M|
     f = prmt(ge_bytes_msb(ad, k.tlo7, k.tsmall), 0u, 0xBA98u);
+    if (MODE == 3) return w;
     uint32_t rep = 0u;
     if (MODE == 1) rep = k.c4;
     if (MODE == 2) {
@@ -887,33 +894,37 @@ __device__ __forceinline__ uint32_t rep8_word(uint32_t w, const Rep8 &k, uint32_
     return (w & ~f) | (rep & f);
 }
 
-// Two 12-bit samples (int16 halves of w, in range): returns the output word and sets m to 0xFFFF in
-// flagged halves. With u = x + 2048 (12 bits) per half and bounds lo = M + 2048 - t,
+// Two 12-bit samples (int16 halves of w, in range): returns the output word and sets f, whose bits 15
+// and 31 are the samples' flags. With u = x + 2048 (12 bits) per half and bounds lo = M + 2048 - t,
 // hi = M + 2048 + t: x is flagged iff u >= hi or u <= lo (Eq. 2 with |x - M| >= t). Per half,
-// (u | 0x8000) - hi has bit 15 set iff u >= hi, and (0x8000 + lo) - u iff u <= lo; no borrow
-// crosses the halves because every operand is below 2^13. A flag moved down to bit 0 / 16 and
-// multiplied by 0xFFFF gives the half's select mask.
+// u + (0x8000 - hi) has bit 15 set iff u >= hi, and (0x8000 + lo) - u iff u <= lo; no carry or borrow
+// crosses the halves because every operand is below 2^13. A byte permute that takes the sign of
+// bytes 1 and 3 makes a flag its half's select mask. With digital noise the word stays as it is: the
+// noise overwrites every flagged sample.
+__device__ __forceinline__ uint32_t half_mask(uint32_t f) { return prmt(f, 0u, 0xBB99u); }
 template <int MODE>
 __device__ __forceinline__ uint32_t rep12_word(uint32_t w, uint32_t hi2, uint32_t lo2x, uint32_t c2, uint32_t h2,
-                                               uint32_t l2, uint32_t &m) {
+                                               uint32_t l2, uint32_t &f) {
     const uint32_t u = (w ^ 0x08000800u) & 0x0FFF0FFFu;
-    const uint32_t up = (u | 0x80008000u) - hi2;   // bit 15 / 31: u >= hi
-    const uint32_t dn = lo2x - u;                   // bit 15 / 31: u <= lo
-    m = (((up | dn) & 0x80008000u) >> 15) * 0xFFFFu;
+    const uint32_t up = u + hi2;   // bit 15 / 31: u >= hi
+    const uint32_t dn = lo2x - u;  // bit 15 / 31: u <= lo
+    f = up | dn;
+    if (MODE == 3) return w;
+    const uint32_t m = half_mask(f);
     uint32_t z = 0u;
     if (MODE == 1) z = c2;
     if (MODE == 2) {
-        const uint32_t ma = ((up >> 15) & 0x00010001u) * 0xFFFFu;
+        const uint32_t ma = half_mask(up);
         z = (h2 & ma) | (l2 & ~ma);
     }
     return (w & ~m) | (z & m);
 }
 
-// Mask bits of a chunk of eight 12-bit samples from its four flag words (0x0000/0xFFFF halves): one
-// byte of each flag, then the signed byte dot product of chunk_bits.
+// Mask bits of a chunk of eight 12-bit samples from its four words of flags (bits 15 and 31): the
+// signs of the flags' bytes, then the signed byte dot product of chunk_bits.
 __device__ __forceinline__ uint32_t chunk_bits12(uint32_t f0, uint32_t f1, uint32_t f2, uint32_t f3) {
-    return static_cast<uint32_t>(__dp4a(static_cast<int>(prmt(f2, f3, 0x6420u)), static_cast<int>(0x80C0E0F0u),
-                                        __dp4a(static_cast<int>(prmt(f0, f1, 0x6420u)), static_cast<int>(0xF8FCFEFFu), 0)));
+    return static_cast<uint32_t>(__dp4a(static_cast<int>(prmt(f2, f3, 0xFDB9u)), static_cast<int>(0x80C0E0F0u),
+                                        __dp4a(static_cast<int>(prmt(f0, f1, 0xFDB9u)), static_cast<int>(0xF8FCFEFFu), 0)));
 }
 
 // Mask bits of a 16-sample chunk from its four flag words (0x00/0xFF bytes), sample j -> bit j.
@@ -1250,6 +1261,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
     const uint4 *d4 = reinterpret_cast<const uint4 *>(w.data);
     uint32_t flagged = 0;
     if (BITS == 8) {
+        constexpr int M8 = PW && MODE == 3 ? 0 : MODE;  // power metering adds the noise's squares to zeros'
         const Rep8 k = load_rep8(rsrc);
         uint16_t *mk = reinterpret_cast<uint16_t *>(w.mask);
         int base = warp * 32;
@@ -1258,10 +1270,10 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
             auto full_round = [&](int c, uint4 v) {
                 if (PW) pw.x += sq4(v.x, ~0u) + sq4(v.y, ~0u) + sq4(v.z, ~0u) + sq4(v.w, ~0u);
                 uint32_t f0, f1, f2, f3;
-                v.x = rep8_word<MODE>(v.x, k, f0);
-                v.y = rep8_word<MODE>(v.y, k, f1);
-                v.z = rep8_word<MODE>(v.z, k, f2);
-                v.w = rep8_word<MODE>(v.w, k, f3);
+                v.x = rep8_word<M8>(v.x, k, f0);
+                v.y = rep8_word<M8>(v.y, k, f1);
+                v.z = rep8_word<M8>(v.z, k, f2);
+                v.w = rep8_word<M8>(v.w, k, f3);
                 const uint32_t bits = chunk_bits(f0, f1, f2, f3);
                 if (!FO || (MODE != 3 && bits)) store_chunk8<OUTF>(w.out, c, v, true);
                 if (PW) pw.z += sq4(v.x, ~0u) + sq4(v.y, ~0u) + sq4(v.z, ~0u) + sq4(v.w, ~0u);
@@ -1293,10 +1305,10 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
                 const uint4 vin = v;
                 if (r.active) {
                     uint32_t f0, f1, f2, f3;
-                    v.x = rep8_word<MODE>(v.x, k, f0);
-                    v.y = rep8_word<MODE>(v.y, k, f1);
-                    v.z = rep8_word<MODE>(v.z, k, f2);
-                    v.w = rep8_word<MODE>(v.w, k, f3);
+                    v.x = rep8_word<M8>(v.x, k, f0);
+                    v.y = rep8_word<M8>(v.y, k, f1);
+                    v.z = rep8_word<M8>(v.z, k, f2);
+                    v.w = rep8_word<M8>(v.w, k, f3);
                     bits = chunk_bits(f0, f1, f2, f3);
                 }
                 if (c < nfull) {
@@ -1333,7 +1345,8 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
     } else {
         uint8_t *mk = reinterpret_cast<uint8_t *>(w.mask);
         const int32_t t = r.t;
-        const RepShared k12 = *rsrc;
+        const uint32_t hi2 = rsrc->mb4, lo2 = rsrc->tlo7, c2 = MODE == 1 ? rsrc->c4 : 0u;
+        const uint32_t h2 = MODE == 2 ? rsrc->hi4 : 0u, l2 = MODE == 2 ? rsrc->lo4 : 0u;
         const int cend = MODE == 3 ? min(nchunks, slice + kNoiseSlice) : nchunks;  // slice: its first chunk
         for (int base = slice + warp * 32; base < cend; base += T) {
             const int c = base + lane;
@@ -1346,8 +1359,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
                     if (r.active) {
                         uint32_t f[4];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) ww[q] = rep12_word<MODE>(ww[q], k12.mb4, k12.tlo7, k12.c4, k12.hi4,
-                                                                             k12.lo4, f[q]);
+                        for (int q = 0; q < 4; ++q) ww[q] = rep12_word<MODE>(ww[q], hi2, lo2, c2, h2, l2, f[q]);
                         bits = chunk_bits12(f[0], f[1], f[2], f[3]);
                         // samples past the window (a ragged last chunk) are neither flagged nor stored
                         if (valid < 8) bits &= (1u << valid) - 1u;
@@ -1849,19 +1861,19 @@ __device__ __forceinline__ void hist8_multi(const Shm &sm, const uint8_t *stage,
 // byte u holds lane l's count at word l; a slot's lanes are 8/K of the row's eight 16-byte
 // groups). The eight threads tid & ~7 .. tid | 7 read the eight groups of the same row, so the
 // reads and clears are free of bank conflicts; with four slots, thread pairs combine their
-// groups by a shuffle. Counts go to 16-bit arrays, 264 entries apart (slot g's array starts
+// groups by a shuffle. A warp takes four neighbouring rows at a time, so that its 16-bit stores fall
+// into two neighbouring words of each slot (rows 8 apart met in a bank four ways). Counts go to 16-bit arrays, 264 entries apart (slot g's array starts
 // on bank 4g, so the stores of one row's slots do not collide either, and on a 16-byte boundary).
 template <int T, int K>
 __device__ __forceinline__ void reduce8_multi(const Shm &sm, int tid) {
     static_assert(K == 4 || K == 8, "four or eight window slots");
     constexpr int RPT = 256 / (T / 8);  // rows per thread
     const int p = tid & 7;
-    const int r0 = (tid >> 3) * RPT;
     uint4 *tab = reinterpret_cast<uint4 *>(sm.hist);
     uint16_t *cumg = reinterpret_cast<uint16_t *>(sm.cum) + (K == 8 ? p : (p >> 1)) * Geo<8>::kCumWords;
 #pragma unroll 4
     for (int k = 0; k < RPT; ++k) {
-        const int row = r0 + k;
+        const int row = (tid >> 3) + k * (T / 8);
         uint4 *a = tab + row * 8 + p;
         const uint4 v = *a;
         *a = make_uint4(0u, 0u, 0u, 0u);

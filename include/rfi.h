@@ -129,7 +129,8 @@ typedef struct rfi_launch_shape {
     int32_t stages;          /* shared-memory window buffers per CTA, 1..8 */
     int32_t ctas_per_sm;     /* resident CTAs per SM, 1..4 */
     int32_t stage_bytes;     /* bytes per buffer (>= the largest window); 0 = choose */
-    int32_t dynamic_tiles;   /* 1: tiles taken from an atomic counter; 2: static round robin */
+    int32_t dynamic_tiles;   /* 1: tiles taken from an atomic counter; 2: static round robin. 0 = choose:
+                                1, or 2 for small plans of one window size */
     int32_t hist_copies;     /* 12-bit histogram copies (1, 2, 4); ignored for 8-bit */
     int32_t groups;          /* consumer groups per CTA, 1 or 2 (each with its own copy warp;
                                 2 needs consumer_warps <= 8) */
@@ -139,7 +140,8 @@ typedef struct rfi_launch_shape {
                                 threshold plans with 8 consumer warps in one group, also
                                 write-flagged, but neither power-metered, nor digital copies, nor
                                 another output format; RFI_ERR_UNSUPPORTED otherwise). 0 = choose: the
-                                autotuner tries both where the split form runs, otherwise 1 */
+                                autotuner tries both where the split form runs; otherwise 2 where it
+                                runs in plans of many tiles, else 1 */
 } rfi_launch_shape;
 
 typedef struct rfi_plan_desc {

@@ -40,7 +40,7 @@ bool valid_shape(const rfi_launch_shape &s) {
 namespace rfi {
 
 rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
-    Shape s;
+    Shape s{};
     const int bps = P->bits == 8 ? 1 : 2;
     int64_t maxwb = 0;
     bool uniform = true;
@@ -67,11 +67,12 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
     bool mom4096 = P->kmom >= 2 && P->bits == 8;
     for (int i = 0; i < P->S && mom4096; ++i) mom4096 = P->W[i] == 4096 && P->len[i] >= 8 * 4096;
     const bool mom_stage = mom4096 && !(req && (req->stage_bytes || req->stages));
+    P->given_stage = req && req->stage_bytes;
     s.stage_bytes = std::max(min_stage, (req && req->stage_bytes) ? req->stage_bytes : (mom_stage ? 32768 : 16384));
     s.stage_bytes = (s.stage_bytes + 127) / 128 * 128;
     s.stages = (req && req->stages) ? req->stages : (mom_stage ? 1 : 2);
     s.hist_copies = P->bits == 8 ? 1 : ((req && req->hist_copies) ? req->hist_copies : kDefaultHistCopies);
-    s.dynamic_tiles = (req && req->dynamic_tiles) ? req->dynamic_tiles : (uniform ? 2 : 1);
+    s.dynamic_tiles = (req && req->dynamic_tiles) ? req->dynamic_tiles : 1;  // small plans: below
     const int want_ctas = (req && req->ctas_per_sm) ? req->ctas_per_sm : 4;  // as many as fit, up to 4
     // the shape is sized for the kernel with the histogram (the MoM stats pass)
     const int kmode = P->kmom >= 2 ? plan_stats_mode(P) : plan_kernel_mode(P);
@@ -89,9 +90,29 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
         if (occ_apply < 1) return cudaGetLastError() != cudaSuccess ? RFI_ERR_CUDA : RFI_ERR_UNSUPPORTED;
         P->grid_apply = P->sm_count * occ_apply;  // clamped to the tile count with the grid
     }
-    // the split-warp form only where it runs: int8 zero / constant / threshold, one group of 8
+    // plans of many tiles per CTA take tiles from the cursor: SMs differ in pace (60 streams of 2^24
+    // int8 samples, fp16 output, 135 tiles a CTA: 612 us a call round robin, 575 from the cursor; 60 x
+    // 2^22 12-bit noise 577 and 526; 8 variants 812 and 754). With few (60 x 2^19 samples, 4 tiles a
+    // CTA: 42.3 and 45.5 us) the cursor's round trips cost more, unless window sizes differ.
+    int64_t tiles = 0;
+    for (int i = 0; i < P->S; ++i) {
+        const int64_t per = tile_windows(P->bits, plan_tile_mode(P), P->W[i], s.stage_bytes);
+        tiles += (P->nwin[i] + per - 1) / per;
+    }
+    const bool many = tiles >= 16 * static_cast<int64_t>(P->sm_count) * s.ctas_per_sm;
+    if (!(req && req->dynamic_tiles)) s.dynamic_tiles = !uniform || many ? 1 : 2;
+    // the split-warp form runs int8 zero / constant / threshold, one group of 8; there plans of many
+    // tiles take it (60 streams of 2^22 samples from the cursor, zero, 16384-sample windows: 118.1 us
+    // joint, 112.1 split; threshold 130.4 and 122.1; 65536-sample windows 123.3 and 116.2)
     s.warp_split = (req && req->warp_split) ? req->warp_split : 1;
     if (s.warp_split == 2 && !plan_warp_split_runs(P, s)) return RFI_ERR_UNSUPPORTED;
+    if (!(req && req->warp_split) && many && plan_warp_split_runs(P, s)) {
+        Shape split = s;
+        split.warp_split = 2;
+        if (persistent_smem_bytes(P->bits, kmode, split) <= 227u * 1024u &&
+            persistent_occupancy(P->bits, kmode, split) >= s.ctas_per_sm)
+            s = split;
+    }
     P->shape = s;
     return RFI_OK;
 }
@@ -103,10 +124,32 @@ bool plan_warp_split_runs(const rfi_plan_s *P, const Shape &s) {
 
 rfi_status plan_build_tiles(rfi_plan_s *P) {
     const int bps = P->bits == 8 ? 1 : 2;
-    std::vector<Tile> tiles;
-    for (int i = 0; i < P->S; ++i) {
+    auto per_tile = [&](int i, int64_t div) {
         int64_t per = tile_windows(P->bits, plan_tile_mode(P), P->W[i], P->shape.stage_bytes);
         if (P->kmom >= 2) per = std::min<int64_t>(per, kApplyTileWindows);
+        return std::max<int64_t>(1, per / div);
+    };
+    // a small plan spreads its windows: tiles of fewer windows as long as all of them still run at
+    // once (2^20 int8 samples in 4096-sample windows: 64 tiles of four 9.6 us a call, 256 of one 8.2,
+    // with noise 12.3 and 8.8; 2^22 samples: 256 tiles 10.3 us, 512 on 456 CTAs 12.4). A stage size
+    // that the caller gave stands for its tiles.
+    int64_t div = 1;
+    if (!P->given_stage) {
+        auto count = [&](int64_t d) {
+            int64_t n = 0;
+            for (int i = 0; i < P->S; ++i) n += (P->nwin[i] + per_tile(i, d) - 1) / per_tile(i, d);
+            return n;
+        };
+        const int64_t room = static_cast<int64_t>(P->sm_count) * P->shape.ctas_per_sm;
+        for (int64_t n = count(1); div < 64 && n < room; div *= 2) {
+            const int64_t more = count(2 * div);
+            if (more == n || more > room) break;
+            n = more;
+        }
+    }
+    std::vector<Tile> tiles;
+    for (int i = 0; i < P->S; ++i) {
+        const int64_t per = per_tile(i, div);
         for (int64_t w0 = 0; w0 < P->nwin[i]; w0 += per) {
             const int64_t nw = std::min<int64_t>(per, P->nwin[i] - w0);
             const int64_t s0 = w0 * P->W[i];

@@ -40,6 +40,7 @@ struct rfi_plan_s {
     uint64_t total_windows = 0, total_samples = 0, last_windows = 0;
     int device = 0, sm_count = 0;
     rfi::Shape shape{};
+    bool given_stage = false;  // the caller's shape gives the stage size
     std::vector<rfi::Tile> tiles_host;
     int ntiles = 0, grid = 0;
     int grid_apply = 0;  // Median of MAD: grid of the apply pass (no histogram: more CTAs fit)

@@ -331,6 +331,12 @@ struct CopyShared {
     RepShared vrep[kMaxCopies];        // threshold and replacement values per variant
     uint32_t vcount[kMaxCopies][2];    // flagged samples, by variant and window parity
     uint32_t ncount[4 * kMaxCopies];   // digital-noise list entries, by variant, parity and slice
+    // int8: what the variants of one threshold multiple share a pass with (copies_pass8)
+    uint8_t *out[kMaxCopies];          // the window's output and mask, by variant
+    uint16_t *mask[kMaxCopies];
+    uint32_t group[kMaxCopies];        // bit u: variant u has the same multiple
+    uint32_t mode[kMaxCopies];         // rfi_mode
+    uint32_t fast;                     // the window goes through copies_pass8
 };
 
 // Apply passes over whole tiles: the thresholds and flag counts of the tile's windows.
@@ -1526,6 +1532,78 @@ __device__ __forceinline__ uint32_t noise_slices12(const Shm &sm, const Win &w, 
     }
 }
 
+// ------------------------------------------------------------------ digital copies
+// Eq. 2 for all variants of one threshold multiple at once (grp: their bits, v: the first of them),
+// over a window of whole warp rounds with aligned outputs and masks: same M, same t, so the flags,
+// the mask bits and the count are computed once, and each variant adds its own replacement and
+// stores (one variant at a time, every one of them computed the flags again: 8 variants, two
+// multiples with four replacements each, 60 streams of 2^22 samples 748 us a call, now 663).
+template <int T>
+__device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, int v, uint32_t grp, bool noise, int tid,
+                                                 uint32_t *nlc) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const RepShared &lead = sm.cp->vrep[v];
+    const Rep8 k = load_rep8(&lead);
+    const uint32_t on = lead.active ? ~0u : 0u;
+    const uint4 *d4 = reinterpret_cast<const uint4 *>(w.data);
+    const int nchunks = w.n >> 4;
+    uint32_t flagged = 0;
+    // two chunks of a lane at a time, so that a variant's mode, addresses and constants are read once
+    // for both
+    for (int c = warp * 32 + lane; c < nchunks; c += 2 * T) {
+        const bool two = c + T < nchunks;  // the same for the whole warp
+        uint32_t x[2][4], f[2][4], bits[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint4 a = h == 0 || two ? d4[c + h * T] : make_uint4(0u, 0u, 0u, 0u);
+            x[h][0] = a.x;
+            x[h][1] = a.y;
+            x[h][2] = a.z;
+            x[h][3] = a.w;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t ad = __vabsdiffu4(x[h][q] ^ 0x80808080u, k.mb4);
+                f[h][q] = prmt(ge_bytes_msb(ad, k.tlo7, k.tsmall) & on, 0u, 0xBA98u);
+            }
+            bits[h] = chunk_bits(f[h][0], f[h][1], f[h][2], f[h][3]);
+        }
+        flagged += __popc(bits[0]) + (two ? __popc(bits[1]) : 0);
+        for (uint32_t g = grp; g; g &= g - 1u) {
+            const int u = __ffs(static_cast<int>(g)) - 1;
+            const uint32_t mode = sm.cp->mode[u];
+            const uint32_t c4 = mode == 1u ? sm.cp->vrep[u].c4 : 0u;
+            uint4 *const out = reinterpret_cast<uint4 *>(sm.cp->out[u]) + c;
+            uint16_t *const mk = sm.cp->mask[u] + c;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1 && !two) break;
+                uint32_t o[4];
+                if (mode == 3u) {  // the noise overwrites every flagged sample
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) o[q] = x[h][q];
+                } else if (mode == 2u) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const uint32_t up =
+                            k.unone ? 0u : prmt(ge_bytes_msb(x[h][q] ^ 0x80808080u, k.ulo7, k.usmall), 0u, 0xBA98u);
+                        o[q] = (x[h][q] & ~f[h][q]) | (((k.hi4 & up) | (k.lo4 & ~up)) & f[h][q]);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) o[q] = (x[h][q] & ~f[h][q]) | (c4 & f[h][q]);
+                }
+                __stcs(out + h * T, make_uint4(o[0], o[1], o[2], o[3]));
+                mk[h * T] = static_cast<uint16_t>(bits[h]);
+            }
+        }
+        if (noise) {
+            noise_note8(sm, lane, c, bits[0], nlc);
+            if (two) noise_note8(sm, lane, c + T, bits[1], nlc);
+        }
+    }
+    return flagged;
+}
+
 // ------------------------------------------------------------------ one window
 // All T threads of the group call this. The 12-bit tables must be zero at a group's first window.
 // Uses the group's named barrier after the histogram, after the reduce and after the search. There is no barrier at the end: each warp adds its flag count and marks itself done,
@@ -1632,11 +1710,51 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     }
     if (COPIES) {
         // every variant's values from the window's M and D, then its replace pass
-        if (tid < params_nvar(p)) {
-            const Variant vr = params_var(p)[tid];
-            sm.cp->vrep[tid] = make_rep<BITS, kRepAll>(r.M, r.D, vr.kq, vr.cval);
+        const int nvar = params_nvar(p);
+        if (tid < 32) {
+            bool slow = false;
+            if (tid < nvar) {
+                const Variant vr = params_var(p)[tid];
+                sm.cp->vrep[tid] = make_rep<BITS, kRepAll>(r.M, r.D, vr.kq, vr.cval);
+                if constexpr (BITS == 8) {
+                    const Seg &sv = vsegs[static_cast<int64_t>(tid) * params_seg_stride(p)];
+                    uint32_t grp = 0u;
+                    for (int u = 0; u < nvar; ++u) grp |= params_var(p)[u].kq == vr.kq ? 1u << u : 0u;
+                    sm.cp->group[tid] = grp;
+                    sm.cp->mode[tid] = static_cast<uint32_t>(vr.mode);
+                    sm.cp->out[tid] = sv.out + widx * sv.W;
+                    sm.cp->mask[tid] = reinterpret_cast<uint16_t *>(sv.mask + widx * sv.mask_words);
+                    slow = sv.vec == 0 || sv.mask == nullptr || (w.n & 511) != 0;
+                }
+            }
+            const bool any_slow = __any_sync(0xFFFFFFFFu, slow);
+            if (BITS == 8 && tid == 0) sm.cp->fast = any_slow ? 0u : 1u;
         }
         named_bar(sm.bar_id, T);
+        uint32_t todo = BITS == 8 && sm.cp->fast ? (1u << nvar) - 1u : 0u;
+        const bool grouped = todo != 0u;
+        while (todo) {
+            const int v = __ffs(static_cast<int>(todo)) - 1;
+            const uint32_t grp = sm.cp->group[v];
+            todo &= ~grp;
+            uint32_t noise = 0u;
+            for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.cp->mode[u] == 3u ? 1u << u : 0u;
+            uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
+            uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
+            fv = __reduce_add_sync(0xFFFFFFFFu, fv);
+            if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
+            for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
+                const int u = __ffs(static_cast<int>(m)) - 1;
+                Win wu = w;
+                wu.out = sm.cp->out[u];
+                const uint64_t seed = params_var(p)[u].seed;
+                noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
+                                                 KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,
+                                                 pw);
+            }
+            if (noise && todo) named_bar(sm.bar_id, T);  // the next group lists its own
+        }
+        if (!grouped)
         for (int v = 0; v < params_nvar(p); ++v) {
             const Variant vr = params_var(p)[v];
             const Seg &sv = vsegs[static_cast<int64_t>(v) * params_seg_stride(p)];

@@ -18,9 +18,10 @@
 // read as unsigned) for lane l is word u*32 + l, so the 32 lanes of a warp always hit 32
 // different banks and 32 different words; warps share the table through shared-memory
 // atomics, and the reduce phase reads row u into logical bin u ^ 128 = x + 128. 12-bit
-// samples use 1, 2 or 4 plain copies of a 4096-bin table selected by lane, which spreads
-// same-bin collisions within a warp. One warp searches the cumulative counts for M and D and
-// broadcasts the threshold and replacement values through shared memory.
+// samples use 1, 2 or 4 plain copies of a 4096-bin table selected by lane, of which only the
+// totals of 256 rows of 16 bins are scanned (phase_rows12, phase_search12). One warp searches the
+// cumulative counts for M and D and broadcasts the threshold and replacement values through
+// shared memory.
 //
 // The int8 replace pass works on four samples per 32-bit word: a native byte absolute
 // difference, a three-operation byte compare against t, a byte permute that replicates each
@@ -33,8 +34,9 @@
 // over a half-warp into a per-warp queue of positions, and evaluate Philox whenever 32 are
 // queued, so every lane of a batch has a sample. 12-bit (dense flags): the replace pass writes
 // the flagged samples' positions into a per-group list, and after one more group barrier all
-// threads evaluate Philox for the list; a window whose list would overflow hands the rest of
-// its flagged samples to a per-warp path that numbers them across the warp.
+// threads evaluate Philox for the list, in slices of 8192 samples; a slice whose list would
+// overflow hands the rest of its flagged samples to a per-warp path that numbers them across the
+// warp.
 //
 // Small int8 windows (2^l = 512..8192 samples) can go several to a table (process_tile_multi8):
 // window slot g of a tile is counted by its own group of lanes, so up to eight windows share one
@@ -1156,8 +1158,8 @@ __device__ __forceinline__ void noise_note8(const Shm &sm, int lane, int c, uint
 // lane takes one (two, whose Philox chains interleave) and emit evaluates and stores its noise.
 // Fewer are left for the end. Every lane does Philox work in every batch but the last, however
 // the flags are spread over the chunks, and the chunks are shared out evenly between the warps.
-// PAIR (60 streams of 2^22 samples, noise): 16384-sample windows 260 -> 257 us, 65536 385 -> 357,
-// fp16 output 281 -> 275.
+// PAIR, and no branch per batch for runs across a multiple of 2^32 (60 streams of 2^22 samples,
+// noise): 16384-sample windows 259 -> 252 us, 65536 377 -> 350, fp16 output 281 -> 271.
 template <int T, bool PAIR, class Emit, class Emit2>
 __device__ __forceinline__ void noise_expand8(const Shm &sm, uint32_t n, int tid, Emit &&emit, Emit2 &&emit2) {
     constexpr uint32_t NW = T / 32, B = PAIR ? 64 : 32, RING = 2 * B;

@@ -359,7 +359,6 @@ struct MultiTile {
 };
 
 struct Ctl {
-    uint32_t warp_tot[32];
     RepShared rep;       // threshold and replacement values of the current window
     uint32_t count[2];   // flagged samples, by window parity
     uint32_t done[2];    // warps finished with the window, by window parity
@@ -390,7 +389,7 @@ struct Shm {
     CopyShared *cp;      // digital copy: per-variant state (or null)
     uint16_t *nlist;     // digital noise work area (or null): int8, the entries of the chunks that
                          // hold flagged samples (32-bit); 12-bit, the positions of flagged samples
-    uint32_t *nring;     // int8 digital noise: noise_ring(mode) positions per consumer warp (or null)
+    uint32_t *nring;     // int8 digital noise: kNoiseRingBytes per consumer warp (or null)
     ApplyTile *at;       // apply passes: the current tile's thresholds and counts (or null)
     struct MultiTile *mt;  // 8-bit, one group: state of a multi-window tile (or null)
 };
@@ -409,7 +408,8 @@ constexpr int kNoiseSlice = 1024, kNoiseSliceAny = 1023;
 // kernel and the output formats; in the kernels with multi-window tiles or several variants the
 // registers it takes cost more than the overlap gives.
 __host__ __device__ constexpr bool noise_pairs(int mode) { return (mode & (kModeMulti | kModeAny | kModeApply | kModeCopies | kModePower)) == 0; }
-__host__ __device__ constexpr int noise_ring(int mode) { return noise_pairs(mode) ? 128 : 64; }
+// Bytes of a warp's ring: 128 positions of 16 bits (a window's samples) or 64 of 32 bits.
+constexpr int kNoiseRingBytes = 256;
 
 // Per-thread sums of x^2 and z^2 of the power-metered excision. A thread sees at most
 // 65536 / 128 samples of a window, each below 2^22, so 32 bits hold its sums.
@@ -1162,22 +1162,24 @@ __device__ __forceinline__ void noise_note8(const Shm &sm, int lane, int c, uint
 // noise): 16384-sample windows 259 -> 252 us, 65536 377 -> 350, fp16 output 281 -> 271.
 template <int T, bool PAIR, class Emit, class Emit2>
 __device__ __forceinline__ void noise_expand8(const Shm &sm, uint32_t n, int tid, Emit &&emit, Emit2 &&emit2) {
+    using Pos = typename std::conditional<PAIR, uint16_t, uint32_t>::type;
     constexpr uint32_t NW = T / 32, B = PAIR ? 64 : 32, RING = 2 * B;
+    static_assert(RING * sizeof(Pos) == kNoiseRingBytes, "ring size");
     constexpr uint32_t RM = RING - 1;
     const int lane = tid & 31;
     const uint32_t warp = static_cast<uint32_t>(tid >> 5);
     const uint32_t *list = reinterpret_cast<const uint32_t *>(sm.nlist);
-    uint32_t *ring = sm.nring + warp * RING;
+    Pos *ring = reinterpret_cast<Pos *>(sm.nring) + warp * RING;
     const uint32_t j = static_cast<uint32_t>(lane & 15);
     const uint32_t below = (1u << lane) - 1u;
     uint32_t head = 0u, tail = 0u;  // positions taken / queued so far (tail - head < B between steps)
-    auto at = [&](uint32_t i) { return ring[(head + i + static_cast<uint32_t>(lane)) & RM]; };
+    auto at = [&](uint32_t i) -> uint32_t { return ring[(head + i + static_cast<uint32_t>(lane)) & RM]; };
     for (uint32_t e0 = 2u * warp; e0 < n; e0 += 2u * NW) {
         const uint32_t e = e0 + static_cast<uint32_t>(lane >> 4);
         const uint32_t ent = e < n ? list[e] : 0u;
         const bool fl = ((ent >> j) & 1u) != 0u;
         const uint32_t bal = __ballot_sync(0xFFFFFFFFu, fl);
-        if (fl) ring[(tail + static_cast<uint32_t>(__popc(bal & below))) & RM] = (ent >> 16) * 16u + j;
+        if (fl) ring[(tail + static_cast<uint32_t>(__popc(bal & below))) & RM] = static_cast<Pos>((ent >> 16) * 16u + j);
         tail += static_cast<uint32_t>(__popc(bal));
         if (tail - head >= B) {
             __syncwarp();

@@ -78,13 +78,13 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     const bool noise = ((mode & 3) == 3 || (mode & kModeCopies) != 0) && (mode & kModeStats) == 0;
     L.nlist = noise ? meta_end : 0;
     // int8: a 32-bit entry for every 16-byte chunk of a stage that may hold a flagged sample,
-    // then each consumer warp's ring of noise_ring(mode) 32-bit positions (multi-window tiles keep the
+    // then each consumer warp's ring of positions (multi-window tiles keep the
     // rings in their cumulative-count area, which is idle by then and large enough); 12-bit: the
     // position list
     // (any-window tiles: a chunk that two windows share has an entry for each)
     const int list_bytes = align_up(stage_bytes / 4 > 128 ? stage_bytes / 4 : 128, 128) + ((mode & kModeAny) ? 128 : 0);
-    const int ring_bytes = multi ? 0 : cw * noise_ring(mode) * 4;
-    static_assert(noise_ring(kModeMulti) * 4 * 16 <= Geo<8>::kCumWords * 2 * kMultiMax, "rings of 16 warps fit the multi-window counts");
+    const int ring_bytes = multi ? 0 : cw * kNoiseRingBytes;
+    static_assert(kNoiseRingBytes * 16 <= Geo<8>::kCumWords * 2 * kMultiMax, "rings of 16 warps fit the multi-window counts");
     const int noise_bytes = BITS == 8 ? list_bytes + ring_bytes : kNoiseList * 2;
     L.nring = (noise && BITS == 8) ? (multi ? L.cum : meta_end + list_bytes) : 0;
     const int list_end = noise ? align_up(meta_end + noise_bytes, 128) : meta_end;

@@ -1747,6 +1747,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
             fv = __reduce_add_sync(0xFFFFFFFFu, fv);
             if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
+            __syncwarp();  // lane 0 announces the window for every lane that counted
             for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
                 const int u = __ffs(static_cast<int>(m)) - 1;
                 Win wu = w;

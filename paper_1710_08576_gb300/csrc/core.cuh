@@ -1605,6 +1605,13 @@ __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, in
             if (two) noise_note8(sm, lane, c + T, bits[1], nlc);
         }
     }
+    // mask pieces past the window's last sample (a short last window of whole rounds)
+    if (nchunks < 2 * w.mask_words) {
+        for (uint32_t g = grp; g; g &= g - 1u) {
+            uint16_t *const mk = sm.cp->mask[__ffs(static_cast<int>(g)) - 1];
+            for (int c = nchunks + tid; c < 2 * w.mask_words; c += T) mk[c] = 0;
+        }
+    }
     return flagged;
 }
 

@@ -1,6 +1,9 @@
-"""Digital copies, window by window: the counts of every variant over many windows."""
+"""Digital copies, window by window: the counts of every variant over many windows, and the mask of a
+short last window."""
+import numpy as np
 import pytest
 
+import oracle
 import synth
 
 pytestmark = pytest.mark.gpu
@@ -34,5 +37,28 @@ def test_every_variant_counts_every_window(cuda, rfi):
             for v in range(len(variants)):
                 assert torch.equal(counts[v][0].to(torch.int64), _popcounts(masks[v][0], nwin)), (call, v)
             assert totals.flagged == sum(int(c[0].sum()) for c in counts)
+    finally:
+        plan.close()
+
+
+@pytest.mark.parametrize("W,tail", [(16384, 512), (16384, 15872), (4096, 2048), (1000, 512), (560, 512)])
+def test_mask_ends_with_zeros_after_a_short_last_window(cuda, rfi, W, tail):
+    """The last window holds a multiple of 512 samples and less than W: its mask words past the last
+    sample are written as 0 for every variant, whatever the buffer held."""
+    import torch
+    variants = [(3.0, 0, 0, 0), (3.0, 3, 0, 7), (5.0, 2, 0, 0), (3.0, 1, 9, 0)]
+    n = 3 * W + tail
+    p = synth.params(seed=11, sigma=16.0, burst_rate=1e-2, burst_len_max=64, bits=8)
+    x = synth.fill(p, 0, n)
+    plan = rfi.CopiesPlan(8, [n], [W], variants)
+    try:
+        xd = torch.from_numpy(x).cuda()
+        outs = [[torch.empty_like(xd)] for _ in variants]
+        masks = [[torch.full((plan.mask_words(0),), -1, dtype=torch.int32, device="cuda")] for _ in variants]
+        plan.excise([xd], outs, masks)
+        for v, (k, mode, const, seed) in enumerate(variants):
+            r = oracle.excise(x, W, k, mode, const=const, seed=seed, stream_id=0)
+            assert np.array_equal(masks[v][0].cpu().numpy().view(np.uint32), r["mask"]), v
+            assert np.array_equal(outs[v][0].cpu().numpy(), r["z"]), v
     finally:
         plan.close()

@@ -1742,32 +1742,32 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             if (BITS == 8 && tid == 0) sm.cp->fast = any_slow ? 0u : 1u;
         }
         named_bar(sm.bar_id, T);
-        uint32_t todo = BITS == 8 && sm.cp->fast ? (1u << nvar) - 1u : 0u;
-        const bool grouped = todo != 0u;
-        while (todo) {
+        const bool fast = BITS == 8 && sm.cp->fast;
+        for (uint32_t todo = (1u << nvar) - 1u; todo;) {
             const int v = __ffs(static_cast<int>(todo)) - 1;
-            const uint32_t grp = sm.cp->group[v];
+            const uint32_t grp = fast ? sm.cp->group[v] : 1u << v;
             todo &= ~grp;
-            uint32_t noise = 0u;
-            for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.cp->mode[u] == 3u ? 1u << u : 0u;
             uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
-            uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
-            fv = __reduce_add_sync(0xFFFFFFFFu, fv);
-            if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
-            __syncwarp();  // lane 0 announces the window for every lane that counted
-            for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
-                const int u = __ffs(static_cast<int>(m)) - 1;
-                Win wu = w;
-                wu.out = sm.cp->out[u];
-                const uint64_t seed = params_var(p)[u].seed;
-                noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
-                                                 KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,
-                                                 pw);
+            if (BITS == 8 && (grp & (grp - 1u))) {  // several variants of one multiple
+                uint32_t noise = 0u;
+                for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.cp->mode[u] == 3u ? 1u << u : 0u;
+                uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
+                fv = __reduce_add_sync(0xFFFFFFFFu, fv);
+                if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
+                __syncwarp();  // lane 0 announces the window for every lane that counted
+                for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
+                    const int u = __ffs(static_cast<int>(m)) - 1;
+                    Win wu = w;
+                    wu.out = sm.cp->out[u];
+                    const uint64_t seed = params_var(p)[u].seed;
+                    noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
+                                                     KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,
+                                                     pw);
+                }
+                if (noise && todo) named_bar(sm.bar_id, T);  // the next group lists its own
+                continue;
             }
-            if (noise && todo) named_bar(sm.bar_id, T);  // the next group lists its own
-        }
-        if (!grouped)
-        for (int v = 0; v < params_nvar(p); ++v) {
+            // a variant with a multiple of its own: the pass built for its replacement
             const Variant vr = params_var(p)[v];
             const Seg &sv = vsegs[static_cast<int64_t>(v) * params_seg_stride(p)];
             Win wv = w;
@@ -1776,7 +1776,6 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             wv.vec = sv.vec != 0;
             const Rep rv = load_rep(sm.cp->vrep[v]);
             const KeysSeed vkey{static_cast<uint32_t>(vr.seed), static_cast<uint32_t>(vr.seed >> 32)};
-            uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
             uint32_t fv;
             switch (vr.mode) {
                 case 0: fv = phase_replace<BITS, 0, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]); break;
@@ -1795,7 +1794,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                         noise_deferred8<T, false, false>(sm, wv, rv, vkey, tid, nc, pw);
                     }
                     // the noise work area and the first indices are reused by the next variant
-                    if (v + 1 < params_nvar(p)) named_bar(sm.bar_id, T);
+                    if (todo) named_bar(sm.bar_id, T);
                     break;
             }
             fv = __reduce_add_sync(0xFFFFFFFFu, fv);

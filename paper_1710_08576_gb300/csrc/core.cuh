@@ -1722,12 +1722,15 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     if (COPIES) {
         // every variant's values from the window's M and D, then its replace pass
         const int nvar = params_nvar(p);
+        // only whole rounds with aligned buffers and masks share passes; where the first variant's are not,
+        // warp 0 gathers nothing for it
+        const bool may = BITS == 8 && w.vec && w.mask && (w.n & 511) == 0;
         if (tid < 32) {
-            bool slow = false;
+            bool slow = !may;
             if (tid < nvar) {
                 const Variant vr = params_var(p)[tid];
                 sm.cp->vrep[tid] = make_rep<BITS, kRepAll>(r.M, r.D, vr.kq, vr.cval);
-                if constexpr (BITS == 8) {
+                if (BITS == 8 && may) {
                     const Seg &sv = vsegs[static_cast<int64_t>(tid) * params_seg_stride(p)];
                     uint32_t grp = 0u;
                     for (int u = 0; u < nvar; ++u) grp |= params_var(p)[u].kq == vr.kq ? 1u << u : 0u;
@@ -1735,7 +1738,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                     sm.cp->mode[tid] = static_cast<uint32_t>(vr.mode);
                     sm.cp->out[tid] = sv.out + widx * sv.W;
                     sm.cp->mask[tid] = reinterpret_cast<uint16_t *>(sv.mask + widx * sv.mask_words);
-                    slow = sv.vec == 0 || sv.mask == nullptr || (w.n & 511) != 0;
+                    slow = sv.vec == 0 || sv.mask == nullptr;
                 }
             }
             const bool any_slow = __any_sync(0xFFFFFFFFu, slow);

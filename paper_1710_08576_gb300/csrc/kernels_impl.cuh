@@ -169,8 +169,9 @@ __device__ __forceinline__ Win make_win_any(const Seg &sg, int64_t w, uint32_t w
 // Resident CTAs per SM that the register budget is sized for (0: left to the compiler). One
 // group of 8 + 1 warps runs three CTAs per SM, which its shared memory allows and 72 registers
 // a thread fit; the hint keeps the allocator from cutting registers for a fourth CTA that the
-// shared memory never grants.
-constexpr int min_ctas_per_sm(int cw, int g) { return g != 1 ? 0 : (cw == 8 ? 3 : (cw == 4 ? 4 : 0)); }
+// shared memory never grants. 16 + 1 warps run two CTAs, in 56 registers; without the hint 12-bit
+// noise took 88, which lets one run (60 streams of 2^22 samples: 671 us a call, 449 with it).
+constexpr int min_ctas_per_sm(int cw, int g) { return g != 1 ? 0 : (cw == 8 ? 3 : (cw == 4 ? 4 : 2)); }
 
 // ------------------------------------------------------------------ split-warp consumers
 // The consumer warps of the split-warp form (int8, zero / constant / threshold, also

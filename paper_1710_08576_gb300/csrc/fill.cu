@@ -63,12 +63,14 @@ __global__ void __launch_bounds__(kFillThreads) noise_fill_kernel(const Seg *__r
     const KeysPre key{p};
     int s = 0;
     // the first unit of a warp is its own (spread over the CTAs, so that few units take many SMs),
-    // the others come from the cursor, fetched while the unit before is worked on
+    // the others come from the cursor, fetched while the unit before is worked on. Where every unit
+    // has a warp of its own nobody asks the cursor: thousands of additions to one word at once took 2 us
+    // (2^22 int8 samples, few flagged: 16.7 us a call with them, 14.5 without)
     const uint32_t nwarps = gridDim.x * kFillWarps;
     uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     for (; u < nunits;) {
-        uint32_t next = 0u;
-        if (lane == 0) next = nwarps + atomicAdd(counter, 1u);
+        uint32_t next = nunits;
+        if (nunits > nwarps && lane == 0) next = nwarps + atomicAdd(counter, 1u);
         while (s + 1 < nseg && fwin[s + 1] <= u) ++s;  // a warp's units ascend
         const Seg &g = segs[s];
         const uint32_t W = static_cast<uint32_t>(g.W), mw = static_cast<uint32_t>(g.mask_words);

@@ -34,9 +34,9 @@
 // over a half-warp into a per-warp queue of positions, and evaluate Philox whenever 32 are
 // queued, so every lane of a batch has a sample. 12-bit (dense flags): the replace pass writes
 // the flagged samples' positions into a per-group list, and after one more group barrier all
-// threads evaluate Philox for the list, in slices of 8192 samples; a slice whose list would
-// overflow hands the rest of its flagged samples to a per-warp path that numbers them across the
-// warp.
+// threads evaluate Philox for the list, in slices of 8192 samples where a whole window's flags would
+// not fit; what a list has no room for goes through a per-warp path that numbers the samples across
+// the warp.
 //
 // Small int8 windows (2^l = 512..8192 samples) can go several to a table (process_tile_multi8):
 // window slot g of a tile is counted by its own group of lanes, so up to eight windows share one
@@ -366,7 +366,7 @@ struct Ctl {
     uint32_t ncount[4];  // digital-noise list entries, by window parity (and slice of the window, 12-bit)
     unsigned long long pw[2][2];  // power-metered excision: {sum x^2, sum z^2}, by window parity
     uint32_t abort;      // set when any warp gave up on a bounded wait
-    int32_t pad;
+    int32_t wide;        // 12-bit noise: the window before had few enough flags for one list
     unsigned long long flagged;  // group total
 };
 
@@ -394,11 +394,8 @@ struct Shm {
     struct MultiTile *mt;  // 8-bit, one group: state of a multi-window tile (or null)
 };
 
-// Capacity of the digital-noise work area (16-bit entries: int8 chunk masks of windows up to
-// 65536 samples, or 12-bit flagged positions) and the mark of a list entry that was handed to
-// the per-warp path.
+// Capacity of the 12-bit digital-noise list (16-bit positions in a window of up to 65536 samples).
 constexpr int kNoiseList = 4096;
-constexpr uint16_t kNoiseSkip = 0xFFFFu;
 // 12-bit digital noise goes through a window in slices of this many chunks (8192 samples; in the
 // any-window form 33 rounds of 31 chunks), so that the list serves slices with up to half their samples
 // flagged whatever the window's length.
@@ -1066,12 +1063,11 @@ __device__ __forceinline__ void noise_batch(const Win &w, const Rep &r, const K 
 
 // Digital noise, replace pass (12-bit): the warp numbers its flagged samples of this round, reserves
 // that many list entries with one shared atomic, and each lane writes its positions, counted from
-// the slice's first sample. Rounds that do not fit in the list take the per-warp path at once;
-// list entries reserved beyond the written ones are marked skipped. Called by all lanes of the warp
-// with the flags of samples s0, s0 + 1, ...
+// the window's first sample. Samples beyond the list's end take the per-warp path at once. Called by
+// all lanes of the warp with the flags of samples s0, s0 + 1, ...
 template <int BITS, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const Rep &r, const K &p, int lane,
-                                             int s0, int slice0, uint32_t bits, uint32_t *nlc, Pow &pw) {
+                                             int s0, uint32_t bits, uint32_t *nlc, Pow &pw) {
     if (!__any_sync(0xFFFFFFFFu, bits != 0u)) return;
     const uint32_t cnt = __popc(bits);
     uint32_t inc = cnt;
@@ -1084,31 +1080,32 @@ __device__ __forceinline__ void noise_append(const Shm &sm, const Win &w, const 
     uint32_t base = kNoiseList;
     if (sm.nlist != nullptr && lane == 31) base = atomicAdd(nlc, total);
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
+    uint32_t off = base + inc - cnt;
     if (base + total <= static_cast<uint32_t>(kNoiseList)) {
-        uint32_t off = base + inc - cnt;
         // one predicated store per sample of the chunk: with a quarter of the samples flagged in
         // bursts some lane has all eight, and a loop over the set bits costs more per step (with the
         // noise words shared over a tile, 60 streams of 2^25 samples in 8192-sample windows: 4.54 -> 4.27 ms)
 #pragma unroll
         for (int j = 0; j < Geo<BITS>::kChunkSamples; ++j)
-            if ((bits >> j) & 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 - slice0 + j);
+            if ((bits >> j) & 1u) sm.nlist[off++] = static_cast<uint16_t>(s0 + j);
         return;
     }
-    for (uint32_t i = base + lane; i < static_cast<uint32_t>(kNoiseList); i += 32) sm.nlist[i] = kNoiseSkip;
+    uint32_t beyond = bits;  // what the list has no room for
+    for (; off < static_cast<uint32_t>(kNoiseList) && beyond; beyond &= beyond - 1u)
+        sm.nlist[off++] = static_cast<uint16_t>(s0 + __ffs(static_cast<int>(beyond)) - 1);
     __syncwarp();  // the round's chunk stores come first
-    noise_batch<BITS, PW, K, OUTF>(w, r, p, lane, s0, bits, pw);
+    noise_batch<BITS, PW, K, OUTF>(w, r, p, lane, s0, beyond, pw);
 }
 
 // Digital noise, after the group barrier that follows the replace pass: every thread of the
 // group evaluates Philox for a share of the list and stores the value over the chunk's output.
 template <int BITS, int T, bool PW, class K, int OUTF = 0>
 __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
-                                           int slice0, const uint32_t *nlc, Pow &pw) {
+                                           const uint32_t *nlc, Pow &pw) {
     if (sm.nlist == nullptr) return;
     const uint32_t n = min(*nlc, static_cast<uint32_t>(kNoiseList));
     const NoiseRun<BITS, K> run = w.template noise<BITS>(p);
-    auto put = [&](uint32_t l, uint32_t pos, int32_t z) {
-        if (l == kNoiseSkip) return;
+    auto put = [&](uint32_t pos, int32_t z) {
         store_sample<BITS, OUTF>(w.out, static_cast<int>(pos), z);
         if (PW) pw.z += static_cast<uint32_t>(z * z);
     };
@@ -1119,18 +1116,18 @@ __device__ __forceinline__ void noise_list(const Shm &sm, const Win &w, const Re
         // windows, a quarter of them flagged: 4.60 -> 4.53 ms per call)
         for (; i + T < n; i += 2 * T) {
             const uint32_t la = sm.nlist[i], lb = sm.nlist[i + T];
-            const int2 z = run.value2(slice0 + la, slice0 + lb, r.sig2, r.moff);
-            put(la, slice0 + la, z.x);
-            put(lb, slice0 + lb, z.y);
+            const int2 z = run.value2(la, lb, r.sig2, r.moff);
+            put(la, z.x);
+            put(lb, z.y);
         }
         if (i < n) {
             const uint32_t l = sm.nlist[i];
-            put(l, slice0 + l, run.value(slice0 + l, r.sig2, r.moff));
+            put(l, run.value(l, r.sig2, r.moff));
         }
     } else {  // a window across a multiple of 2^32
         for (; i < n; i += T) {
             const uint32_t l = sm.nlist[i];
-            if (l != kNoiseSkip) put(l, slice0 + l, run.value_any(slice0 + l, r.sig2, r.moff));
+            put(l, run.value_any(l, r.sig2, r.moff));
         }
     }
 }
@@ -1262,7 +1259,7 @@ __device__ __forceinline__ uint32_t sq4(uint32_t w, uint32_t keep) {
 template <int BITS, int MODE, int T, bool PW, class K, int OUTF = 0, bool FO = false, bool PAIR = false>
 __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, const Rep &r, const K &p,
                                                   int tid, uint32_t *nlc, Pow &pw, const RepShared *rsrc,
-                                                  int slice = 0) {
+                                                  int slice = 0, int send = 0) {
     constexpr int BPS = Geo<BITS>::kBps;
     const int lane = tid & 31, warp = tid >> 5;
     const int nbytes = w.n * BPS;
@@ -1357,7 +1354,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
         const int32_t t = r.t;
         const uint32_t hi2 = rsrc->mb4, lo2 = rsrc->tlo7, c2 = MODE == 1 ? rsrc->c4 : 0u;
         const uint32_t h2 = MODE == 2 ? rsrc->hi4 : 0u, l2 = MODE == 2 ? rsrc->lo4 : 0u;
-        const int cend = MODE == 3 ? min(nchunks, slice + kNoiseSlice) : nchunks;  // slice: its first chunk
+        const int cend = MODE == 3 ? min(nchunks, send) : nchunks;  // chunks [slice, send)
         for (int base = slice + warp * 32; base < cend; base += T) {
             const int c = base + lane;
             uint32_t bits = 0;
@@ -1415,7 +1412,7 @@ __device__ __forceinline__ uint32_t phase_replace(const Shm &sm, const Win &w, c
                 }
                 if (mk) mk[c] = static_cast<uint8_t>(bits);
             }
-            if (MODE == 3) noise_append<12, PW, K, OUTF>(sm, w, r, p, lane, c * 8, slice * 8, bits, nlc, pw);
+            if (MODE == 3) noise_append<12, PW, K, OUTF>(sm, w, r, p, lane, c * 8, bits, nlc, pw);
         }
         if (mk && cend == nchunks) {
             for (int c = nchunks + tid; c < 4 * w.mask_words; c += T) mk[c] = 0;
@@ -1497,42 +1494,62 @@ __device__ __forceinline__ void mask_padding(const Win &w, int i, int nt) {
 
 template <int BITS, int MODE, int T, class K>
 __device__ __forceinline__ uint32_t phase_replace_any(const Shm &sm, const Win &w, const Rep &r, const K &p, int tid,
-                                                      uint32_t *nlc, Pow &pw, const RepShared *rsrc, int slice = 0) {
+                                                      uint32_t *nlc, Pow &pw, const RepShared *rsrc, int slice = 0, int send = 0) {
     constexpr int BPS = Geo<BITS>::kBps, CS = Geo<BITS>::kChunkSamples;
     const int lane = tid & 31, warp = tid >> 5;
     const int nch = (w.off + w.n * BPS + 15) >> 4;
-    const int cend = BITS == 12 && MODE == 3 ? min(nch, slice + kNoiseSliceAny) : nch;
+    const int cend = BITS == 12 && MODE == 3 ? min(nch, send) : nch;
     uint32_t flagged = 0;
     for (int base = slice + warp * 31; base < cend; base += (T / 32) * 31) {
         const uint32_t bits = replace_round_any<BITS, MODE>(w, r, rsrc, base, lane);
         flagged += __popc(bits);
         if (MODE == 3) {
             if (BITS == 8) noise_note8(sm, lane, base + lane, bits, nlc);
-            else noise_append<12, false, K>(sm, w, r, p, lane, (base + lane) * CS - w.off / BPS, slice * CS - w.off / BPS,
-                                             bits, nlc, pw);
+            else noise_append<12, false, K>(sm, w, r, p, lane, (base + lane) * CS - w.off / BPS, bits, nlc, pw);
         }
     }
     if (cend == nch) mask_padding<BITS>(w, tid, T);
     return flagged;
 }
 
-// 12-bit digital noise of one window, in slices: replace(counter, first chunk) lists a slice's flagged
-// samples and gives the thread's flag count, list(first sample, counter) evaluates them. nlc: two
-// counters, both zero on entry, used in turn; the one of the slice before is zeroed between the two
-// barriers around a slice's evaluation, when no thread reads it any more.
-template <int T, bool ANY, class Replace, class List>
+// 12-bit digital noise of one window, in slices: replace(counter, chunks from, to) lists their flagged
+// samples and gives the thread's flag count, list(counter) evaluates them. A list per slice leaves
+// lanes of many last batches idle and adds two barriers each; one list for a window whose flags do
+// not fit leaves the rest to the per-warp path. So a window is one slice where the CTA's window before
+// had room in the list for its flags (ctl->wide), and a CTA of one window (ALONE) lets the first slice
+// tell: the others join its list where it promises room (the threads agree through the vote of the
+// barrier). 60 streams of 2^22 samples in 32768-sample windows, 1.6 % and 10 % flagged: always one list 480 and
+// 759 us a call, always slices of 8192 samples 532 and 660, this 456 and 583; 30 of them, one CTA a
+// window, 1.6 %: 555 us in slices, 495 this.
+// nlc: two counters, both zero on entry, used in turn; the one of the list before is zeroed between
+// the two barriers around a list's evaluation, when no thread reads it any more.
+template <int T, bool ANY, bool ALONE, class Replace, class List>
 __device__ __forceinline__ uint32_t noise_slices12(const Shm &sm, const Win &w, uint32_t *nlc, int tid, Replace &&replace,
                                                    List &&list) {
     constexpr int STEP = ANY ? kNoiseSliceAny : kNoiseSlice;
     const int nch = (w.off + 2 * w.n + 15) >> 4;
     uint32_t f = 0;
-    for (int c = 0, k = 0;; c += STEP, k ^= 1) {
-        f += replace(nlc + k, c);
-        named_bar(sm.bar_id, T);  // every flagged position of the slice is in the list
-        if (c + STEP < nch && tid == 0) nlc[k ^ 1] = 0u;
-        list(c * 8 - w.off / 2, nlc + k);
-        if (c + STEP >= nch) return f;
+    int step = STEP;
+    if (!ALONE && nch > STEP && sm.ctl->wide) step = nch;
+    for (int c = 0, k = 0;;) {
+        f += replace(nlc + k, c, c + step);
+        c += step;
+        if (ALONE && c == STEP && c < nch) {
+            // the warp that lists last reads the whole length
+            const uint32_t length = *static_cast<volatile uint32_t *>(nlc + k);
+            const uint32_t slices = static_cast<uint32_t>((nch + STEP - 1) / STEP);
+            if (!named_bar_or(sm.bar_id, T, 8u * slices * length > 7u * kNoiseList)) {
+                step = nch;
+                continue;
+            }
+        } else {
+            named_bar(sm.bar_id, T);  // every flagged position of the list is in it
+        }
+        if (c < nch && tid == 0) nlc[k ^ 1] = 0u;
+        list(nlc + k);
+        if (c >= nch) return f;
         named_bar(sm.bar_id, T);  // the list is free again
+        k ^= 1;
     }
 }
 
@@ -1628,7 +1645,7 @@ __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, in
 // kModeApply skips phases 1-4, reads the window's M from sg.med and its dispersion from sg.mad
 // and runs phase 5 (amd, when given, holds the window's {M, dispersion} in shared memory).
 // kModePower also sums x^2 and z^2 over the window into sg.power.
-template <int BITS, int MODE, int T, int ROWB>
+template <int BITS, int MODE, int T, int ROWB, bool ALONE = false>
 __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64_t widx, const Params &p,
                                int tid, int par, uint32_t release_bar, bool stage_ok, RowSums &rs,
                                const int2 *amd = nullptr, const Seg *vsegs = nullptr) {
@@ -1703,19 +1720,19 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     Pow pw = {0u, 0u};
     const KeysPre key{p};
     // the replace pass, and the digital noise of the samples it listed
-    auto replace = [&](uint32_t *nlc, int slice) {
-        if constexpr (ANY) return phase_replace_any<BITS, RMODE, T, KeysPre>(sm, w, r, key, tid, nlc, pw, &sm.ctl->rep, slice);
+    auto replace = [&](uint32_t *nlc, int slice, int send) {
+        if constexpr (ANY) return phase_replace_any<BITS, RMODE, T, KeysPre>(sm, w, r, key, tid, nlc, pw, &sm.ctl->rep, slice, send);
         else return phase_replace<BITS, RMODE, T, PW, KeysPre, OUTF, (MODE & kModeFlaggedOnly) != 0>(sm, w, r, key, tid, nlc, pw,
-                                                                                                    &sm.ctl->rep, slice);
+                                                                                                    &sm.ctl->rep, slice, send);
     };
     if constexpr (!STATS && !COPIES) {
         uint32_t *const nlc = &sm.ctl->ncount[2 * par];
         if constexpr (BITS == 12 && RMODE == 3) {
-            f = noise_slices12<T, ANY>(sm, w, nlc, tid, replace, [&](int slice0, const uint32_t *c) {
-                noise_list<12, T, PW, KeysPre, OUTF>(sm, w, r, key, tid, slice0, c, pw);
+            f = noise_slices12<T, ANY, ALONE>(sm, w, nlc, tid, replace, [&](const uint32_t *c) {
+                noise_list<12, T, PW, KeysPre, OUTF>(sm, w, r, key, tid, c, pw);
             });
         } else {
-            f = replace(nlc, 0);
+            f = replace(nlc, 0, 0);
             if constexpr (RMODE == 3) noise_deferred8<T, PW, noise_pairs(MODE), KeysPre, OUTF>(sm, w, r, key, tid, nlc, pw);
         }
     }
@@ -1786,12 +1803,12 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                 case 2: fv = phase_replace<BITS, 2, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]); break;
                 default:
                     if constexpr (BITS == 12) {
-                        fv = noise_slices12<T, false>(
+                        fv = noise_slices12<T, false, false>(
                             sm, wv, nc, tid,
-                            [&](uint32_t *c, int slice) {
-                                return phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, c, pw, &sm.cp->vrep[v], slice);
+                            [&](uint32_t *c, int slice, int send) {
+                                return phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, c, pw, &sm.cp->vrep[v], slice, send);
                             },
-                            [&](int slice0, const uint32_t *c) { noise_list<BITS, T, false>(sm, wv, rv, vkey, tid, slice0, c, pw); });
+                            [&](const uint32_t *c) { noise_list<BITS, T, false>(sm, wv, rv, vkey, tid, c, pw); });
                     } else {
                         fv = phase_replace<BITS, 3, T, false>(sm, wv, rv, vkey, tid, nc, pw, &sm.cp->vrep[v]);
                         noise_deferred8<T, false, false>(sm, wv, rv, vkey, tid, nc, pw);
@@ -1826,17 +1843,23 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             sm.ctl->done[par] = 0u;
             if (RMODE == 3 && !COPIES) {  // every warp has read them
                 sm.ctl->ncount[2 * par] = 0u;
-                if (BITS == 12) sm.ctl->ncount[2 * par + 1] = 0u;
+                if (BITS == 12) {
+                    sm.ctl->ncount[2 * par + 1] = 0u;
+                    sm.ctl->wide = 8u * cnt <= 7u * kNoiseList;
+                }
             }
             if (COPIES) {
+                uint32_t most = 0u;
                 for (int v = 0; v < params_nvar(p); ++v) {
                     const uint32_t cv = atomicExch(&sm.cp->vcount[v][par], 0u);
+                    most = cv > most ? cv : most;
                     sm.cp->ncount[4 * v + 2 * par] = 0u;
                     sm.cp->ncount[4 * v + 2 * par + 1] = 0u;
                     const Seg &sv = vsegs[static_cast<int64_t>(v) * params_seg_stride(p)];
                     if (sv.counts) sv.counts[widx] = cv;
                     sm.ctl->flagged += cv;
                 }
+                if (BITS == 12) sm.ctl->wide = 8u * most <= 7u * kNoiseList;
             }
             if (PW) {
                 const unsigned long long sx = atomicExch(&sm.ctl->pw[par][0], 0ull);

@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(CW * 32) stream_kernel(Seg sg, int64_t w_begin
     __syncthreads();
     const Win win = make_win(sg, w, buf, BPS);
     RowSums rs = {{0u, 0u}};
-    process_window<BITS, MODE, T, Geo<BITS>::row_bytes(1)>(sm, win, sg, w, p, tid, 0, 0u, true, rs);
+    process_window<BITS, MODE, T, Geo<BITS>::row_bytes(1), true>(sm, win, sg, w, p, tid, 0, 0u, true, rs);
     __syncthreads();
     if (tid == 0 && sm.ctl->flagged) atomicAdd(p.flagged, sm.ctl->flagged);
 }

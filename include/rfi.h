@@ -143,7 +143,8 @@ typedef struct rfi_launch_shape {
                                 write-flagged, but neither power-metered, nor digital copies, nor
                                 another output format; RFI_ERR_UNSUPPORTED otherwise). 0 = choose: the
                                 autotuner tries both where the split form runs; otherwise 2 where it
-                                runs in plans of many tiles, else 1 */
+                                runs in plans of many tiles, else 1. A plan that took 2 unasked runs
+                                calls on unaligned buffers in the joint form */
 } rfi_launch_shape;
 
 typedef struct rfi_plan_desc {

@@ -151,6 +151,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
         }
         if (hit) {
             P->shape = cached;
+            P->split_by_rule = false;
             rfi_status rs = plan_build_tiles(P);
             return rs == RFI_OK ? plan_alloc_workspace(P) : rs;
         }
@@ -301,6 +302,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
     cudaStreamDestroy(st);
     if (best_ms >= 1e29f) return RFI_ERR_UNSUPPORTED;
     P->shape = best;
+    P->split_by_rule = false;
     {
         std::lock_guard<std::mutex> g(g_cache_mu);
         g_cache[key] = best;

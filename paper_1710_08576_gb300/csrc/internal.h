@@ -181,6 +181,13 @@ inline int shape_mode(int bits, int mode, const Shape &s) {
     return s.warp_split == 2 && warp_split_runs(bits, mode, s) ? (mode | kModeWarpSplit) : mode;
 }
 
+// Whether a call of a plan that took the split-warp form unasked runs the joint form instead: tiles that
+// are not 16-byte aligned are loaded byte by byte by the consumers and stored so, by half the threads
+// in the split form. 60 streams of 2^22 samples, zero, 16384-sample windows: unaligned 1306 us a call
+// joint, 2002 split, aligned 118 and 112; 65536-sample windows 3427, 5766, 123 and 116. So it pays
+// from about a hundredth of the samples on.
+inline bool joint_for_unaligned(uint64_t unaligned, uint64_t total) { return 128 * unaligned > total; }
+
 // Bytes of dynamic shared memory the kernels need.
 size_t persistent_smem_bytes(int bits, int mode, const Shape &s);
 size_t stream_smem_bytes(int bits, int mode, int consumer_warps, int ncopies, int window_bytes);

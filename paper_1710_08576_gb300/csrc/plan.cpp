@@ -41,6 +41,7 @@ namespace rfi {
 
 rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
     Shape s{};
+    P->split_by_rule = false;
     const int bps = P->bits == 8 ? 1 : 2;
     int64_t maxwb = 0;
     bool uniform = true;
@@ -110,8 +111,10 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
         Shape split = s;
         split.warp_split = 2;
         if (persistent_smem_bytes(P->bits, kmode, split) <= 227u * 1024u &&
-            persistent_occupancy(P->bits, kmode, split) >= s.ctas_per_sm)
+            persistent_occupancy(P->bits, kmode, split) >= s.ctas_per_sm) {
             s = split;
+            P->split_by_rule = true;
+        }
     }
     P->shape = s;
     return RFI_OK;
@@ -273,13 +276,16 @@ Params plan_params(const rfi_plan_s *P) {
     return p;
 }
 
-// Enqueue the persistent launch (with its counter reset) on st.
-rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st) {
+// Enqueue the persistent launch (with its counter reset) on st; joint: in the joint form whatever the
+// plan's shape says (it needs less shared memory, so the same CTAs fit).
+rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st, bool joint) {
     RFI_CUDA(cudaMemsetAsync(P->d_ctr, 0, sizeof(DevCounters), st));
     const int inject = (P->flags & RFI_PLAN_INJECT_TIMEOUT) ? 1 : 0;
     if (P->kmom < 2) {
         const Params p = plan_params(P);
-        RFI_CUDA(launch_persistent(P->bits, plan_kernel_mode(P), P->shape, P->grid, P->d_segs, P->d_tiles,
+        Shape s = P->shape;
+        if (joint) s.warp_split = 1;
+        RFI_CUDA(launch_persistent(P->bits, plan_kernel_mode(P), s, P->grid, P->d_segs, P->d_tiles,
                                    P->ntiles, p, &P->d_ctr->tile_counter, inject, st));
         if (P->fill) RFI_CUDA(launch_noise_fill(P->bits, P->d_segs, P->S, P->d_fwin, P->nfwin, P->fill_unit, p, &P->d_ctr->fill_counter,
                                    P->fill_grid, st));
@@ -685,11 +691,17 @@ rfi_status plan_run_batched(rfi_plan_s *P, const std::vector<Seg> &segs, cudaStr
     } else {
         P->last_seg_writes = 0;
     }
-    if (P->gexec) {
+    bool joint = false;
+    if (P->split_by_rule) {
+        uint64_t unaligned = 0;
+        for (int i = 0; i < P->S; ++i) unaligned += segs[i].vec ? 0 : static_cast<uint64_t>(segs[i].len);
+        joint = joint_for_unaligned(unaligned, P->total_samples);
+    }
+    if (P->gexec && !joint) {
         RFI_CUDA(cudaGraphLaunch(P->gexec, st));
         return RFI_OK;
     }
-    return plan_enqueue_batched(P, st);
+    return plan_enqueue_batched(P, st, joint);
 }
 
 }  // namespace rfi

@@ -41,6 +41,7 @@ struct rfi_plan_s {
     int device = 0, sm_count = 0;
     rfi::Shape shape{};
     bool given_stage = false;  // the caller's shape gives the stage size
+    bool split_by_rule = false;  // the split-warp form was neither asked for nor tuned
     std::vector<rfi::Tile> tiles_host;
     int ntiles = 0, grid = 0;
     int grid_apply = 0;  // Median of MAD: grid of the apply pass (no histogram: more CTAs fit)
@@ -101,7 +102,7 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req);
 bool plan_warp_split_runs(const rfi_plan_s *P, const Shape &s);
 rfi_status plan_build_tiles(rfi_plan_s *P);
 rfi_status plan_alloc_workspace(rfi_plan_s *P);
-rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st);
+rfi_status plan_enqueue_batched(rfi_plan_s *P, cudaStream_t st, bool joint = false);
 rfi_status plan_build_graph(rfi_plan_s *P);
 rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req);
 void plan_release_host_pipe(rfi_plan_s *P);

@@ -50,7 +50,7 @@ constexpr int kModeWarpSplit = 1024;
 // rounded out to 16-byte chunks, and the window phases take windows that start and end anywhere in
 // a chunk; several 8-bit windows of up to kMultiMaxWindow samples of any length share a histogram
 // table as in the multi-window form. For plans with windows that the aligned forms serve badly
-// (needs_any_form). 24 int8 streams of 2^18..2^22 samples in windows of 1000..40000, threshold: 200 -> 65
+// (any_form_gain). 24 int8 streams of 2^18..2^22 samples in windows of 1000..40000, threshold: 200 -> 65
 // us a call (host included); 24 x 2466361 int8 samples in 2000-sample windows: 126 -> 77 us; 1.04 G
 // 12-bit samples in 829-sample windows, noise: 28.8 -> 14.7 ms.
 constexpr int kModeAny = 2048;
@@ -60,14 +60,26 @@ constexpr int kMultiMaxWindow = 8192;  // largest window that shares a table (16
 inline bool multi_window(int bits, int32_t W) {
     return bits == 8 && W >= 512 && W <= kMultiMaxWindow && (W & (W - 1)) == 0;
 }
-// Whether the aligned forms serve a stream of windows W badly: windows whose bytes are no multiple
-// of 16 are loaded byte by byte by the consumers with no copy in flight and stored byte by byte,
-// one window a tile; int8 windows of up to 8192 samples that are no power of two go one at a time
-// through the histogram's reduce and the barriers.
-inline bool needs_any_form(int bits, int32_t W, int64_t len) {
+// What the any-window form saves on a sample of a stream of windows W, in us per call of 60 x 2^22 samples
+// (negative: what it costs). noise: digital noise in the excision kernel; mom: Median of MAD.
+//  - Windows whose bytes are no multiple of 16 are loaded byte by byte by the aligned forms' consumers with
+//    no copy in flight and stored byte by byte, one window a tile (int8, noise: 1001 samples 2112 aligned, 445
+//    any; 8001: 1476, 296; 50001: 3392, 262; 12-bit 1001: 3096, 1291; Median of MAD 1001: 2582, 758).
+//  - Other int8 windows of up to 8192 samples that are no power of two go one at a time through the
+//    histogram's reduce and the barriers there (zero: 528 samples 1326 and 553, 1600: 468 and 315, 3200: 279
+//    and 238, 4000: 233 and 221, 4800: 205 and 228, 8000: 152 and 239; noise: 528 samples 2133 and 657, 4800: 329
+//    and 277, 8000: 231 and 287; Median of MAD 1600: 622 and 480, 4000: 300 and 281, 4800: 282 and 275).
+//  - Windows of the multi-window form lose its fixed layout (zero: 512 samples 380 and 531, 2048: 166 and 257,
+//    4096: 154 and 250; Median of MAD: 411 and 1121, -, 179 and 285), the rest a lane in 32 and the
+//    stages' tighter fit (zero, 16384 samples: 118 and 142; 65536: 123 and 171; 12-bit 16384: 267 and 297;
+//    Median of MAD 16384: 173 and 187).
+inline int64_t any_form_gain(int bits, bool noise, bool mom, int32_t W, int64_t len) {
     const int bps = bits == 8 ? 1 : 2;
-    if (static_cast<int64_t>(W) * bps % 16 != 0) return len > 16;
-    return bits == 8 && W <= kMultiMaxWindow && !multi_window(bits, W) && len >= 2 * static_cast<int64_t>(W);
+    if (static_cast<int64_t>(W) * bps % 16 != 0) return len <= 16 ? 0 : (mom ? 1800 : 1200);
+    if (bits != 8) return -50;
+    if (W > kMultiMaxWindow || len < 2 * static_cast<int64_t>(W)) return mom ? -15 : -40;
+    if (multi_window(bits, W)) return mom ? -30 - 350000 / W : -100 - 25000 / W;
+    return noise ? 860000 / W - 150 : 480000 / W - (mom ? 95 : 117);
 }
 // Windows per tile of a stage: as many whole ones as fit (the any-window form keeps 16 bytes for
 // the tile's distance to the 16-byte boundary before it).

@@ -514,17 +514,14 @@ static rfi_status plan_create(const rfi_plan_desc *d, int32_t nvar, const rfi_va
         for (int i = 0; i < P->S && !P->multi; ++i)
             P->multi = multi_window(P->bits, P->W[i]) && P->len[i] >= 2 * static_cast<int64_t>(P->W[i]);
         // windows that the aligned forms serve badly: the any-window form (built for one group of 8
-        // consumer warps), where they are enough of the plan: it takes their byte-wise loads from
-        // about 8 to 1 times an aligned window's time and the small ones from 1.6 to 1, and costs the
-        // plan's other windows up to a tenth (31 of 32 lanes own a chunk; no split-warp form)
+        // consumer warps), where what it saves on them is more than it costs on the plan's others
         const rfi_launch_shape *q = d->shape;
         if (!q || ((q->consumer_warps == 0 || q->consumer_warps == 8) && q->groups <= 1 && q->warp_split <= 1)) {
-            uint64_t bytewise = 0, small = 0;
-            for (int i = 0; i < P->S; ++i) {
-                if (!needs_any_form(P->bits, P->W[i], P->len[i])) continue;
-                (static_cast<int64_t>(P->W[i]) * (P->bits == 8 ? 1 : 2) % 16 ? bytewise : small) += P->len[i];
-            }
-            P->any = 70 * bytewise + 7 * small > total_s;
+            double gain = 0.0;
+            for (int i = 0; i < P->S; ++i)
+                gain += static_cast<double>(P->len[i]) * static_cast<double>(any_form_gain(
+                            P->bits, P->mode == RFI_REPLACE_NOISE && !P->fill, P->kmom >= 2, P->W[i], P->len[i]));
+            P->any = gain > 0.0;
         }
     }
 

@@ -59,7 +59,7 @@ struct rfi_plan_s {
     bool power = false;
     // some stream has windows of 2^l samples, 512 <= 2^l <= 8192: the multi-window form
     bool multi = false;
-    // windows that the aligned forms serve badly: the any-window form (needs_any_form)
+    // windows that the aligned forms serve badly: the any-window form (any_form_gain)
     bool any = false;
     // RFI_PLAN_WRITE_FLAGGED: in place, only changed chunks are stored
     bool write_flagged = false;

@@ -1,0 +1,40 @@
+"""The rules that choose a plan's kernel form, called on the host: a small program is compiled against
+the library's internal header and prints their answers."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1710_08576_gb300", "csrc")
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+
+def answers(tmp_path, body):
+    """The integers that a program with the given main body prints."""
+    src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
+    src.write_text('#include <cstdio>\n#include <cuda_runtime.h>\n#include "internal.h"\nusing namespace rfi;\n'
+                   "int main() {\n" + body + "\nreturn 0;\n}\n")
+    subprocess.check_call(["g++", "-std=c++17", "-I" + CSRC, "-I" + os.path.join(ROOT, "include"),
+                           "-I" + os.path.join(CUDA, "include"), str(src), "-o", str(exe)])
+    return [int(v) for v in subprocess.check_output([str(exe)], text=True).split()]
+
+
+PLANS = [  # (bits, noise, mom, [(streams, window)], whether the any-window form is the faster one)
+    (8, 0, 0, [(60, 1001)], True), (8, 1, 0, [(60, 50001)], True), (12, 1, 0, [(60, 1001)], True),
+    (8, 0, 0, [(60, 1600)], True), (8, 0, 0, [(60, 3200)], True), (8, 0, 0, [(60, 4000)], True), (8, 0, 0, [(60, 4800)], False), (8, 0, 0, [(60, 8000)], False),
+    (8, 1, 0, [(60, 4800)], True), (8, 1, 0, [(60, 8000)], False), (8, 0, 0, [(60, 10000)], False),
+    (8, 0, 0, [(60, 4096)], False), (8, 0, 0, [(60, 16384)], False), (12, 0, 0, [(60, 1600)], False),
+    (8, 0, 0, [(10, 3200), (50, 4096)], False), (8, 0, 0, [(10, 3200), (50, 16384)], False),
+    (8, 0, 0, [(8, 1000), (52, 16384)], True), (8, 0, 0, [(1, 16385), (59, 16384)], False),
+    (8, 0, 1, [(10, 1600), (50, 512)], False), (8, 0, 1, [(60, 1600)], True), (8, 0, 1, [(60, 4800)], True), (8, 0, 1, [(60, 8000)], False),
+    (8, 0, 1, [(4, 1001), (56, 4096)], True), (8, 0, 1, [(4, 1001), (56, 16384)], True),
+]
+
+
+@pytest.mark.parametrize("i", range(len(PLANS)))
+def test_the_any_window_form_where_it_is_the_faster_one(tmp_path, i):
+    bits, noise, mom, streams, want = PLANS[i]
+    gains = answers(tmp_path, "".join('printf("%%lld\\n", (long long)any_form_gain(%d, %d, %d, %d, 1 << 22));' %
+                                      (bits, noise, mom, W) for _, W in streams))
+    assert (sum(n * g for (n, _), g in zip(streams, gains)) > 0) == want, gains

@@ -580,12 +580,22 @@ static rfi_status plan_create(const rfi_plan_desc *d, int32_t nvar, const rfi_va
             return RFI_OK;
         }
     }
-    rs = plan_choose_shape(P, d->shape);
-    if (rs == RFI_OK) rs = plan_build_tiles(P);
-    if (rs == RFI_OK) rs = plan_alloc_workspace(P);
-    if (rs == RFI_OK && (P->flags & RFI_PLAN_AUTOTUNE) && !(P->flags & RFI_PLAN_PER_STREAM) && P->kmom < 2 &&
-        !P->power && P->ncopy == 0 && P->out_format == RFI_OUT_SAME)
-        rs = plan_autotune(P, d->shape);
+    auto prepare = [&] {
+        rfi_status s = plan_choose_shape(P, d->shape);
+        if (s == RFI_OK) s = plan_build_tiles(P);
+        if (s == RFI_OK) s = plan_alloc_workspace(P);
+        if (s == RFI_OK && (P->flags & RFI_PLAN_AUTOTUNE) && !(P->flags & RFI_PLAN_PER_STREAM) && P->kmom < 2 &&
+            !P->power && P->ncopy == 0 && P->out_format == RFI_OUT_SAME)
+            s = plan_autotune(P, d->shape);
+        return s;
+    };
+    rs = prepare();
+    if (rs == RFI_ERR_UNSUPPORTED && P->any) {
+        // the any-window form takes 3.7 KB more shared memory and other stage sizes: a shape that it cannot
+        // run may fit the aligned forms
+        P->any = false;
+        rs = prepare();
+    }
     if (rs == RFI_OK && (P->flags & RFI_PLAN_GRAPH)) rs = plan_build_graph(P);
     if (rs != RFI_OK) {
         rfi_plan_destroy(P);

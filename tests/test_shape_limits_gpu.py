@@ -1,0 +1,31 @@
+"""Explicit launch shapes close to the shared memory of an SM, against the CPU oracle, bit for bit: the plans
+that fit in one form of a kernel and not in another."""
+import pytest
+
+import synth
+
+from .parity import assert_same, gpu_run, oracle_run
+
+pytestmark = pytest.mark.gpu
+
+
+def _streams(bits, lens):
+    p = synth.params(seed=21, sigma=16.0 if bits == 8 else 120.0, burst_rate=5e-3, burst_len_max=64, bits=bits)
+    return [synth.fill(p, s, n) for s, n in enumerate(lens)]
+
+
+@pytest.mark.parametrize("bits,W,mode,flags,shape", [
+    (8, 65001, 0, 0, dict(stages=3)), (8, 48500, 2, 0, dict(stages=4)), (8, 59501, 3, 0, dict(stages=3)),
+    (8, 24570, 0, 0, dict(stages=8)), (12, 31613, 3, 0, dict(stages=3)),
+    (8, 3200, 0, "tune", dict(stage_bytes=6400)), (8, 3200, 3, "tune", dict(stage_bytes=12800, stages=2)),
+])
+def test_odd_windows_in_shapes_that_only_the_aligned_form_fits(cuda, rfi, bits, W, mode, flags, shape):
+    """Windows that the any-window form would serve, in shapes that it has no room or no stage size for."""
+    lens = [W * 3 + 77, W * 2]
+    xs = _streams(bits, lens)
+    ref = oracle_run(xs, [W] * 2, bits, 3.0, mode, 0, 5)
+    got, st, _, info = gpu_run(rfi, xs, [W] * 2, bits, 3.0, mode, 0, 5, flags=rfi.RFI_PLAN_AUTOTUNE if flags else 0, shape=shape)
+    assert st == 0
+    assert_same(got, ref)
+    for field, v in shape.items():
+        assert getattr(info.shape, field) == v

@@ -333,13 +333,19 @@ struct CopyShared {
     RepShared vrep[kMaxCopies];        // threshold and replacement values per variant
     uint32_t vcount[kMaxCopies][2];    // flagged samples, by variant and window parity
     uint32_t ncount[4 * kMaxCopies];   // digital-noise list entries, by variant, parity and slice
-    // int8: what the variants of one threshold multiple share a pass with (copies_pass8)
+};
+
+// Digital copy, int8: what the variants of one threshold multiple share a pass with (copies_pass8). It lies
+// over the cumulative counts, which are idle from the search to the next window's reduce, so that
+// copies take no more shared memory for it.
+struct CopyPass {
     uint8_t *out[kMaxCopies];          // the window's output and mask, by variant
     uint16_t *mask[kMaxCopies];
     uint32_t group[kMaxCopies];        // bit u: variant u has the same multiple
     uint32_t mode[kMaxCopies];         // rfi_mode
     uint32_t fast;                     // the window goes through copies_pass8
 };
+static_assert(sizeof(CopyPass) <= 256 * 4, "over the cumulative counts");
 
 // Apply passes over whole tiles: the thresholds and flag counts of the tile's windows.
 struct ApplyTile {
@@ -387,6 +393,7 @@ struct Shm {
     int ncopies;         // 12-bit only
     int bar_id;          // named barrier of this consumer group
     CopyShared *cp;      // digital copy: per-variant state (or null)
+    CopyPass *pass;      // digital copy, int8: the state of shared passes (or null)
     uint16_t *nlist;     // digital noise work area (or null): int8, the entries of the chunks that
                          // hold flagged samples (32-bit); 12-bit, the positions of flagged samples
     uint32_t *nring;     // int8 digital noise: kNoiseRingBytes per consumer warp (or null)
@@ -1591,10 +1598,10 @@ __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, in
         flagged += __popc(bits[0]) + (two ? __popc(bits[1]) : 0);
         for (uint32_t g = grp; g; g &= g - 1u) {
             const int u = __ffs(static_cast<int>(g)) - 1;
-            const uint32_t mode = sm.cp->mode[u];
+            const uint32_t mode = sm.pass->mode[u];
             const uint32_t c4 = mode == 1u ? sm.cp->vrep[u].c4 : 0u;
-            uint4 *const out = reinterpret_cast<uint4 *>(sm.cp->out[u]) + c;
-            uint16_t *const mk = sm.cp->mask[u] + c;
+            uint4 *const out = reinterpret_cast<uint4 *>(sm.pass->out[u]) + c;
+            uint16_t *const mk = sm.pass->mask[u] + c;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (h == 1 && !two) break;
@@ -1625,7 +1632,7 @@ __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, in
     // mask pieces past the window's last sample (a short last window of whole rounds)
     if (nchunks < 2 * w.mask_words) {
         for (uint32_t g = grp; g; g &= g - 1u) {
-            uint16_t *const mk = sm.cp->mask[__ffs(static_cast<int>(g)) - 1];
+            uint16_t *const mk = sm.pass->mask[__ffs(static_cast<int>(g)) - 1];
             for (int c = nchunks + tid; c < 2 * w.mask_words; c += T) mk[c] = 0;
         }
     }
@@ -1751,26 +1758,26 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                     const Seg &sv = vsegs[static_cast<int64_t>(tid) * params_seg_stride(p)];
                     uint32_t grp = 0u;
                     for (int u = 0; u < nvar; ++u) grp |= params_var(p)[u].kq == vr.kq ? 1u << u : 0u;
-                    sm.cp->group[tid] = grp;
-                    sm.cp->mode[tid] = static_cast<uint32_t>(vr.mode);
-                    sm.cp->out[tid] = sv.out + widx * sv.W;
-                    sm.cp->mask[tid] = reinterpret_cast<uint16_t *>(sv.mask + widx * sv.mask_words);
+                    sm.pass->group[tid] = grp;
+                    sm.pass->mode[tid] = static_cast<uint32_t>(vr.mode);
+                    sm.pass->out[tid] = sv.out + widx * sv.W;
+                    sm.pass->mask[tid] = reinterpret_cast<uint16_t *>(sv.mask + widx * sv.mask_words);
                     slow = sv.vec == 0 || sv.mask == nullptr;
                 }
             }
             const bool any_slow = __any_sync(0xFFFFFFFFu, slow);
-            if (BITS == 8 && tid == 0) sm.cp->fast = any_slow ? 0u : 1u;
+            if (BITS == 8 && tid == 0) sm.pass->fast = any_slow ? 0u : 1u;
         }
         named_bar(sm.bar_id, T);
-        const bool fast = BITS == 8 && sm.cp->fast;
+        const bool fast = BITS == 8 && sm.pass->fast;
         for (uint32_t todo = (1u << nvar) - 1u; todo;) {
             const int v = __ffs(static_cast<int>(todo)) - 1;
-            const uint32_t grp = fast ? sm.cp->group[v] : 1u << v;
+            const uint32_t grp = fast ? sm.pass->group[v] : 1u << v;
             todo &= ~grp;
             uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
             if (BITS == 8 && (grp & (grp - 1u))) {  // several variants of one multiple
                 uint32_t noise = 0u;
-                for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.cp->mode[u] == 3u ? 1u << u : 0u;
+                for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.pass->mode[u] == 3u ? 1u << u : 0u;
                 uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
                 fv = __reduce_add_sync(0xFFFFFFFFu, fv);
                 if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
@@ -1778,7 +1785,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                 for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
                     const int u = __ffs(static_cast<int>(m)) - 1;
                     Win wu = w;
-                    wu.out = sm.cp->out[u];
+                    wu.out = sm.pass->out[u];
                     const uint64_t seed = params_var(p)[u].seed;
                     noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
                                                      KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,

@@ -123,6 +123,7 @@ __device__ __forceinline__ Shm group_view(uint8_t *smem, const Layout &L, int g,
     sm.nlist = L.nlist ? reinterpret_cast<uint16_t *>(gb + L.nlist) : nullptr;
     sm.nring = L.nlist && BITS == 8 ? reinterpret_cast<uint32_t *>(gb + L.nring) : nullptr;
     sm.cp = L.cps ? reinterpret_cast<CopyShared *>(gb + L.cps) : nullptr;
+    sm.pass = L.cps && BITS == 8 ? reinterpret_cast<CopyPass *>(gb + L.cum) : nullptr;
     sm.at = L.atile ? reinterpret_cast<ApplyTile *>(gb + L.atile) : nullptr;
     sm.mt = L.mt ? reinterpret_cast<MultiTile *>(gb + L.mt) : nullptr;
     return sm;

@@ -29,3 +29,26 @@ def test_odd_windows_in_shapes_that_only_the_aligned_form_fits(cuda, rfi, bits, 
     assert_same(got, ref)
     for field, v in shape.items():
         assert getattr(info.shape, field) == v
+
+
+@pytest.mark.parametrize("bits,W,shape", [(8, 59648, dict(stages=3)), (8, 26752, dict(stages=7)), (12, 31488, dict(stages=3, hist_copies=1)),
+                                          (12, 23296, dict(stages=3, hist_copies=4))])
+def test_copies_in_the_largest_stages_that_fit(cuda, rfi, bits, W, shape):
+    """Digital copies whose window fills the largest stage of that number: as with the default shape."""
+    import torch
+    variants = [(3.0, 0, 0, 0), (3.0, 3, 0, 7), (4.0, 2, 0, 0), (3.0, 1, 5, 0)]
+    lens = [W * 4, W * 2 + 512]
+    xs = [torch.from_numpy(x).cuda() for x in _streams(bits, lens)]
+    res = []
+    for s in (shape, None):
+        plan = rfi.CopiesPlan(bits, lens, [W] * 2, variants, shape=s)
+        try:
+            outs = [[torch.empty_like(x) for x in xs] for _ in variants]
+            masks = [[torch.full((plan.mask_words(i),), -1, dtype=torch.int32, device="cuda") for i in range(2)] for _ in variants]
+            for _ in range(2):
+                plan.excise(xs, outs, masks)
+            assert plan.stats()[0] == 0 and (s is None or plan.info().shape.stages == s["stages"])
+            res.append((sum(outs, []), sum(masks, [])))
+        finally:
+            plan.close()
+    assert all(torch.equal(a, b) for k in range(2) for a, b in zip(res[0][k], res[1][k]))

@@ -388,7 +388,7 @@ struct Shm {
     uint32_t hist_s;     // histogram (shared address)
     uint32_t grp;        // 8-bit: byte offset of this group's half row (0 or 128)
     uint32_t *cum;       // cumulative counts; 12-bit: the histogram's second table (table12)
-    uint32_t *coarse;    // 12-bit estimation pass: the rows' cumulative counts (or null: see rows12)
+    uint32_t *coarse;    // 12-bit estimation pass: the rows' cumulative counts (or null: phase_rows12)
     Ctl *ctl;
     int ncopies;         // 12-bit only
     int bar_id;          // named barrier of this consumer group
@@ -652,7 +652,7 @@ __device__ __forceinline__ int scan256_warp(uint32_t *cum, uint32_t half, int la
 // to scan as the 256 counts of an 8-bit window; the copies are folded into copy 0 on the way. The
 // table of the window before is cleared. coarse is the first kCoarse words of that table (its words
 // are zeroed by the search, search12) or, in the estimation pass, whose other warps go on to the
-// next window's histogram during the search, a region of its own. Eight lanes of a row's
+// next window's histogram during the search, a region of its own (kModeTight: none). Eight lanes of a row's
 // 16-byte read touch all banks (the pieces are taken in an order rotated by row pairs).
 // A full scan of the 4096 bins, which this replaces, took the group two more passes over the
 // table, a block-wide offset exchange and a fourth barrier: about 1400 instructions of its warps per
@@ -1664,6 +1664,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     constexpr int OUTF = (MODE & kModeF16) ? 1 : ((MODE & kModeBF16) ? 2 : 0);
     constexpr int RMODE = MODE & 3;
     constexpr bool ANY = (MODE & kModeAny) != 0;
+    constexpr bool TIGHT = (MODE & kModeTight) != 0;
     const int lane = tid & 31;
     if (STATS) {
         // Estimation only (the first pass of Eq. 3): M and D of the window. Nothing reads the
@@ -1681,13 +1682,14 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
         // int8: the counts go to one warp, which scans them and searches while the other warps
         // start the next window (one group barrier fewer than a block-wide scan)
         if constexpr (BITS == 8) phase_reduce8_counts<T, ROWB>(sm, tid, rs);
-        else phase_rows12<T>(sm, tid, par, sm.coarse);
+        else phase_rows12<T>(sm, tid, par, TIGHT ? table12(sm, par ^ 1) : sm.coarse);
         named_bar(sm.bar_id, T);
         if (tid < 32) {
             if constexpr (BITS == 8) {
                 phase_search8<MODE>(sm, w.n, lane, p.kq, p.cval);
             } else {
-                phase_search12<MODE>(sm, table12(sm, par), sm.coarse, false, w.n, lane, p.kq, p.cval);
+                phase_search12<MODE>(sm, table12(sm, par), TIGHT ? table12(sm, par ^ 1) : sm.coarse, TIGHT, w.n, lane, p.kq,
+                                     p.cval);
             }
             if (lane == 0) {  // the lane that wrote the record
                 if (med) med[widx] = sm.ctl->rep.M;
@@ -1695,6 +1697,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                 if (BITS == 12 && atomicExch(&sm.ctl->err[par], 0u)) atomicOr(p.status, kStatusSampleRange);
             }
         }
+        if (TIGHT) named_bar(sm.bar_id, T);  // the search worked in the next window's table
         return true;
     }
     if (!APPLY) {

@@ -60,6 +60,11 @@ constexpr int kMultiMaxWindow = 8192;  // largest window that shares a table (16
 inline bool multi_window(int bits, int32_t W) {
     return bits == 8 && W >= 512 && W <= kMultiMaxWindow && (W & (W - 1)) == 0;
 }
+// Flag bit of the 12-bit estimation pass in shapes that leave no room for the rows' counts (fit_mode): they
+// lie over the idle table, and the other warps wait for the search. Its own instantiation: as a
+// branch of the usual one it cost that 2 % (1024-sample windows 1229 -> 1260 us a call).
+constexpr int kModeTight = 4096;
+
 // What the any-window form saves on a sample of a stream of windows W, in us per call of 60 x 2^22 samples
 // (negative: what it costs). noise: digital noise in the excision kernel; mom: Median of MAD.
 //  - Windows whose bytes are no multiple of 16 are loaded byte by byte by the aligned forms' consumers with

@@ -35,8 +35,18 @@ cudaError_t launch_mom_b12(const MomChunk *, int, const int32_t *, int32_t *, in
 cudaError_t launch_stream_b8(int, int, const Seg &, int64_t, int64_t, const Params &, cudaStream_t);
 cudaError_t launch_stream_b12(int, int, const Seg &, int64_t, int64_t, const Params &, cudaStream_t);
 
-size_t persistent_smem_bytes(int bits, int mode, const Shape &s) {
+// The mode that a launch of this shape runs: that of shape_mode, in the tight form where the estimation pass
+// does not fit a CTA's shared memory otherwise.
+static int fit_mode(int bits, int mode, const Shape &s) {
     mode = shape_mode(bits, mode, s);
+    if (bits == 12 && (mode & kModeStats) && !(mode & kModeAny) &&
+        dev::layout<12>(s.hist_copies, s.stages, s.stage_bytes, s.consumer_warps, s.groups, mode).total > 227 * 1024)
+        mode |= kModeTight;
+    return mode;
+}
+
+size_t persistent_smem_bytes(int bits, int mode, const Shape &s) {
+    mode = fit_mode(bits, mode, s);
     return bits == 8
                ? dev::layout<8>(s.hist_copies, s.stages, s.stage_bytes, s.consumer_warps, s.groups, mode).total
                : dev::layout<12>(s.hist_copies, s.stages, s.stage_bytes, s.consumer_warps, s.groups, mode).total;
@@ -49,7 +59,7 @@ size_t stream_smem_bytes(int bits, int mode, int consumer_warps, int ncopies, in
 }
 
 int persistent_occupancy(int bits, int mode, const Shape &s) {
-    mode = shape_mode(bits, mode, s);
+    mode = fit_mode(bits, mode, s);
     if (mode & kModeAny) return bits == 8 ? persistent_occupancy_any_b8(mode, s) : persistent_occupancy_any_b12(mode, s);
     if (mode & kModeWarpSplit) return persistent_occupancy_split_b8(mode, s);
     if (mode & kModeMulti) return bits == 8 ? persistent_occupancy_multi_b8(mode, s) : 0;
@@ -61,7 +71,7 @@ int persistent_occupancy(int bits, int mode, const Shape &s) {
 
 cudaError_t launch_persistent(int bits, int mode, const Shape &s, int grid, const Seg *segs, const Tile *tiles,
                               int ntiles, const Params &p, unsigned *counter, int inject, cudaStream_t st) {
-    mode = shape_mode(bits, mode, s);
+    mode = fit_mode(bits, mode, s);
     if (mode & kModeAny)
         return bits == 8 ? launch_persistent_any_b8(mode, s, grid, segs, tiles, ntiles, p, counter, inject, st)
                          : launch_persistent_any_b12(mode, s, grid, segs, tiles, ntiles, p, counter, inject, st);

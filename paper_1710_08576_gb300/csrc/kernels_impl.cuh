@@ -97,7 +97,7 @@ __host__ __device__ inline Layout layout(int ncopies, int stages, int stage_byte
     const int cps_end = copies ? align_up(amd_end + static_cast<int>(sizeof(CopyShared)), 128) : amd_end;
     L.mt = multi ? cps_end : 0;
     L.grp_size = multi ? align_up(cps_end + static_cast<int>(sizeof(MultiTile)), 128) : cps_end;
-    const bool coarse = BITS == 12 && (mode & kModeStats) != 0;
+    const bool coarse = BITS == 12 && (mode & kModeStats) != 0 && (mode & kModeTight) == 0;
     L.coarse = coarse ? L.grp_size : 0;
     if (coarse) L.grp_size = align_up(L.grp_size + kCoarse * 4, 128);
     L.split = split ? L.grp_size : 0;

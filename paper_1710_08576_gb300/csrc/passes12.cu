@@ -4,11 +4,23 @@
 
 namespace rfi {
 
+static_assert(kModeStats + kModeTight == 4100, "mode number of the cases below");
+
+#define RFI_DISPATCH_TIGHT(FN, MODE, CW, G, ...)                   \
+    do {                                                           \
+        switch (MODE * 1000 + CW * 10 + G) {                       \
+            RFI_CASES_MOM_CW(12, FN, 4100, __VA_ARGS__)            \
+            default: break;                                        \
+        }                                                          \
+    } while (0)
+
 cudaError_t launch_persistent_mom_b12(int mode, const Shape &s, int grid, const Seg *segs, const Tile *tiles,
                                       int ntiles, const Params &p, unsigned *counter, int inject,
                                       cudaStream_t st) {
     RFI_DISPATCH_MOM(12, dev::persistent_launch_t, mode, s.consumer_warps, s.groups, s, grid, segs, tiles, ntiles,
                      p, counter, inject, st);
+    RFI_DISPATCH_TIGHT(dev::persistent_launch_t, mode, s.consumer_warps, s.groups, s, grid, segs, tiles, ntiles, p,
+                      counter, inject, st);
     RFI_DISPATCH_FMT12(dev::persistent_launch_t, mode, s.consumer_warps, s.groups, s, grid, segs, tiles, ntiles, p,
                       counter, inject, st);
     return cudaErrorInvalidValue;
@@ -16,6 +28,7 @@ cudaError_t launch_persistent_mom_b12(int mode, const Shape &s, int grid, const 
 
 int persistent_occupancy_mom_b12(int mode, const Shape &s) {
     RFI_DISPATCH_MOM(12, dev::persistent_occ_t, mode, s.consumer_warps, s.groups, s);
+    RFI_DISPATCH_TIGHT(dev::persistent_occ_t, mode, s.consumer_warps, s.groups, s);
     RFI_DISPATCH_FMT12(dev::persistent_occ_t, mode, s.consumer_warps, s.groups, s);
     return 0;
 }

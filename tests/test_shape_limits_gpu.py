@@ -52,3 +52,29 @@ def test_copies_in_the_largest_stages_that_fit(cuda, rfi, bits, W, shape):
         finally:
             plan.close()
     assert all(torch.equal(a, b) for k in range(2) for a, b in zip(res[0][k], res[1][k]))
+
+
+@pytest.mark.parametrize("W,shape", [(32960, dict(stages=3, hist_copies=1)), (22656, dict(stages=4, hist_copies=2)),
+                                     (9280, dict(stages=8, hist_copies=4)), (32953, dict(stages=3, hist_copies=1))])
+def test_estimation_in_the_largest_stages_that_fit(cuda, rfi, W, shape):
+    """12-bit Median of MAD whose window fills the largest stage of that number: as with the default
+    shape, window for window."""
+    import torch
+    lens = [W * 9 + 8, W * 4, W]
+    xs = [torch.from_numpy(x).cuda() for x in _streams(12, lens)]
+    res = []
+    for s in (shape, None):
+        plan = rfi.Plan(12, lens, [W] * 3, 3.0, 2, 0, 0, 0, None, s, 4)
+        try:
+            outs = [torch.empty_like(x) for x in xs]
+            meds, mads, moms = [[torch.full((n,), -99, dtype=torch.int32, device="cuda") for n in plan.num_windows] for _ in range(3)]
+            for _ in range(2):
+                plan.excise(xs, outs)
+            st, _ = plan.stats(meds, mads)
+            plan.stats_mom(moms)
+            torch.cuda.synchronize()
+            assert st == 0 and (s is None or plan.info().shape.stages == s["stages"])
+            res.append(outs + meds + mads + moms)
+        finally:
+            plan.close()
+    assert all(torch.equal(a, b) for a, b in zip(*res))

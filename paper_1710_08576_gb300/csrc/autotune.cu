@@ -3,7 +3,7 @@
 // for 12-bit samples, histogram copies. Every candidate that fits is timed with CUDA events on a
 // scratch copy of the plan's own window layout (capped at 256 MiB of input) filled with
 // noise-like samples; the fastest shape is kept. Results are cached per process by
-// (device, sample width, mode, window layout), and in the file named by the environment
+// (device, sample width, mode, window layout, the caller's constraints: tune_key), and in the file named by the environment
 // variable RFI_TUNE_CACHE when it is set (one "key<TAB>shape" line per entry).
 
 #include <algorithm>
@@ -73,18 +73,11 @@ std::vector<Tile> tiles_for(int bits, int mode, const std::vector<int64_t> &len,
 std::mutex g_cache_mu;
 std::map<std::string, Shape> g_cache;
 
-std::string cache_key(const rfi_plan_s *P) {
+std::string cache_key(const rfi_plan_s *P, const rfi_launch_shape *req) {
     cudaDeviceProp prop;
     std::string k;
     if (cudaGetDeviceProperties(&prop, P->device) == cudaSuccess) k = prop.name;
-    char buf[96];
-    std::snprintf(buf, sizeof(buf), "|%d|%d|%d|", P->bits, plan_kernel_mode(P), P->S);
-    k += buf;
-    for (int i = 0; i < P->S; ++i) {
-        std::snprintf(buf, sizeof(buf), "%d:%lld,", P->W[i], static_cast<long long>(P->len[i] / P->W[i]));
-        k += buf;
-    }
-    return k;
+    return k + tune_key(P->bits, plan_kernel_mode(P), P->len, P->W, req);
 }
 
 bool cache_file_lookup(const std::string &key, Shape *out) {
@@ -138,25 +131,34 @@ struct Scratch {
 }  // namespace
 
 rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
-    const std::string key = cache_key(P);
+    const std::string key = cache_key(P, req);
+    const int bps = P->bits == 8 ? 1 : 2;
+    int64_t maxwb = 0;
+    bool uniform = true;
+    for (int i = 0; i < P->S; ++i) {
+        maxwb = std::max<int64_t>(maxwb, std::min<int64_t>(P->W[i], P->len[i]) * bps);
+        uniform = uniform && P->W[i] == P->W[0];
+    }
+    const int min_stage = min_stage_bytes(plan_tile_mode(P), maxwb);
     {
         std::lock_guard<std::mutex> g(g_cache_mu);
         auto it = g_cache.find(key);
         Shape cached{};
         bool hit = it != g_cache.end();
         if (hit) cached = it->second;
-        else if (cache_file_lookup(key, &cached)) {
-            hit = persistent_occupancy(P->bits, plan_kernel_mode(P), cached) >= cached.ctas_per_sm;
-            if (hit) g_cache[key] = cached;
-        }
+        else hit = cache_file_lookup(key, &cached);
+        // a file may hold anything
+        hit = hit && tuned_shape_fits(cached, min_stage) &&
+              persistent_occupancy(P->bits, plan_kernel_mode(P), cached) >= cached.ctas_per_sm;
         if (hit) {
+            g_cache[key] = cached;
             P->shape = cached;
             P->split_by_rule = false;
             rfi_status rs = plan_build_tiles(P);
             return rs == RFI_OK ? plan_alloc_workspace(P) : rs;
         }
+        cudaGetLastError();
     }
-    const int bps = P->bits == 8 ? 1 : 2;
     // scratch layout: every stream, each cut to an equal share of the budget (whole windows,
     // at least one window)
     const int64_t share = std::max<int64_t>(1, kScratchBudget / bps / P->S);
@@ -203,13 +205,6 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
         return RFI_ERR_CUDA;
 
     // candidate shapes
-    int64_t maxwb = 0;
-    bool uniform = true;
-    for (int i = 0; i < P->S; ++i) {
-        maxwb = std::max<int64_t>(maxwb, std::min<int64_t>(P->W[i], P->len[i]) * bps);
-        uniform = uniform && P->W[i] == P->W[0];
-    }
-    const int min_stage = min_stage_bytes(plan_tile_mode(P), maxwb);
     std::vector<Shape> cands;
     for (int cw : {4, 8, 16})
       for (int grp : {1, 2})

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <string>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -114,6 +115,34 @@ rfi_status plan_check_buffers(const rfi_plan_s *P, const void *const *in, void *
 rfi_status plan_run_batched(rfi_plan_s *P, const std::vector<Seg> &segs, cudaStream_t st);
 inline int plan_nsegs(const rfi_plan_s *P) {
     return P->kmom >= 2 ? 2 * P->S : (P->ncopy > 0 ? P->ncopy * P->S : P->S);
+}
+// Key of a tuned shape, after the device's name: what the candidates and their times depend on. A stream
+// shorter than its window counts with its length, which its stage is sized for; a shape tuned under
+// the caller's constraints is kept apart from others.
+inline std::string tune_key(int bits, int mode, const std::vector<int64_t> &len, const std::vector<int32_t> &W,
+                            const rfi_launch_shape *req) {
+    std::string k = "|" + std::to_string(bits) + "|" + std::to_string(mode) + "|" + std::to_string(len.size()) + "|";
+    for (size_t i = 0; i < len.size(); ++i) {
+        k += std::to_string(W[i]) + ":" + std::to_string(len[i] / W[i]);
+        k += len[i] < W[i] ? "/" + std::to_string(len[i]) + "," : ",";
+    }
+    if (req) {
+        const int32_t f[] = {req->consumer_warps, req->stages, req->ctas_per_sm, req->stage_bytes,
+                             req->dynamic_tiles, bits == 12 ? req->hist_copies : 0, req->groups, req->warp_split};
+        bool any = false;
+        for (int32_t v : f) any = any || v != 0;
+        if (any)
+            for (int32_t v : f) k += "|" + std::to_string(v);
+    }
+    return k;
+}
+// Whether a shape from the cache is one that the tuner could have made for windows that need min_stage bytes.
+inline bool tuned_shape_fits(const Shape &s, int min_stage) {
+    return (s.consumer_warps == 4 || s.consumer_warps == 8 || s.consumer_warps == 16) && s.stages >= 1 && s.stages <= 8 &&
+           s.ctas_per_sm >= 1 && s.ctas_per_sm <= 4 && s.stage_bytes >= min_stage && s.stage_bytes <= 227 * 1024 &&
+           s.stage_bytes % 128 == 0 && (s.dynamic_tiles == 1 || s.dynamic_tiles == 2) &&
+           (s.hist_copies == 1 || s.hist_copies == 2 || s.hist_copies == 4) && (s.groups == 1 || s.groups == 2) &&
+           (s.warp_split == 1 || s.warp_split == 2);
 }
 // Stage class of a window of wb bytes: 0 up to 16 KiB, 1 up to 32 KiB, 2 larger.
 inline int window_class(int64_t wb) { return wb <= 16384 ? 0 : (wb <= 32768 ? 1 : 2); }

@@ -13,7 +13,7 @@ CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 def answers(tmp_path, body):
     """The integers that a program with the given main body prints."""
     src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
-    src.write_text('#include <cstdio>\n#include <cuda_runtime.h>\n#include "internal.h"\nusing namespace rfi;\n'
+    src.write_text('#include <cstdio>\n#include <cuda_runtime.h>\n#include "rfi.h"\n#include "internal.h"\n#include "plan_impl.h"\nusing namespace rfi;\n'
                    "int main() {\n" + body + "\nreturn 0;\n}\n")
     subprocess.check_call(["g++", "-std=c++17", "-I" + CSRC, "-I" + os.path.join(ROOT, "include"),
                            "-I" + os.path.join(CUDA, "include"), str(src), "-o", str(exe)])
@@ -38,3 +38,25 @@ def test_the_any_window_form_where_it_is_the_faster_one(tmp_path, i):
     gains = answers(tmp_path, "".join('printf("%%lld\\n", (long long)any_form_gain(%d, %d, %d, %d, 1 << 22));' %
                                       (bits, noise, mom, W) for _, W in streams))
     assert (sum(n * g for (n, _), g in zip(streams, gains)) > 0) == want, gains
+
+
+def test_tuned_shapes_are_kept_apart(tmp_path):
+    """A short stream's length and the caller's constraints are in the key of a tuned shape; whole
+    windows are, and nothing else of a longer stream."""
+    keys = ["tune_key(8, 0, {100}, {65536}, nullptr)", "tune_key(8, 0, {60000}, {65536}, nullptr)",
+            "tune_key(8, 0, {70000}, {65536}, nullptr)", "tune_key(8, 0, {70001}, {65536}, nullptr)",
+            "tune_key(8, 0, {70000}, {65536}, &none)", "tune_key(8, 0, {70000}, {65536}, &two)"]
+    got = answers(tmp_path, "rfi_launch_shape none{}, two{};\ntwo.stages = 2;\nstd::string k[] = {" + ", ".join(keys) + "};\n" +
+                  "for (int i = 0; i < 6; ++i) for (int j = 0; j < 6; ++j) printf(\"%d\\n\", k[i] == k[j]);")
+    same = {(2, 3), (2, 4), (3, 4)}
+    assert got == [int(i == j or (min(i, j), max(i, j)) in same) for i in range(6) for j in range(6)]
+
+
+def test_cached_shapes_have_to_hold_the_windows(tmp_path):
+    """A cached shape whose stage is smaller than the plan's largest window, or that no tuner wrote, is
+    not taken."""
+    shapes = [("8, 2, 3, 512, 1, 1, 1, 1", 65536, 0), ("8, 2, 1, 65536, 1, 1, 1, 1", 65536, 1), ("8, 2, 1, 65537, 1, 1, 1, 1", 65536, 0),
+              ("8, 9, 1, 65536, 1, 1, 1, 1", 65536, 0), ("8, 2, 0, 65536, 1, 1, 1, 1", 65536, 0), ("5, 2, 1, 65536, 1, 1, 1, 1", 65536, 0),
+              ("8, 2, 1, 65536, 1, 3, 1, 1", 65536, 0), ("16, 1, 2, 1024, 2, 4, 1, 2", 128, 1)]
+    got = answers(tmp_path, "".join('printf("%%d\\n", (int)tuned_shape_fits(Shape{%s}, %d));' % s[:2] for s in shapes))
+    assert got == [s[2] for s in shapes]

@@ -52,13 +52,12 @@ __global__ void fill_scratch(uint8_t *buf, int64_t n, int bits) {
     }
 }
 
-std::vector<Tile> tiles_for(int bits, int mode, const std::vector<int64_t> &len, const std::vector<int32_t> &W,
-                            int stage_bytes) {
+std::vector<Tile> tiles_for(int bits, const std::vector<int64_t> &len, const std::vector<int32_t> &W,
+                            const std::vector<int64_t> &per_tile) {
     const int bps = bits == 8 ? 1 : 2;
     std::vector<Tile> tiles;
     for (size_t i = 0; i < len.size(); ++i) {
-        const int64_t per = tile_windows(bits, mode, W[i], stage_bytes);
-        const int64_t nwin = (len[i] + W[i] - 1) / W[i];
+        const int64_t per = per_tile[i], nwin = (len[i] + W[i] - 1) / W[i];
         for (int64_t w0 = 0; w0 < nwin; w0 += per) {
             const int64_t nw = std::min<int64_t>(per, nwin - w0);
             const int64_t s1 = std::min<int64_t>(len[i], (w0 + nw) * W[i]);
@@ -162,12 +161,13 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
     // scratch layout: every stream, each cut to an equal share of the budget (whole windows,
     // at least one window)
     const int64_t share = std::max<int64_t>(1, kScratchBudget / bps / P->S);
-    std::vector<int64_t> slen(P->S), soff(P->S);
+    std::vector<int64_t> slen(P->S), soff(P->S), snwin(P->S);
     std::vector<int64_t> mwoff(P->S), woff(P->S);
     int64_t tot = 0, totw = 0, totmw = 0;
     for (int i = 0; i < P->S; ++i) {
         const int64_t nw = std::max<int64_t>(1, std::min<int64_t>(P->nwin[i], share / P->W[i]));
         slen[i] = std::min<int64_t>(P->len[i], nw * P->W[i]);
+        snwin[i] = nw;
         soff[i] = tot;
         woff[i] = totw;
         mwoff[i] = totmw;
@@ -252,14 +252,18 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
     Shape best{};
     float best_ms = 1e30f;
     std::vector<Tile> cur;
-    int cur_stage = -1;
+    std::vector<int64_t> cur_per;
     for (const Shape &s : cands) {
         if (persistent_occupancy(P->bits, plan_kernel_mode(P), s) < s.ctas_per_sm) {
             cudaGetLastError();
             continue;
         }
-        if (s.stage_bytes != cur_stage) {
-            cur = tiles_for(P->bits, plan_tile_mode(P), slen, P->W, s.stage_bytes);
+        const std::vector<int64_t> per_tile =
+            windows_per_tile(P->bits, plan_tile_mode(P), false, P->given_stage, snwin, P->W, s.stage_bytes,
+                             static_cast<int64_t>(P->sm_count) * s.ctas_per_sm);
+        if (per_tile != cur_per) {
+            cur = tiles_for(P->bits, slen, P->W, per_tile);
+            cur_per.clear();
             cudaFree(sc.tiles);
             sc.tiles = nullptr;
             if (cudaMalloc(&sc.tiles, sizeof(Tile) * cur.size()) != cudaSuccess ||
@@ -267,7 +271,7 @@ rfi_status plan_autotune(rfi_plan_s *P, const rfi_launch_shape *req) {
                 cudaGetLastError();
                 continue;
             }
-            cur_stage = s.stage_bytes;
+            cur_per = per_tile;
         }
         p.ncopies = s.hist_copies;
         const int nt = static_cast<int>(cur.size());

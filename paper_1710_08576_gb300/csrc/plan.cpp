@@ -127,32 +127,12 @@ bool plan_warp_split_runs(const rfi_plan_s *P, const Shape &s) {
 
 rfi_status plan_build_tiles(rfi_plan_s *P) {
     const int bps = P->bits == 8 ? 1 : 2;
-    auto per_tile = [&](int i, int64_t div) {
-        int64_t per = tile_windows(P->bits, plan_tile_mode(P), P->W[i], P->shape.stage_bytes);
-        if (P->kmom >= 2) per = std::min<int64_t>(per, kApplyTileWindows);
-        return std::max<int64_t>(1, per / div);
-    };
-    // a small plan spreads its windows: tiles of fewer windows as long as all of them still run at
-    // once (2^20 int8 samples in 4096-sample windows: 64 tiles of four 9.6 us a call, 256 of one 8.2,
-    // with noise 12.3 and 8.8; 2^22 samples: 256 tiles 10.3 us, 512 on 456 CTAs 12.4). A stage size
-    // that the caller gave stands for its tiles.
-    int64_t div = 1;
-    if (!P->given_stage) {
-        auto count = [&](int64_t d) {
-            int64_t n = 0;
-            for (int i = 0; i < P->S; ++i) n += (P->nwin[i] + per_tile(i, d) - 1) / per_tile(i, d);
-            return n;
-        };
-        const int64_t room = static_cast<int64_t>(P->sm_count) * P->shape.ctas_per_sm;
-        for (int64_t n = count(1); div < 64 && n < room; div *= 2) {
-            const int64_t more = count(2 * div);
-            if (more == n || more > room) break;
-            n = more;
-        }
-    }
+    const std::vector<int64_t> per_tile =
+        windows_per_tile(P->bits, plan_tile_mode(P), P->kmom >= 2, P->given_stage, P->nwin, P->W, P->shape.stage_bytes,
+                         static_cast<int64_t>(P->sm_count) * P->shape.ctas_per_sm);
     std::vector<Tile> tiles;
     for (int i = 0; i < P->S; ++i) {
-        const int64_t per = per_tile(i, div);
+        const int64_t per = per_tile[i];
         for (int64_t w0 = 0; w0 < P->nwin[i]; w0 += per) {
             const int64_t nw = std::min<int64_t>(per, P->nwin[i] - w0);
             const int64_t s0 = w0 * P->W[i];

@@ -116,6 +116,33 @@ rfi_status plan_run_batched(rfi_plan_s *P, const std::vector<Seg> &segs, cudaStr
 inline int plan_nsegs(const rfi_plan_s *P) {
     return P->kmom >= 2 ? 2 * P->S : (P->ncopy > 0 ? P->ncopy * P->S : P->S);
 }
+// Windows per tile of each stream: as many as a stage holds, fewer in a small plan, which spreads its
+// windows: tiles are halved as long as all of them still run at once on `room` CTAs (2^20 int8 samples
+// in 4096-sample windows: 64 tiles of four 9.6 us a call, 256 of one 8.2, with noise 12.3 and 8.8;
+// 2^22 samples: 256 tiles 10.3 us, 512 on 456 CTAs 12.4). whole: a stage size that the caller gave
+// stands for its tiles. The tuner times the same lists.
+inline std::vector<int64_t> windows_per_tile(int bits, int mode, bool mom, bool whole, const std::vector<int64_t> &nwin,
+                                             const std::vector<int32_t> &W, int stage_bytes, int64_t room) {
+    std::vector<int64_t> per(W.size());
+    auto set = [&](int64_t div) {  // the tiles
+        int64_t n = 0;
+        for (size_t i = 0; i < W.size(); ++i) {
+            int64_t p = tile_windows(bits, mode, W[i], stage_bytes);
+            if (mom) p = p < kApplyTileWindows ? p : kApplyTileWindows;
+            per[i] = p / div > 1 ? p / div : 1;
+            n += (nwin[i] + per[i] - 1) / per[i];
+        }
+        return n;
+    };
+    int64_t div = 1;
+    for (int64_t n = set(1); !whole && div < 64 && n < room; div *= 2) {
+        const int64_t more = set(2 * div);
+        if (more == n || more > room) break;
+        n = more;
+    }
+    set(div);
+    return per;
+}
 // Key of a tuned shape, after the device's name: what the candidates and their times depend on. A stream
 // shorter than its window counts with its length, which its stage is sized for; a shape tuned under
 // the caller's constraints is kept apart from others.

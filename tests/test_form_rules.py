@@ -60,3 +60,16 @@ def test_cached_shapes_have_to_hold_the_windows(tmp_path):
               ("8, 2, 1, 65536, 1, 3, 1, 1", 65536, 0), ("16, 1, 2, 1024, 2, 4, 1, 2", 128, 1)]
     got = answers(tmp_path, "".join('printf("%%d\\n", (int)tuned_shape_fits(Shape{%s}, %d));' % s[:2] for s in shapes))
     assert got == [s[2] for s in shapes]
+
+
+def test_tiles_of_small_plans(tmp_path):
+    """Tiles are halved while all of them run at once; a large plan, a stage size of the caller's, and
+    windows that are a tile each keep theirs. Median of MAD: at most the apply pass' 32."""
+    plans = [  # (windows of each stream, their length, stage, caller's stage, mom) -> windows per tile
+        ([256], [4096], 16384, 0, 0, [1]), ([1024], [4096], 16384, 0, 0, [4]), ([256], [4096], 16384, 1, 0, [4]),
+        ([256], [1024], 16384, 0, 0, [1]), ([1024], [1024], 16384, 0, 0, [4]), ([4096], [512], 16384, 0, 0, [16]),
+        ([64], [16384], 16384, 0, 0, [1]), ([32, 300], [8192, 1024], 16384, 0, 0, [1, 1]), ([100000], [16], 16384, 0, 1, [32]),
+    ]
+    body = "".join("for (auto v : windows_per_tile(8, 0, %d, %d, {%s}, {%s}, %d, 456)) printf(\"%%lld\\n\", (long long)v);\n" %
+                   (mom, whole, ", ".join(map(str, n)), ", ".join(map(str, W)), stage) for n, W, stage, whole, mom, _ in plans)
+    assert answers(tmp_path, body) == sum((p[-1] for p in plans), [])

@@ -573,7 +573,10 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
             if (sg.vec && tl.nw >= 2u && W >= 512u && W <= 8192u && (W & (W - 1u)) == 0u && tl.bytes == tl.nw * W) {
                 if (dirty) {
                     zero_shared(sm.hist, 32768, tid, T);
-                    named_bar(sm.bar_id, T);
+                    if (named_bar_or(sm.bar_id, T, false)) {
+                        timed_out = true;
+                        break;
+                    }
                     dirty = false;
                 }
                 const int lw = 31 - __clz(static_cast<int>(W));
@@ -608,7 +611,10 @@ persistent_kernel(const Seg *__restrict__ segs, const Tile *__restrict__ tiles, 
             if (tl.nw >= 2u && sg.W <= kMultiMaxWindow) {
                 if (dirty) {
                     zero_shared(sm.hist, 32768, tid, T);
-                    named_bar(sm.bar_id, T);
+                    if (named_bar_or(sm.bar_id, T, false)) {
+                        timed_out = true;
+                        break;
+                    }
                     dirty = false;
                 }
                 const uint32_t K = tl.nw > 4u ? 8u : 4u;

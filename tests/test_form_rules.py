@@ -73,3 +73,12 @@ def test_tiles_of_small_plans(tmp_path):
     body = "".join("for (auto v : windows_per_tile(8, 0, %d, %d, {%s}, {%s}, %d, 456)) printf(\"%%lld\\n\", (long long)v);\n" %
                    (mom, whole, ", ".join(map(str, n)), ", ".join(map(str, W)), stage) for n, W, stage, whole, mom, _ in plans)
     assert answers(tmp_path, body) == sum((p[-1] for p in plans), [])
+
+
+def test_consumers_agree_on_a_timeout_at_their_first_barrier():
+    """Every barrier of the joint consumers' loop between the bounded wait for a stage and the window passes
+    carries a vote: at a plain one, a thread whose wait timed out would be taken for one that is
+    there, and its vote would be lost."""
+    text = open(os.path.join(CSRC, "kernels_impl.cuh")).read()
+    loop = text[text.index("bool dirty = false;"):text.index("// the group's flagged total")]
+    assert "named_bar_or(" in loop and "named_bar(" not in loop

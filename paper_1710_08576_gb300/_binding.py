@@ -193,6 +193,7 @@ def _addresses(seq):
     in one pass (5.8 us for 60 against 30 us for _ptr_array; every call reads them anew)."""
     if seq is None:
         return None, None
+    len(seq)  # an iterator is refused: its tensors would be gone before the kernel runs
     torch = sys.modules.get("torch")
     if torch is not None:
         try:

@@ -91,20 +91,18 @@ rfi_status plan_choose_shape(rfi_plan_s *P, const rfi_launch_shape *req) {
         if (occ_apply < 1) return cudaGetLastError() != cudaSuccess ? RFI_ERR_CUDA : RFI_ERR_UNSUPPORTED;
         P->grid_apply = P->sm_count * occ_apply;  // clamped to the tile count with the grid
     }
-    // plans of many tiles per CTA take tiles from the cursor: SMs differ in pace (60 streams of 2^24
-    // int8 samples, fp16 output, 135 tiles a CTA: 612 us a call round robin, 575 from the cursor; 60 x
-    // 2^22 12-bit noise 577 and 526; 8 variants 812 and 754). With few (60 x 2^19 samples, 4 tiles a
-    // CTA: 42.3 and 45.5 us) the cursor's round trips cost more, unless window sizes differ.
+    // plans of many tiles per CTA take tiles from the cursor (many_tiles)
     int64_t tiles = 0;
     for (int i = 0; i < P->S; ++i) {
         const int64_t per = tile_windows(P->bits, plan_tile_mode(P), P->W[i], s.stage_bytes);
         tiles += (P->nwin[i] + per - 1) / per;
     }
-    const bool many = tiles >= 16 * static_cast<int64_t>(P->sm_count) * s.ctas_per_sm;
+    const bool many = many_tiles(tiles, static_cast<int64_t>(P->sm_count) * s.ctas_per_sm);
     if (!(req && req->dynamic_tiles)) s.dynamic_tiles = !uniform || many ? 1 : 2;
     // the split-warp form runs int8 zero / constant / threshold, one group of 8; there plans of many
-    // tiles take it (60 streams of 2^22 samples from the cursor, zero, 16384-sample windows: 118.1 us
-    // joint, 112.1 split; threshold 130.4 and 122.1; 65536-sample windows 123.3 and 116.2)
+    // tiles take it (from the cursor, 16384-sample windows, zero: 12 tiles a CTA 49.3 us joint, 46.3 split, 16
+    // tiles 61.3 and 57.8, 34 tiles 118.1 and 112.1; threshold 53.7 and 51.4, 67.8 and 63.7, 130.4 and
+    // 122.1; 65536-sample windows, 25 tiles 123.3 and 116.2)
     s.warp_split = (req && req->warp_split) ? req->warp_split : 1;
     if (s.warp_split == 2 && !plan_warp_split_runs(P, s)) return RFI_ERR_UNSUPPORTED;
     if (!(req && req->warp_split) && many && plan_warp_split_runs(P, s)) {

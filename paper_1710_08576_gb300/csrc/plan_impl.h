@@ -116,6 +116,13 @@ rfi_status plan_run_batched(rfi_plan_s *P, const std::vector<Seg> &segs, cudaStr
 inline int plan_nsegs(const rfi_plan_s *P) {
     return P->kmom >= 2 ? 2 * P->S : (P->ncopy > 0 ? P->ncopy * P->S : P->S);
 }
+// Whether a plan of one window size takes its tiles from the cursor and not round robin. SMs differ in
+// pace, which the cursor evens out, but its round trips cost a plan of few tiles. us a call, round robin
+// and cursor, int8 noise in 16384-sample windows (12-bit noise, 8192 samples; fp16 output): 5.3 tiles a CTA
+// 33.2 and 33.3 (37.5 and 38.6; 32.8 and 33.1), 9.1 tiles 51.8 and 53.5 (58.5 and 59.7; 51.4 and 50.8), 12
+// tiles 66.0 and 64.1 (74.2 and 74.2; 64.0 and 62.9), 16 tiles 84.7 and 82.8 (96.0 and 94.3; 81.9 and
+// 79.2), 40 tiles 197 and 190 (225 and 218; 189 and 180).
+inline bool many_tiles(int64_t tiles, int64_t ctas) { return tiles >= 12 * ctas; }
 // Windows per tile of each stream: as many as a stage holds, fewer in a small plan, which spreads its
 // windows: tiles are halved as long as all of them still run at once on `room` CTAs (2^20 int8 samples
 // in 4096-sample windows: 64 tiles of four 9.6 us a call, 256 of one 8.2, with noise 12.3 and 8.8;

@@ -75,6 +75,12 @@ def test_tiles_of_small_plans(tmp_path):
     assert answers(tmp_path, body) == sum((p[-1] for p in plans), [])
 
 
+def test_plans_of_many_tiles(tmp_path):
+    """Twelve tiles a CTA and more come from the cursor, fewer round robin."""
+    got = answers(tmp_path, "".join('printf("%%d\\n", (int)many_tiles(%d, 456));' % n for n in (1, 456 * 9, 456 * 12 - 1, 456 * 12, 456 * 40)))
+    assert got == [0, 0, 0, 1, 1]
+
+
 def test_consumers_agree_on_a_timeout_at_their_first_barrier():
     """Every barrier of the joint consumers' loop between the bounded wait for a stage and the window passes
     carries a vote: at a plain one, a thread whose wait timed out would be taken for one that is

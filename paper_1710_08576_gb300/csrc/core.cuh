@@ -1562,10 +1562,10 @@ __device__ __forceinline__ uint32_t noise_slices12(const Shm &sm, const Win &w, 
 
 // ------------------------------------------------------------------ digital copies
 // Eq. 2 for all variants of one threshold multiple at once (grp: their bits, v: the first of them),
-// over a window of whole warp rounds with aligned outputs and masks: same M, same t, so the flags,
-// the mask bits and the count are computed once, and each variant adds its own replacement and
-// stores (one variant at a time, every one of them computed the flags again: 8 variants, two
-// multiples with four replacements each, 60 streams of 2^22 samples 748 us a call, now 663).
+// over a window of whole warp rounds that uses all its mask words, with aligned outputs and masks: same
+// M, same t, so the flags, the mask bits and the count are computed once, and each variant adds its own
+// replacement and stores (one variant at a time, every one of them computed the flags again: 8 variants, two
+// multiples with four replacements each, 60 streams of 2^22 samples 748 us a call, now 653).
 template <int T>
 __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, int v, uint32_t grp, bool noise, int tid,
                                                  uint32_t *nlc) {
@@ -1627,13 +1627,6 @@ __device__ __forceinline__ uint32_t copies_pass8(const Shm &sm, const Win &w, in
         if (noise) {
             noise_note8(sm, lane, c, bits[0], nlc);
             if (two) noise_note8(sm, lane, c + T, bits[1], nlc);
-        }
-    }
-    // mask pieces past the window's last sample (a short last window of whole rounds)
-    if (nchunks < 2 * w.mask_words) {
-        for (uint32_t g = grp; g; g &= g - 1u) {
-            uint16_t *const mk = sm.pass->mask[__ffs(static_cast<int>(g)) - 1];
-            for (int c = nchunks + tid; c < 2 * w.mask_words; c += T) mk[c] = 0;
         }
     }
     return flagged;
@@ -1749,9 +1742,10 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
     if (COPIES) {
         // every variant's values from the window's M and D, then its replace pass
         const int nvar = params_nvar(p);
-        // only whole rounds with aligned buffers and masks share passes; where the first variant's are not,
-        // warp 0 gathers nothing for it
-        const bool may = BITS == 8 && w.vec && w.mask && (w.n & 511) == 0;
+        // variants share passes over whole rounds with aligned buffers and masks and without mask words past the
+        // window's last sample (the shared pass writes none); where the first variant's are not so, warp 0
+        // gathers nothing for it
+        const bool may = BITS == 8 && params_share(p) && w.vec && w.mask && (w.n & 511) == 0 && w.n == 32 * w.mask_words;
         if (tid < 32) {
             bool slow = !may;
             if (tid < nvar) {
@@ -1772,32 +1766,33 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
             if (BITS == 8 && tid == 0) sm.pass->fast = any_slow ? 0u : 1u;
         }
         named_bar(sm.bar_id, T);
-        const bool fast = BITS == 8 && sm.pass->fast;
-        for (uint32_t todo = (1u << nvar) - 1u; todo;) {
+        uint32_t todo = BITS == 8 && sm.pass->fast ? (1u << nvar) - 1u : 0u;
+        const bool grouped = todo != 0u;
+        while (todo) {
             const int v = __ffs(static_cast<int>(todo)) - 1;
-            const uint32_t grp = fast ? sm.pass->group[v] : 1u << v;
+            const uint32_t grp = sm.pass->group[v];
             todo &= ~grp;
+            uint32_t noise = 0u;
+            for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.pass->mode[u] == 3u ? 1u << u : 0u;
             uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
-            if (BITS == 8 && (grp & (grp - 1u))) {  // several variants of one multiple
-                uint32_t noise = 0u;
-                for (int u = v; u < nvar; ++u) noise |= ((grp >> u) & 1u) != 0u && sm.pass->mode[u] == 3u ? 1u << u : 0u;
-                uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
-                fv = __reduce_add_sync(0xFFFFFFFFu, fv);
-                if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
-                __syncwarp();  // lane 0 announces the window for every lane that counted
-                for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
-                    const int u = __ffs(static_cast<int>(m)) - 1;
-                    Win wu = w;
-                    wu.out = sm.pass->out[u];
-                    const uint64_t seed = params_var(p)[u].seed;
-                    noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
-                                                     KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,
-                                                     pw);
-                }
-                if (noise && todo) named_bar(sm.bar_id, T);  // the next group lists its own
-                continue;
+            uint32_t fv = copies_pass8<T>(sm, w, v, grp, noise != 0u, tid, nc);
+            fv = __reduce_add_sync(0xFFFFFFFFu, fv);
+            if (lane < nvar && ((grp >> lane) & 1u) && fv) atomicAdd(&sm.cp->vcount[lane][par], fv);
+            __syncwarp();  // lane 0 announces the window for every lane that counted
+            for (uint32_t m = noise; m; m &= m - 1u) {  // the same list, each with its own key
+                const int u = __ffs(static_cast<int>(m)) - 1;
+                Win wu = w;
+                wu.out = sm.pass->out[u];
+                const uint64_t seed = params_var(p)[u].seed;
+                noise_deferred8<T, false, false>(sm, wu, load_rep(sm.cp->vrep[u]),
+                                                 KeysSeed{static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32)}, tid, nc,
+                                                 pw);
             }
-            // a variant with a multiple of its own: the pass built for its replacement
+            if (noise && todo) named_bar(sm.bar_id, T);  // the next group lists its own
+        }
+        if (!grouped)
+        for (int v = 0; v < params_nvar(p); ++v) {
+            uint32_t *nc = &sm.cp->ncount[4 * v + 2 * par];
             const Variant vr = params_var(p)[v];
             const Seg &sv = vsegs[static_cast<int64_t>(v) * params_seg_stride(p)];
             Win wv = w;
@@ -1824,7 +1819,7 @@ __device__ bool process_window(const Shm &sm, const Win &w, const Seg &sg, int64
                         noise_deferred8<T, false, false>(sm, wv, rv, vkey, tid, nc, pw);
                     }
                     // the noise work area and the first indices are reused by the next variant
-                    if (todo) named_bar(sm.bar_id, T);
+                    if (v + 1 < params_nvar(p)) named_bar(sm.bar_id, T);
                     break;
             }
             fv = __reduce_add_sync(0xFFFFFFFFu, fv);

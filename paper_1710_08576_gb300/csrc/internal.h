@@ -151,8 +151,8 @@ struct Params {
     uint32_t *status;             // device status word (atomicOr of kStatus*)
     unsigned long long *flagged;  // device total of flagged samples
     uint32_t rk0[10], rk1[10];    // Philox4x32-10 round keys of `seed` (see set_round_keys)
-    // Digital copy: the number of variants (bits 0-3) and the distance between one variant's
-    // segment table and the next (bits 4-31), and the byte offset of the variant table from the
+    // Digital copy: the number of variants (bits 0-3), whether those of one multiple share a pass (bit
+    // 4, copies_share), the distance between one variant's segment table and the next (bits 5-31), and the byte offset of the variant table from the
     // status word (both live in the plan's workspace). Packed into 8 bytes: a larger parameter
     // block changes the register allocation of every excision kernel for the worse.
     int32_t copies;
@@ -160,7 +160,22 @@ struct Params {
 };
 
 __host__ __device__ inline int params_nvar(const Params &p) { return p.copies & 15; }
-__host__ __device__ inline int params_seg_stride(const Params &p) { return p.copies >> 4; }
+__host__ __device__ inline bool params_share(const Params &p) { return (p.copies & 16) != 0; }
+__host__ __device__ inline int params_seg_stride(const Params &p) { return p.copies >> 5; }
+// Whether digital copies of n variants, variant v of multiple kq(v), run one pass per multiple. A variant that
+// shares a pass saves 24 us of a call on 60 streams of 2^22 samples, but the pass that chooses its
+// variants' replacements as it stores costs each multiple 15 us over the pass built for one (two multiples of
+// four variants 626 us apart, 480 shared; one of two 208, 196; one of one 157, 171; eight of one 591, 708).
+template <class Multiple>
+inline bool copies_share(int n, Multiple &&kq) {
+    int groups = 0;
+    for (int v = 0; v < n; ++v) {
+        bool first = true;
+        for (int u = 0; u < v; ++u) first = first && kq(u) != kq(v);
+        groups += first ? 1 : 0;
+    }
+    return 24 * (n - groups) > 15 * groups;
+}
 __host__ __device__ inline const Variant *params_var(const Params &p) {
     return reinterpret_cast<const Variant *>(reinterpret_cast<const char *>(p.status) + p.var_off);
 }

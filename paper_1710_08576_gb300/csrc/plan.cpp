@@ -247,7 +247,8 @@ Params plan_params(const rfi_plan_s *P) {
     p.status = &P->d_ctr->status;
     p.flagged = &P->d_ctr->flagged;
     set_round_keys(p);
-    p.copies = P->ncopy | (P->S << 4);
+    const bool share = copies_share(P->ncopy, [&](int v) { return P->variants[v].kq; });
+    p.copies = P->ncopy | (share ? 16 : 0) | (P->S << 5);
     p.var_off = P->d_var ? static_cast<int32_t>(reinterpret_cast<const char *>(P->d_var) -
                                                 reinterpret_cast<const char *>(&P->d_ctr->status))
                          : 0;

@@ -81,6 +81,16 @@ def test_plans_of_many_tiles(tmp_path):
     assert got == [0, 0, 0, 1, 1]
 
 
+def test_copies_share_passes_where_that_is_the_faster_way(tmp_path):
+    """Multiples of the variants -> one pass per multiple: not for variants with a multiple each, nor where
+    the shared ones are too few to pay for the others."""
+    cases = [([3], 0), ([3, 3], 1), ([3, 5], 0), ([3] * 4 + [5] * 4, 1), ([1, 2, 3, 4, 5, 6, 7, 8], 0), ([3, 3, 5, 5, 7, 7, 9, 9], 1),
+             ([3, 3, 5], 0), ([3, 5, 3, 5, 2, 3, 5, 9], 1), ([3, 3, 3, 5, 6, 7], 0)]
+    body = "".join("{ int64_t k[] = {%s}; printf(\"%%d\\n\", (int)copies_share(%d, [&](int v) { return k[v]; })); }\n" %
+                   (", ".join(map(str, k)), len(k)) for k, _ in cases)
+    assert answers(tmp_path, body) == [w for _, w in cases]
+
+
 def test_consumers_agree_on_a_timeout_at_their_first_barrier():
     """Every barrier of the joint consumers' loop between the bounded wait for a stage and the window passes
     carries a vote: at a plain one, a thread whose wait timed out would be taken for one that is

@@ -104,7 +104,9 @@ typedef enum { RFI_OUT_SAME = 0, RFI_OUT_F16 = 1, RFI_OUT_BF16 = 2 } rfi_out_for
                                      (same bits; one more launch per call). Faster for large int8
                                      plans at ordinary flag densities (6 % flagged, 60 streams of
                                      2^26 samples: 2.72 ms against 3.38; of 2^22: 214 us against
-                                     223), slower for small plans (2^20: 83 us against 71). The
+                                     223), slower for small plans (2^20: 83 us against 71), about
+                                     even for 12-bit ones (a quarter flagged, 60 streams of 2^25
+                                     samples: 3.83 ms against 3.88). The
                                      first rfi_excise with a NULL mask for some stream allocates a
                                      plan-owned mask array (ceil(W/32) words per window) that
                                      rfi_plan_destroy frees. Ignored with RFI_PLAN_PER_STREAM,
@@ -120,8 +122,10 @@ typedef enum { RFI_OUT_SAME = 0, RFI_OUT_F16 = 1, RFI_OUT_BF16 = 2 } rfi_out_for
                                         chunks with a flag) instead of 2. 8-bit batched plans with
                                         per-window MAD only, without RFI_PLAN_POWER, fp16/bf16
                                         output or digital copies (RFI_ERR_UNSUPPORTED otherwise);
-                                        RFI_PLAN_NOISE_PASS is ignored; rfi_excise_host writes
-                                        every sample as usual */
+                                        RFI_PLAN_NOISE_PASS is ignored, so a large noise plan is
+                                        slower than one that writes every sample with it (60
+                                        streams of 2^26 samples, k = 3: 3.35 ms against 2.73);
+                                        rfi_excise_host writes every sample as usual */
 #define RFI_PLAN_INJECT_TIMEOUT 0x100u /* test hook: CTA 0 waits on a barrier nothing arrives
                                           on (bounded by 1 ms), latching RFI_ERR_TIMEOUT */
 

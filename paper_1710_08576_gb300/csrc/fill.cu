@@ -1,4 +1,4 @@
-// Digital noise as a second pass (Eq. 2's noise replacement, value as in noise_value).
+// Digital noise as a second pass (Eq. 2's noise replacement, value as in NoiseScale).
 //
 // The excision pass of a noise plan created with RFI_PLAN_NOISE_PASS runs as a zero-replacement
 // pass: it writes 0 at every flagged sample, the flag mask and every window's M and D. This

@@ -228,8 +228,10 @@ size_t stream_smem_bytes(int bits, int mode, int consumer_warps, int ncopies, in
 int persistent_occupancy(int bits, int mode, const Shape &s);
 
 // 12-bit histogram copies where nothing asks for a number: more copies spread a warp's same-bin
-// atomics, but take 16 KiB each from the CTAs (60 streams of 2^22 samples, noise, 8192-sample windows: 618
-// us a call with 1, 3 CTAs per SM, 746 with 2, 1186 with 4; 65536-sample windows, one CTA: 960, 969, 998).
+// atomics, but take 16 KiB each from the CTAs and are folded every window (60 streams of 2^22 samples, sigma
+// 120, 8192-sample windows, 1 and 2 copies: noise 358 us a call with 3 CTAs per SM, 488 with 2, zero 275 and
+// 376; 65536-sample windows, one CTA either way: 318 and 329). Narrow data, whose atomics meet in a few
+// bins, does not pay for them either (sigma 0.7, zero: 218 and 320; 32768-sample windows, one CTA: 234 and 257).
 constexpr int kDefaultHistCopies = 1;
 
 // Persistent batched kernel over a device work list. counter: one zeroed uint32 (dynamic tiles).
